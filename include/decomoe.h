@@ -552,10 +552,9 @@ DECOMOE_API int decomoe_moe_layer_workspace_layout(int64_t T, int d, int E, int 
  *   merged rows in the workspace, and a second small launch merges them in
  *   cluster order (deterministic in both cases).
  *   Prefill sizes (more queries per KV head, n = C or a chunk n < C; Hq / Hkv
- *   even): V is transposed into the workspace, then one tensor-core CTA per
- *   (pair of query heads, 128-query tile) runs the online softmax over 64-key
- *   blocks up to its causal limit (P rounded to bf16 before the P V product;
- *   deterministic).
+ *   even): one tensor-core CTA per (pair of query heads, 128-query tile) runs
+ *   the online softmax over 128-key blocks up to its causal limit (P rounded
+ *   to bf16 before the P V product; deterministic). No workspace.
  *   ws: decomoe_attention_workspace_bytes(n, C, Hq, Hkv, D) bytes, 16-byte
  *   aligned. A wait that runs past the time limit records
  *   DECOMOE_ERR_TIMEOUT in status_dev (may be null).

@@ -11,8 +11,8 @@
 //
 // Decode sizes (few queries per KV head): one launch of split-key blocks on
 // warp-level tensor-core products, the splits of a head merged through the
-// shared memory of their thread-block cluster (below). Prefill sizes: a
-// transpose of V, then the tcgen05 flash-style kernel (further below).
+// shared memory of their thread-block cluster (below). Prefill sizes: the
+// tcgen05 flash-style kernel (further below).
 #include <atomic>
 #include <cfloat>
 
@@ -608,65 +608,61 @@ static int att_active_clusters(int cs) {
 }
 
 // ------------------------------------------------------------------ prefill (tensor cores)
-// Many queries per KV head (the compacted sequence's prefill): flash-style
-// attention on tcgen05. A CTA takes one tile of 128 query rows for two query
-// heads of the same KV group, so each K and V block it streams serves both.
-// Per block j of 64 keys and head x: S_x = Q_x K_j^T (M = 128 queries, N = 64
-// keys, K = 128 features) into tensor memory; four warps per head (one query
-// row per thread) take the row maximum, write p = 2^(s*scale*log2e - m) as
-// bf16 into tensor memory (the A operand of the next product) and add p to
-// the row sum l; then O_x += P_x V_j (N = 128 features, K = 64 keys, V
-// transposed beforehand so that the B operand is K-major) accumulates in
-// tensor memory. The reference maximum m of a row moves only when the block
-// maximum exceeds it by more than 8 (a factor 256): then that row's O and l
-// are scaled by 2^(m_old - m_new) before the next product (otherwise p stays
-// below 256, well inside bf16 and fp32); the final output is O / l either
-// way. Tensor-core work of one head overlaps the other head's softmax: the
-// issue order is PV_0(j), S_0(j+1), PV_1(j), S_1(j+1). Warp 0 streams K_j and
-// V_j^T blocks by TMA into a four-stage ring; warp 1 issues the MMAs. Every
-// wait is bounded; on a timeout the CTA records DECOMOE_ERR_TIMEOUT, lets its
-// copies and MMAs land, frees its tensor memory and returns.
-constexpr int ATP_BM = 128;                 // query rows per CTA
-constexpr int ATP_BN = 64;                  // keys per block
-constexpr int ATP_HEADS = 2;                // query heads per CTA (same KV head)
-constexpr int ATP_NST = 4;                  // K / V ring stages
-constexpr int ATP_QHALF = 128 * 64 * 2;     // Q: 128 rows x 64 features, 128-byte swizzle (16 KB)
-constexpr int ATP_KHALF = ATP_BN * 64 * 2;  // K block: 64 keys x 64 features (8 KB)
-constexpr int ATP_VT = 128 * ATP_BN * 2;    // V^T block: 128 features x 64 keys (16 KB)
-constexpr int ATP_STAGE = 2 * ATP_KHALF + ATP_VT;
-constexpr int ATP_THREADS = 64 + ATP_HEADS * 128;
-constexpr int ATP_TMEM_COLS = 512;          // per head: S [0,64), P [64,96), O [128,256)
-constexpr float ATP_RESCALE = 8.0f;         // log2 of the largest unnormalised p
-constexpr size_t ATP_SMEM = 1024 + ATP_HEADS * 2 * ATP_QHALF + ATP_NST * ATP_STAGE + 32 * 8 + 16;
+// Many queries per KV head (the compacted sequence's prefill, a chunk over a
+// cache): flash-style attention on tcgen05. A CTA takes one tile of 128 query
+// rows for two query heads of the same KV group, so each K and V block it
+// streams serves both. Per block j of 128 keys and head x: S_x = Q_x K_j^T
+// (M = 128 queries, N = 128 keys, K = 128 features) into tensor memory; four
+// warps per head (one query row per thread) read the row, take its maximum,
+// write p = 2^(s*scale*log2e - m) as bf16 over the score columns they have
+// just read (the A operand of the next product) and add p to the row sum l;
+// then O_x += P_x V_j (N = 128 features, K = 128 keys) accumulates in tensor
+// memory. V is read as it lies in the cache: its [key][feature] tile is the
+// feature-major ("MN-major") B operand. The reference maximum m of a row moves
+// only when the block maximum exceeds it by more than 8 (a factor 256): then
+// that row's O and l are scaled by 2^(m_old - m_new) before the next product
+// (otherwise p stays below 256, well inside bf16 and fp32); the final output
+// is O / l either way. Tensor-core work of one head overlaps the other head's
+// softmax: the issue order is PV_0(j), S_0(j+1), PV_1(j), S_1(j+1), and PV
+// starts on the first 64 keys of P while the second 64 are still being
+// exponentiated. Warps 0-7 take the softmax rows, warp 8 streams K and V
+// blocks by TMA through a five-slot ring, warp 9 issues the MMAs. Every wait is bounded; on a timeout the CTA
+// records DECOMOE_ERR_TIMEOUT, lets its copies and MMAs land, frees its tensor
+// memory and returns.
+//
+// Bound: the tensor pipe, once one head's chain (score product, row softmax,
+// P back to tensor memory, value product) fits under the other head's
+// products. Blocks of 128 keys halve the hand-offs per key against 64, and a
+// 128-column score product reads shared memory at its own rate (64 columns:
+// 1.5 times over it); packed fp32 pairs and 208 registers keep a row's 128
+// scores in registers without a spill. 32 query heads on 4 KV heads: 16384
+// rows 1999 -> 1511 us (1100 -> 1455 TFLOP/s), 1553 rows 39.4 -> 26.6 us, 509
+// rows over 4605 keys 90.8 -> 59.7 us against 64-key blocks with a separate
+// transpose of V.
+constexpr int ATP_BM = 128;                  // query rows per CTA
+constexpr int ATP_BN = 128;                  // keys per block
+constexpr int ATP_HEADS = 2;                 // query heads per CTA (same KV head)
+constexpr int ATP_NST = 5;                   // ring slots, each one K or one V block
+constexpr int ATP_HALF = 128 * 64 * 2;       // 128 rows x 64 features, 128-byte swizzle (16 KB)
+constexpr int ATP_SLOT = 2 * ATP_HALF;       // one block of 128 rows x 128 features
+constexpr int ATP_THREADS = ATP_HEADS * 128 + 128;  // two softmax warpgroups, TMA + MMA + two idle warps
+// Registers: 384 threads start with 168 each (504 per triple of warpgroups);
+// the softmax rows (128 scores in registers) take 208, the others 88.
+constexpr int ATP_REGS_SOFTMAX = 208, ATP_REGS_ISSUE = 88;
+static_assert(2 * ATP_REGS_SOFTMAX + ATP_REGS_ISSUE <= 3 * 168, "register split within the launch's total");
+constexpr int ATP_TMEM_COLS = 512;           // per head: S [0,128) (P over [0,64)), O [128,256)
+constexpr float ATP_RESCALE = 8.0f;          // log2 of the largest unnormalised p
+constexpr float ATP_NONE = -1.0e30f;         // reference maximum of a row that has seen no key
+constexpr size_t ATP_SMEM = 1024 + (ATP_HEADS + ATP_NST) * ATP_SLOT + 32 * 8 + 16;
+static_assert(ATP_SMEM <= 232448, "prefill attention shared memory");
 
 struct AttPreArgs {
   int64_t n, C;        // queries (the last n positions), keys
   int Hq, group;       // query heads, query heads per KV head
   float scale_log2;    // scale * log2(e)
-  __nv_bfloat16* out;  // [n, Hq, D]
   int32_t* status;
   uint64_t limit_ns;
 };
-
-// vt[g][d][s] = v[s][g][d] for s < C, 0 up to C_pad (pad columns must be
-// finite: their weights are zero)
-__global__ void __launch_bounds__(256)
-    k_attn_vt(const __nv_bfloat16* __restrict__ v, int64_t C, int Hkv, int64_t C_pad, __nv_bfloat16* __restrict__ vt) {
-  pdl_enter();
-  __shared__ __nv_bfloat16 tile[32][33];
-  const int64_t s0 = static_cast<int64_t>(blockIdx.x) * 32;
-  const int d0 = blockIdx.y * 32, g = blockIdx.z;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
-  for (int r = ty; r < 32; r += 8) {
-    const int64_t s = s0 + r;
-    tile[r][tx] = s < C ? v[(s * Hkv + g) * ATT_D + d0 + tx] : __float2bfloat16_rn(0.f);
-  }
-  __syncthreads();
-  for (int r = ty; r < 32; r += 8) {
-    const int64_t s = s0 + tx;
-    if (s < C_pad) vt[(static_cast<int64_t>(g) * ATT_D + d0 + r) * C_pad + s] = tile[tx][r];
-  }
-}
 
 // D(tmem) (+)= A(tmem) * B(smem desc)^T: A is 128 rows (lanes) x 16 bf16
 // (8 columns, two elements per 32-bit column, the lower index in the low half).
@@ -703,26 +699,69 @@ __device__ __forceinline__ float ex2_approx(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+// Two fp32 lanes in one 64-bit register pair (the packed fp32 pipe).
+__device__ __forceinline__ uint64_t f32x2(float lo, float hi) {
+  uint64_t v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+  return v;
+}
+__device__ __forceinline__ void f32x2_get(uint64_t v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t f32x2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t f32x2_add(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// 3-D TMA store (shared -> global), grouped for cp.async.bulk.wait_group.
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap* m, uint32_t src, int32_t x, int32_t y, int32_t z) {
+  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
+                   reinterpret_cast<uint64_t>(m)),
+               "r"(x), "r"(y), "r"(z), "r"(src)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
+// Descriptor of a [key][feature] tile as an MN-major B operand (N = features,
+// K = keys): 64 features per 128-byte swizzled row, 8-key groups 1024 bytes
+// apart (stride offset), the second 64 features ATP_HALF bytes on (leading
+// offset). Advancing 16 keys adds 2048 bytes.
+__device__ __forceinline__ uint64_t smem_desc_v(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
+  d |= static_cast<uint64_t>(ATP_HALF >> 4) << 16;
+  d |= static_cast<uint64_t>(1024 >> 4) << 32;
+  d |= static_cast<uint64_t>(1) << 46;
+  d |= static_cast<uint64_t>(2) << 61;
+  return d;
+}
 
 __global__ void __launch_bounds__(ATP_THREADS, 1)
     k_attn_prefill(const __grid_constant__ CUtensorMap tma_q, const __grid_constant__ CUtensorMap tma_k,
-                   const __grid_constant__ CUtensorMap tma_vt, const AttPreArgs a) {
+                   const __grid_constant__ CUtensorMap tma_v, const __grid_constant__ CUtensorMap tma_o,
+                   const AttPreArgs a) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t pad = (1024u - (raw & 1023u)) & 1023u;
   uint8_t* smem = smem_raw + pad;
-  const uint32_t sQ = raw + pad;                              // [head][feature half]
-  const uint32_t sKV = sQ + ATP_HEADS * 2 * ATP_QHALF;        // [stage]{K half 0, K half 1, V^T}
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + ATP_HEADS * 2 * ATP_QHALF + ATP_NST * ATP_STAGE);
+  const uint32_t sQ = raw + pad;                     // [head][feature half]; the output tile at the end
+  const uint32_t sKV = sQ + ATP_HEADS * ATP_SLOT;    // ring: K_0, V_0, K_1, V_1, ...
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (ATP_HEADS + ATP_NST) * ATP_SLOT);
   volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(bars + 32);
   volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
   const uint32_t bar0 = smem_u32(bars);
   const uint32_t Q_BAR = bar0, DRAIN = bar0 + 8;
   auto S_FULL = [&](int x) { return bar0 + 16u + 8u * x; };
-  auto P_FULL = [&](int x) { return bar0 + 32u + 8u * x; };
-  auto O_FINAL = [&](int x) { return bar0 + 48u + 8u * x; };
-  auto FULL = [&](int st) { return bar0 + 64u + 8u * st; };
-  auto EMPTY = [&](int st) { return bar0 + 96u + 8u * st; };
+  auto P_FULL = [&](int x, int half) { return bar0 + 32u + 16u * x + 8u * half; };
+  auto O_FINAL = [&](int x) { return bar0 + 64u + 8u * x; };
+  auto FULL = [&](int st) { return bar0 + 80u + 8u * st; };
+  auto EMPTY = [&](int st) { return bar0 + 80u + 8u * ATP_NST + 8u * st; };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int npair = a.Hq / ATP_HEADS;
@@ -742,7 +781,8 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
     mbar_init(DRAIN, 1);
     for (int x = 0; x < ATP_HEADS; ++x) {
       mbar_init(S_FULL(x), 1);
-      mbar_init(P_FULL(x), 128);
+      mbar_init(P_FULL(x, 0), 128);
+      mbar_init(P_FULL(x, 1), 128);
       mbar_init(O_FINAL(x), 1);
     }
     for (int st = 0; st < ATP_NST; ++st) {
@@ -751,79 +791,85 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
     }
     fence_mbar_init();
   }
-  if (warp == 1) {
+  if (warp == 9) {
     tmem_alloc(smem_u32(const_cast<uint32_t*>(s_tmem)), ATP_TMEM_COLS);
     tmem_relinquish();
   }
-  pdl_wait();  // q, k and the transposed v are ready
+  pdl_wait();  // q, k and v are ready
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *s_tmem;
   auto S_TM = [&](int x) { return tmem + 256u * x; };
-  auto P_TM = [&](int x) { return tmem + 256u * x + 64u; };
   auto O_TM = [&](int x) { return tmem + 256u * x + 128u; };
   constexpr uint32_t IDESC_S = idesc_bf16_f32(ATP_BM, ATP_BN);
-  constexpr uint32_t IDESC_O = idesc_bf16_f32(ATP_BM, ATT_D);
+  constexpr uint32_t IDESC_O = idesc_bf16_f32(ATP_BM, ATT_D) | (1u << 16);  // B MN-major
 
-  if (warp == 0) {
+  if (warp >= 8) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ATP_REGS_ISSUE));
+  if (warp == 8) {
     // ------------------------------------------------ TMA producer (lane 0)
     if (lane == 0) {
       tma_prefetch_desc(&tma_q);
       tma_prefetch_desc(&tma_k);
-      tma_prefetch_desc(&tma_vt);
+      tma_prefetch_desc(&tma_v);
+      tma_prefetch_desc(&tma_o);
       bool ok = true;
       uint32_t armed = 0, armed_ph = 0;
-      mbar_arrive_expect_tx(Q_BAR, ATP_HEADS * 2 * ATP_QHALF);
+      mbar_arrive_expect_tx(Q_BAR, ATP_HEADS * ATP_SLOT);
       const int qrow0 = qt * ATP_BM;
       for (int x = 0; x < ATP_HEADS; ++x)
-        for (int kb = 0; kb < 2; ++kb) tma_load_3d(sQ + (2 * x + kb) * ATP_QHALF, &tma_q, Q_BAR, 64 * kb, h0 + x, qrow0);
-      for (int j = 0; j < nblk; ++j) {
-        const int st = j % ATP_NST;
-        const uint32_t ph = (j / ATP_NST) & 1;
+        for (int kb = 0; kb < 2; ++kb) tma_load_3d(sQ + x * ATP_SLOT + kb * ATP_HALF, &tma_q, Q_BAR, 64 * kb, h0 + x, qrow0);
+      int st = 0;
+      uint32_t ph = 0;
+      for (int i = 0; i < 2 * nblk; ++i) {  // K_0, V_0, K_1, V_1, ...
         if (!mbar_wait(EMPTY(st), ph ^ 1u, a.limit_ns, s_abort)) {
           ok = false;
           break;
         }
-        mbar_arrive_expect_tx(FULL(st), ATP_STAGE);
-        const int key0 = j * ATP_BN;
-        const uint32_t base = sKV + st * ATP_STAGE;
-        tma_load_3d(base, &tma_k, FULL(st), 0, g, key0);
-        tma_load_3d(base + ATP_KHALF, &tma_k, FULL(st), 64, g, key0);
-        tma_load_3d(base + 2 * ATP_KHALF, &tma_vt, FULL(st), key0, 0, g);
+        mbar_arrive_expect_tx(FULL(st), ATP_SLOT);
+        const int key0 = (i >> 1) * ATP_BN;
+        const uint32_t base = sKV + st * ATP_SLOT;
+        const CUtensorMap* tm = (i & 1) ? &tma_v : &tma_k;
+        tma_load_3d(base, tm, FULL(st), 0, g, key0);
+        tma_load_3d(base + ATP_HALF, tm, FULL(st), 64, g, key0);
         armed |= 1u << st;
         armed_ph = (armed_ph & ~(1u << st)) | (ph << st);
+        if (++st == ATP_NST) {
+          st = 0;
+          ph ^= 1u;
+        }
       }
       if (!ok) {
         *s_abort = 1;
         report_status(a.status, DECOMOE_ERR_TIMEOUT);
         int no_abort = 0;
         mbar_wait(Q_BAR, 0, a.limit_ns, &no_abort);
-        for (int st = 0; st < ATP_NST; ++st)
-          if ((armed >> st) & 1u) mbar_wait(FULL(st), (armed_ph >> st) & 1u, a.limit_ns, &no_abort);
+        for (int s = 0; s < ATP_NST; ++s)
+          if ((armed >> s) & 1u) mbar_wait(FULL(s), (armed_ph >> s) & 1u, a.limit_ns, &no_abort);
       }
     }
-  } else if (warp == 1) {
+  } else if (warp == 9) {
     // ------------------------------------------------ MMA issuer (lane 0)
     if (lane == 0) {
       // S_x = Q_x K^T over the 128 features (two 64-feature halves)
       auto issue_s = [&](int x, int st) {
-        const uint32_t base = sKV + st * ATP_STAGE;
+        const uint64_t ad = smem_desc_kmajor<64>(sQ + x * ATP_SLOT);
+        const uint64_t bd = smem_desc_kmajor<64>(sKV + st * ATP_SLOT);
 #pragma unroll
-        for (int kb = 0; kb < 2; ++kb) {
-          const uint64_t ad = smem_desc_kmajor<64>(sQ + (2 * x + kb) * ATP_QHALF);
-          const uint64_t bd = smem_desc_kmajor<64>(base + kb * ATP_KHALF);
+        for (int kb = 0; kb < 2; ++kb)
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
-            tc_mma_f16(S_TM(x), ad + 2u * kk, bd + 2u * kk, IDESC_S, (kb | kk) != 0 ? 1u : 0u);
-        }
+            tc_mma_f16(S_TM(x), ad + (ATP_HALF >> 4) * kb + 2u * kk, bd + (ATP_HALF >> 4) * kb + 2u * kk, IDESC_S,
+                       (kb | kk) != 0 ? 1u : 0u);
       };
-      // O_x += P_x V_j over the block's 64 keys
-      auto issue_pv = [&](int x, int st, bool acc) {
-        const uint64_t bd = smem_desc_kmajor<64>(sKV + st * ATP_STAGE + 2 * ATP_KHALF);
+      // O_x += P_x V_j over 64 of the block's keys
+      auto issue_pv = [&](int x, int st, int half, bool acc) {
+        const uint64_t bd = smem_desc_v(sKV + st * ATP_SLOT);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          tc_mma_f16_ts(O_TM(x), P_TM(x) + 8u * kk, bd + 2u * kk, IDESC_O, (acc || kk > 0) ? 1u : 0u);
+          tc_mma_f16_ts(O_TM(x), S_TM(x) + 32u * half + 8u * kk, bd + (2048u >> 4) * (4 * half + kk), IDESC_O,
+                        (acc || half > 0 || kk > 0) ? 1u : 0u);
       };
       bool ok = mbar_wait(Q_BAR, 0, a.limit_ns, s_abort) && mbar_wait(FULL(0), 0, a.limit_ns, s_abort);
       bool issued = false;
@@ -833,32 +879,53 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
           issue_s(x, 0);
           tc_commit(S_FULL(x));
         }
+        tc_commit(EMPTY(0));
         issued = true;
       }
+      int st = 1;  // ring slot of V_j, then of K_{j+1}
+      uint32_t ph = 0;
       for (int j = 0; ok && j < nblk; ++j) {
-        const int st = j % ATP_NST;
-        for (int x = 0; x < ATP_HEADS; ++x) {
-          if (!mbar_wait(P_FULL(x), j & 1, a.limit_ns, s_abort)) {
+        int stk = st + 1;
+        uint32_t phk = ph;
+        if (stk == ATP_NST) {
+          stk = 0;
+          phk ^= 1u;
+        }
+        for (int x = 0; ok && x < ATP_HEADS; ++x) {
+          if (x == 0 && !mbar_wait(FULL(st), ph, a.limit_ns, s_abort)) {
             ok = false;
             break;
           }
-          tc_fence_after();
-          issue_pv(x, st, j > 0);
-          if (x == ATP_HEADS - 1) tc_commit(EMPTY(st));  // K_j and V_j read by every product
+          for (int half = 0; half < 2; ++half) {
+            if (!mbar_wait(P_FULL(x, half), j & 1, a.limit_ns, s_abort)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            issue_pv(x, st, half, j > 0);
+          }
+          if (!ok) break;
+          if (x == ATP_HEADS - 1) tc_commit(EMPTY(st));  // V_j read by both heads' products
           if (j + 1 < nblk) {
-            const int st1 = (j + 1) % ATP_NST;
             if (x == 0) {
-              if (!mbar_wait(FULL(st1), ((j + 1) / ATP_NST) & 1, a.limit_ns, s_abort)) {
+              if (!mbar_wait(FULL(stk), phk, a.limit_ns, s_abort)) {
                 ok = false;
                 break;
               }
               tc_fence_after();
             }
-            issue_s(x, st1);
+            issue_s(x, stk);
             tc_commit(S_FULL(x));
+            if (x == ATP_HEADS - 1) tc_commit(EMPTY(stk));
           } else {
             tc_commit(O_FINAL(x));
           }
+        }
+        st = stk + 1;
+        ph = phk;
+        if (st == ATP_NST) {
+          st = 0;
+          ph ^= 1u;
         }
       }
       if (!ok) {
@@ -871,9 +938,11 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
         }
       }
     }
+  }
   } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(ATP_REGS_SOFTMAX));
     // ------------------------------------------------ softmax rows
-    const int x = (warp - 2) >> 2;          // head of this warp
+    const int x = warp >> 2;                // head of this warp
     const int q = warp & 3;                 // tensor-memory lane quarter of this warp
     const int r = q * 32 + lane;            // query row of the tile
     const int64_t climit = a.C - 1;
@@ -881,7 +950,8 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
     const int64_t wlim = p0 + q * 32 < climit ? p0 + q * 32 : climit;          // smallest of the warp's rows
     const uint32_t lane_off = static_cast<uint32_t>(q * 32) << 16;
     const float sl2 = a.scale_log2;
-    float m = 0.f, l = 0.f;
+    const uint64_t sl2x2 = f32x2(sl2, sl2);
+    float m = ATP_NONE, l = 0.f;
     bool ok = true;
     for (int j = 0; j < nblk; ++j) {
       if (!__all_sync(0xffffffffu, mbar_wait(S_FULL(x), j & 1, a.limit_ns, s_abort))) {  // warp-uniform loads
@@ -891,30 +961,32 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
       tc_fence_after();
       const int64_t key0 = static_cast<int64_t>(j) * ATP_BN;
       uint32_t sv[ATP_BN];
-      tmem_ld32(S_TM(x) + lane_off, *reinterpret_cast<uint32_t(*)[32]>(&sv[0]));
-      tmem_ld32(S_TM(x) + lane_off + 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[32]));
+#pragma unroll
+      for (int c = 0; c < ATP_BN / 32; ++c)
+        tmem_ld32(S_TM(x) + lane_off + 32 * c, *reinterpret_cast<uint32_t(*)[32]>(&sv[32 * c]));
       tc_wait_ld();
       after_wait(sv);
       if (key0 + ATP_BN - 1 > wlim) {  // the causal edge or the end of the keys crosses this warp's rows
         const int64_t d = qlim - key0;
-        const int lim = d < 0 ? -1 : static_cast<int>(d);  // d < 64 here
+        const int lim = d < 0 ? -1 : (d < ATP_BN ? static_cast<int>(d) : ATP_BN);
 #pragma unroll
         for (int c = 0; c < ATP_BN; ++c)
           if (c > lim) sv[c] = __float_as_uint(-INFINITY);
       }
       float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-      for (int c = 0; c < ATP_BN; ++c) mx[c & 3] = fmaxf(mx[c & 3], __uint_as_float(sv[c]));
+      for (int c = 0; c < ATP_BN; c += 8)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          mx[u] = fmaxf(fmaxf(mx[u], __uint_as_float(sv[c + 2 * u])), __uint_as_float(sv[c + 2 * u + 1]));
       const float m_blk = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
       float factor = 1.0f;
-      if (j == 0) {
-        m = m_blk;  // key 0 is visible to every row
-      } else if (m_blk > m + ATP_RESCALE) {
-        factor = ex2_approx(m - m_blk);
+      if (m_blk > m + ATP_RESCALE) {
+        factor = ex2_approx(m - m_blk);  // 0 for a row that had seen no key
         m = m_blk;
         l *= factor;
       }
-      if (__any_sync(0xffffffffu, factor != 1.0f)) {
+      if (j > 0 && __any_sync(0xffffffffu, factor != 1.0f)) {
         // the previous product into O has completed (S_FULL is committed after it)
 #pragma unroll
         for (int c = 0; c < ATT_D / 32; ++c) {
@@ -927,40 +999,59 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
           tmem_st32(O_TM(x) + lane_off + 32 * c, ov);
         }
       }
-      float ls[4] = {0.f, 0.f, 0.f, 0.f};
-      uint32_t pk[32];
+      const uint64_t negm = f32x2(-m, -m);
+      uint64_t ls[2] = {0ull, 0ull};
 #pragma unroll
-      for (int c = 0; c < ATP_BN; c += 2) {
-        const float e0 = ex2_approx(fmaf(__uint_as_float(sv[c]), sl2, -m));
-        const float e1 = ex2_approx(fmaf(__uint_as_float(sv[c + 1]), sl2, -m));
-        ls[(c >> 1) & 3] += e0 + e1;
-        pk[c >> 1] = pack_bf16x2(e0, e1);
+      for (int half = 0; half < 2; ++half) {
+        uint32_t pk[32];
+#pragma unroll
+        for (int c = 0; c < 32; ++c) {
+          const int k = 64 * half + 2 * c;
+          float e0, e1;
+          f32x2_get(f32x2_fma(f32x2(__uint_as_float(sv[k]), __uint_as_float(sv[k + 1])), sl2x2, negm), e0, e1);
+          e0 = ex2_approx(e0);
+          e1 = ex2_approx(e1);
+          ls[c & 1] = f32x2_add(ls[c & 1], f32x2(e0, e1));
+          pk[c] = pack_bf16x2(e0, e1);
+        }
+        tmem_st32(S_TM(x) + lane_off + 32 * half, pk);  // P over the score columns
+        tc_wait_st();
+        tc_fence_before();
+        mbar_arrive(P_FULL(x, half));
       }
-      l += (ls[0] + ls[1]) + (ls[2] + ls[3]);
-      tmem_st32(P_TM(x) + lane_off, pk);
-      tc_wait_st();
-      tc_fence_before();
-      mbar_arrive(P_FULL(x));
+      float l0, l1;
+      f32x2_get(f32x2_add(ls[0], ls[1]), l0, l1);
+      l += l0 + l1;
     }
     if (ok && __all_sync(0xffffffffu, mbar_wait(O_FINAL(x), 0, a.limit_ns, s_abort))) {
       tc_fence_after();
+      // O / l as bf16 over the head's Q tile (every product has read it), in
+      // the 128-byte swizzle, then one TMA store per 64 features: whole lines,
+      // rows past n clipped
       const float inv = 1.0f / l;
-      const int64_t row = static_cast<int64_t>(qt) * ATP_BM + r;
-      uint4* dst = reinterpret_cast<uint4*>(a.out + (row * a.Hq + h0 + x) * ATT_D);
+      uint8_t* so = smem + x * ATP_SLOT + r * 128;
 #pragma unroll
       for (int c = 0; c < ATT_D / 32; ++c) {
         uint32_t ov[32];
         tmem_ld32(O_TM(x) + lane_off + 32 * c, ov);
         tc_wait_ld();
         after_wait(ov);
-        if (row < a.n) {
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const float* o = reinterpret_cast<const float*>(&ov[8 * u]);
-            dst[4 * c + u] = make_uint4(pack_bf16x2(o[0] * inv, o[1] * inv), pack_bf16x2(o[2] * inv, o[3] * inv),
-                                        pack_bf16x2(o[4] * inv, o[5] * inv), pack_bf16x2(o[6] * inv, o[7] * inv));
-          }
+        for (int u = 0; u < 4; ++u) {
+          const float* o = reinterpret_cast<const float*>(&ov[8 * u]);
+          const int chunk = (4 * (c & 1) + u) ^ (r & 7);
+          *reinterpret_cast<uint4*>(so + (c >> 1) * ATP_HALF + 16 * chunk) =
+              make_uint4(pack_bf16x2(o[0] * inv, o[1] * inv), pack_bf16x2(o[2] * inv, o[3] * inv),
+                         pack_bf16x2(o[4] * inv, o[5] * inv), pack_bf16x2(o[6] * inv, o[7] * inv));
         }
+      }
+      fence_proxy_async_smem();
+      named_bar_sync(1 + x, 128);  // the head's four warps
+      if (q == 0 && lane == 0) {
+        for (int kb = 0; kb < 2; ++kb)
+          tma_store_3d(&tma_o, sQ + x * ATP_SLOT + kb * ATP_HALF, 64 * kb, h0 + x, qt * ATP_BM);
+        bulk_commit();
+        bulk_wait_all();
       }
     } else {
       *s_abort = 1;
@@ -970,7 +1061,7 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
   pdl_trigger();
   tc_fence_before();
   __syncthreads();
-  if (warp == 1) {
+  if (warp == 9) {
     __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem, ATP_TMEM_COLS);
@@ -984,12 +1075,10 @@ using namespace decomoe;
 extern "C" {
 
 static bool att_use_prefill(int64_t n, int Hq, int Hkv) { return n * (Hq / Hkv) > ATT_MAXQ; }
-static int64_t att_c_pad(int64_t C) { return (C + 63) / 64 * 64; }
 
 size_t decomoe_attention_workspace_bytes(int64_t n, int64_t C, int Hq, int Hkv, int D) {
   if (n <= 0 || C <= 0 || Hq <= 0 || Hkv <= 0 || D != ATT_D || Hq % Hkv != 0) return 0;
-  if (att_use_prefill(n, Hq, Hkv))  // the transposed values [Hkv][D][C padded to 64]
-    return align_up(static_cast<size_t>(Hkv) * ATT_D * att_c_pad(C) * 2, 256);
+  if (att_use_prefill(n, Hq, Hkv)) return 0;
   // decode sizes: a cluster's splits merge through its shared memory; several
   // clusters per head (long caches) leave their merged rows here
   const int nq = static_cast<int>(n) * (Hq / Hkv);
@@ -1022,29 +1111,23 @@ int decomoe_attention(const void* q, int64_t n, const void* k_cache, const void*
   if (att_use_prefill(n, Hq, Hkv)) {
     DM_ARG_CHECK(G % ATP_HEADS == 0, "attention: prefill sizes need an even number of query heads per KV head (%d)",
                  G);
-    // V transposed (keys contiguous) so that P V_j takes K-major operands
-    const int64_t C_pad = att_c_pad(C);
-    __nv_bfloat16* vt = static_cast<__nv_bfloat16*>(ws);
-    DM_CUDA_CHECK(launch_pdl(k_attn_vt, dim3(static_cast<unsigned>(C_pad / 32), ATT_D / 32, Hkv), dim3(256), 0, s,
-                             static_cast<const __nv_bfloat16*>(v_cache), C, Hkv, C_pad, vt));
-    CUtensorMap tq, tk, tv;
+    // [rows][heads][D] in boxes of 128 rows x 64 features of one head
+    CUtensorMap tq, tk, tv, to;
     const uint64_t dq[3] = {static_cast<uint64_t>(D), static_cast<uint64_t>(Hq), static_cast<uint64_t>(n)};
     const uint64_t sq[2] = {static_cast<uint64_t>(D) * 2, static_cast<uint64_t>(Hq) * D * 2};
     const uint64_t dk[3] = {static_cast<uint64_t>(D), static_cast<uint64_t>(Hkv), static_cast<uint64_t>(C)};
     const uint64_t sk[2] = {static_cast<uint64_t>(D) * 2, static_cast<uint64_t>(Hkv) * D * 2};
-    const uint64_t dv[3] = {static_cast<uint64_t>(C_pad), static_cast<uint64_t>(D), static_cast<uint64_t>(Hkv)};
-    const uint64_t sv[2] = {static_cast<uint64_t>(C_pad) * 2, static_cast<uint64_t>(D) * C_pad * 2};
-    const uint32_t bq[3] = {64, 1, ATP_BM}, bk[3] = {64, 1, ATP_BN}, bv[3] = {ATP_BN, ATT_D, 1};
+    const uint32_t bq[3] = {64, 1, ATP_BM}, bk[3] = {64, 1, ATP_BN};
     DM_RET(make_tmap_bf16_3d(&tq, q, dq, sq, bq));
     DM_RET(make_tmap_bf16_3d(&tk, k_cache, dk, sk, bk));
-    DM_RET(make_tmap_bf16_3d(&tv, vt, dv, sv, bv));
+    DM_RET(make_tmap_bf16_3d(&tv, v_cache, dk, sk, bk));
+    DM_RET(make_tmap_bf16_3d(&to, out, dq, sq, bq));
     AttPreArgs pa;
     pa.n = n;
     pa.C = C;
     pa.Hq = Hq;
     pa.group = G;
     pa.scale_log2 = sc * 1.4426950408889634f;
-    pa.out = static_cast<__nv_bfloat16*>(out);
     pa.status = status_dev;
     pa.limit_ns = static_cast<uint64_t>(wait_limit_ns());
     const int64_t ntile = (n + ATP_BM - 1) / ATP_BM;
@@ -1053,7 +1136,7 @@ int decomoe_attention(const void* q, int64_t n, const void* k_cache, const void*
                                        static_cast<int>(ATP_SMEM)));
     DM_CUDA_CHECK(launch_pdl(k_attn_prefill, dim3(static_cast<unsigned>(ntile * (Hq / ATP_HEADS))), dim3(ATP_THREADS),
                              ATP_SMEM, s,
-                             tq, tk, tv, pa));
+                             tq, tk, tv, to, pa));
     return DECOMOE_OK;
   }
   AttDecArgs a;

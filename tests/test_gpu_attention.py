@@ -72,6 +72,16 @@ def test_attention_prefill_parity(n, C):
     assert_close_out(f64(out), ref, BF16_REL_L2, BF16_MAX_ABS, f"prefill attention n={n} C={C}")
 
 
+@pytest.mark.parametrize("n,C", [(17, 17), (127, 127), (127, 255), (128, 256), (129, 385), (255, 256), (257, 511),
+                                 (130, 1025)])
+def test_attention_prefill_key_block_edges(n, C):
+    """Tiles whose causal edge and key count fall on, before and after a
+    128-key block's edge (a tile's rows then end in one or in two blocks)."""
+    q, k, v = _qkv(n, C, seed=3 * C + n)
+    ref = O.attention(f64(q), f64(k), f64(v))
+    assert_close_out(f64(_run(q, k, v)), ref, BF16_REL_L2, BF16_MAX_ABS, f"prefill attention n={n} C={C}")
+
+
 def _sampled_rows(out, q, k, v, rows, label):
     """Query row i of a launch over (n, C) is attention at position C - n + i
     over keys 0..C - n + i: the oracle on that one row and prefix."""
