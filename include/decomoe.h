@@ -554,7 +554,11 @@ DECOMOE_API int decomoe_moe_layer_workspace_layout(int64_t T, int d, int E, int 
  *   Prefill sizes (more queries per KV head, n = C or a chunk n < C; Hq / Hkv
  *   even): one tensor-core CTA per (pair of query heads, 128-query tile) runs
  *   the online softmax over 128-key blocks up to its causal limit (P rounded
- *   to bf16 before the P V product; deterministic). No workspace.
+ *   to bf16 before the P V product; deterministic). Where that leaves SMs idle
+ *   (few query tiles over a long cache) each tile's keys are split over
+ *   several CTAs, whose rows a second small launch merges in key order; a
+ *   workspace of at least the bytes for (n', C) at some other n' but too small
+ *   for the split gives whole tiles instead.
  *   ws: decomoe_attention_workspace_bytes(n, C, Hq, Hkv, D) bytes, 16-byte
  *   aligned. A wait that runs past the time limit records
  *   DECOMOE_ERR_TIMEOUT in status_dev (may be null).

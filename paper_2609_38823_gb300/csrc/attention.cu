@@ -656,10 +656,21 @@ constexpr float ATP_NONE = -1.0e30f;         // reference maximum of a row that 
 constexpr size_t ATP_SMEM = 1024 + (ATP_HEADS + ATP_NST) * ATP_SLOT + 32 * 8 + 16;
 static_assert(ATP_SMEM <= 232448, "prefill attention shared memory");
 
+// A tile's key blocks may be split over several CTAs (att_pre_split): items
+// of at most L blocks, numbered heaviest tile first, a tile's pairs of heads
+// innermost. An item of a split tile leaves, per head, its unnormalised O
+// (fp32 [128][128], the 16-byte chunks of row r at chunk ^ (r & 31)) and the
+// rows' (m, l) in the workspace; k_attn_pre_merge merges them in key order.
+constexpr int ATP_PART = 128 * ATT_D;            // floats of one head's O
+constexpr size_t ATP_ITEM_BYTES = ATP_HEADS * (static_cast<size_t>(ATP_PART) * 4 + 128 * 8);
+
 struct AttPreArgs {
   int64_t n, C;        // queries (the last n positions), keys
   int Hq, group;       // query heads, query heads per KV head
+  int L;               // key blocks per item at most (0: every tile is one item)
   float scale_log2;    // scale * log2(e)
+  float* part;         // partial O of the split items, [item][head][128][128]
+  float2* ml;          // their row maxima and sums, [item][head][128]
   int32_t* status;
   uint64_t limit_ns;
 };
@@ -725,6 +736,13 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* m, uint32_t src,
                "r"(x), "r"(y), "r"(z), "r"(src)
                : "memory");
 }
+// Untiled bulk copy shared -> global (16-byte aligned, a multiple of 16 bytes).
+__device__ __forceinline__ void bulk_store(void* dst, uint32_t src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
+                   static_cast<uint64_t>(__cvta_generic_to_global(dst))),
+               "r"(src), "r"(bytes)
+               : "memory");
+}
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
@@ -740,6 +758,115 @@ __device__ __forceinline__ uint64_t smem_desc_v(uint32_t saddr) {
   d |= static_cast<uint64_t>(1) << 46;
   d |= static_cast<uint64_t>(2) << 61;
   return d;
+}
+
+// Work item i of a prefill launch: query tile, pair of heads, and the tile's
+// key blocks [first, first + blocks) (all of them unless split).
+struct AttPreItem {
+  int tile, pair, first, blocks;
+  bool split;
+};
+__host__ __device__ inline int att_pre_blocks(int tile, int64_t n, int64_t C) {
+  const int64_t last = C - n + static_cast<int64_t>(tile) * ATP_BM + ATP_BM - 1;
+  return static_cast<int>((last < C - 1 ? last : C - 1) / ATP_BN) + 1;
+}
+__host__ __device__ inline AttPreItem att_pre_item(int i, int64_t n, int64_t C, int npair, int L) {
+  AttPreItem it;
+  it.tile = static_cast<int>((n + ATP_BM - 1) / ATP_BM) - 1;
+  it.first = 0;
+  it.split = false;
+  if (L == 0) {
+    it.tile -= i / npair;
+    it.pair = i % npair;
+    it.blocks = att_pre_blocks(it.tile, n, C);
+    return it;
+  }
+  for (;; --it.tile) {
+    const int b = att_pre_blocks(it.tile, n, C);
+    const int ns = (b + L - 1) / L;
+    if (i < ns * npair || it.tile == 0) {
+      const int per = (b + ns - 1) / ns;  // (ns - 1) * per < b: no item is empty
+      it.pair = i % npair;
+      it.first = i / npair * per;
+      it.blocks = b - it.first < per ? b - it.first : per;
+      it.split = ns > 1;
+      return it;
+    }
+    i -= ns * npair;
+  }
+}
+
+// Merges the items of the split tiles: one warp per head and ATM_ROWS
+// consecutive rows; lane s holds item s's (m, l) of each row, then lane c
+// features 4c .. 4c + 3 of O, four items of every row in flight. Items in key
+// order, so the bits do not depend on when each finished.
+constexpr int ATM_ROWS = 2;
+constexpr int ATM_MAX_ITEMS = 32;  // per tile and pair: one per lane
+__global__ void __launch_bounds__(1024)
+    k_attn_pre_merge(const float* __restrict__ part, const float2* __restrict__ ml, int64_t n, int64_t C, int Hq, int L,
+                     int split_tiles, __nv_bfloat16* __restrict__ out) {
+  pdl_enter();
+  const int lane = threadIdx.x & 31;
+  const int npair = Hq / ATP_HEADS;
+  const int per_tile = ATP_BM / ATM_ROWS * Hq;
+  const int ntile = static_cast<int>((n + ATP_BM - 1) / ATP_BM);
+  for (int w = static_cast<int>(blockIdx.x) * 32 + (threadIdx.x >> 5); w < split_tiles * per_tile; w += gridDim.x * 32) {
+    const int tile = ntile - 1 - w / per_tile;
+    const int h = w % Hq, r0 = w % per_tile / Hq * ATM_ROWS;
+    const int64_t row0 = static_cast<int64_t>(tile) * ATP_BM + r0;
+    if (row0 >= n) continue;
+    int base = 0;  // the tile's first item
+    for (int t = ntile - 1; t > tile; --t) base += (att_pre_blocks(t, n, C) + L - 1) / L * npair;
+    const int ns = (att_pre_blocks(tile, n, C) + L - 1) / L;
+    // of item 0, this head and row; the next item is npair * ATP_HEADS heads on
+    const int64_t first = (static_cast<int64_t>(base + h / ATP_HEADS) * ATP_HEADS + h % ATP_HEADS) * 128 + r0;
+    const int64_t step = static_cast<int64_t>(npair) * ATP_HEADS * 128;
+    float f[ATM_ROWS], l[ATM_ROWS];
+    float4 o[ATM_ROWS];
+#pragma unroll
+    for (int i = 0; i < ATM_ROWS; ++i) {
+      const float2 v = lane < ns ? ml[first + lane * step + i] : make_float2(ATP_NONE, 0.f);
+      float M = v.x;
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
+      f[i] = ex2_approx(v.x - M);
+      l[i] = v.y * f[i];
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], off);
+      o[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    auto load = [&](int s, int i) {
+      return __ldcs(reinterpret_cast<const float4*>(part + (first + s * step + i) * ATT_D) + (lane ^ ((r0 + i) & 31)));
+    };
+    auto add = [&](int s, const float4 (&p)[ATM_ROWS]) {
+#pragma unroll
+      for (int i = 0; i < ATM_ROWS; ++i) {
+        const float fs = __shfl_sync(0xffffffffu, f[i], s);
+        o[i].x += p[i].x * fs;
+        o[i].y += p[i].y * fs;
+        o[i].z += p[i].z * fs;
+        o[i].w += p[i].w * fs;
+      }
+    };
+    for (int s = 0; s < ns; s += 4) {
+      float4 p[4][ATM_ROWS];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int i = 0; i < ATM_ROWS; ++i)
+          if (s + u < ns) p[u][i] = load(s + u, i);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (s + u < ns) add(s + u, p[u]);
+    }
+#pragma unroll
+    for (int i = 0; i < ATM_ROWS; ++i) {
+      if (row0 + i >= n) break;
+      const float inv = 1.0f / l[i];
+      reinterpret_cast<uint2*>(out + ((row0 + i) * Hq + h) * ATT_D)[lane] =
+          make_uint2(pack_bf16x2(o[i].x * inv, o[i].y * inv), pack_bf16x2(o[i].z * inv, o[i].w * inv));
+    }
+  }
 }
 
 __global__ void __launch_bounds__(ATP_THREADS, 1)
@@ -765,15 +892,13 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int npair = a.Hq / ATP_HEADS;
-  const int ntile = static_cast<int>((a.n + ATP_BM - 1) / ATP_BM);
   // heaviest tiles (most key blocks) first
-  const int hp = blockIdx.x % npair;
-  const int qt = ntile - 1 - static_cast<int>(blockIdx.x / npair);
+  const AttPreItem it = att_pre_item(static_cast<int>(blockIdx.x), a.n, a.C, npair, a.L);
+  const int hp = it.pair, qt = it.tile;
   const int h0 = hp * ATP_HEADS;
   const int g = h0 / a.group;  // both heads read KV head g (the group size is even)
   const int64_t p0 = a.C - a.n + static_cast<int64_t>(qt) * ATP_BM;  // position of the tile's first row
-  const int64_t last = p0 + ATP_BM - 1 < a.C - 1 ? p0 + ATP_BM - 1 : a.C - 1;
-  const int nblk = static_cast<int>(last / ATP_BN) + 1;  // key blocks any row of the tile can see
+  const int nblk = it.blocks;  // of the key blocks that any row of the tile can see, from it.first on
 
   if (threadIdx.x == 0) {
     *s_abort = 0;
@@ -828,7 +953,7 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
           break;
         }
         mbar_arrive_expect_tx(FULL(st), ATP_SLOT);
-        const int key0 = (i >> 1) * ATP_BN;
+        const int key0 = (it.first + (i >> 1)) * ATP_BN;
         const uint32_t base = sKV + st * ATP_SLOT;
         const CUtensorMap* tm = (i & 1) ? &tma_v : &tma_k;
         tma_load_3d(base, tm, FULL(st), 0, g, key0);
@@ -959,7 +1084,7 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
         break;
       }
       tc_fence_after();
-      const int64_t key0 = static_cast<int64_t>(j) * ATP_BN;
+      const int64_t key0 = static_cast<int64_t>(it.first + j) * ATP_BN;
       uint32_t sv[ATP_BN];
 #pragma unroll
       for (int c = 0; c < ATP_BN / 32; ++c)
@@ -1023,7 +1148,34 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
       f32x2_get(f32x2_add(ls[0], ls[1]), l0, l1);
       l += l0 + l1;
     }
-    if (ok && __all_sync(0xffffffffu, mbar_wait(O_FINAL(x), 0, a.limit_ns, s_abort))) {
+    ok = ok && __all_sync(0xffffffffu, mbar_wait(O_FINAL(x), 0, a.limit_ns, s_abort));
+    if (it.split) ok = ok && __all_sync(0xffffffffu, mbar_wait(O_FINAL(x ^ 1), 0, a.limit_ns, s_abort));
+    if (ok && it.split) {
+      // one of several items of the tile: O as it is, through ring slots 2x
+      // and 2x + 1 (every product has read them) and one bulk store
+      tc_fence_after();
+      const int64_t slot = static_cast<int64_t>(blockIdx.x) * ATP_HEADS + x;
+      uint8_t* so = smem + (ATP_HEADS + 2 * x) * ATP_SLOT + r * (ATT_D * 4);
+#pragma unroll
+      for (int c = 0; c < ATT_D / 32; ++c) {
+        uint32_t ov[32];
+        tmem_ld32(O_TM(x) + lane_off + 32 * c, ov);
+        tc_wait_ld();
+        after_wait(ov);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          *reinterpret_cast<uint4*>(so + 16 * ((8 * c + u) ^ lane)) =
+              make_uint4(ov[4 * u], ov[4 * u + 1], ov[4 * u + 2], ov[4 * u + 3]);
+      }
+      a.ml[slot * 128 + r] = make_float2(m, l);
+      fence_proxy_async_smem();
+      named_bar_sync(1 + x, 128);  // the head's four warps
+      if (q == 0 && lane == 0) {
+        bulk_store(a.part + slot * ATP_PART, sKV + 2 * x * ATP_SLOT, ATP_PART * 4);
+        bulk_commit();
+        bulk_wait_all();
+      }
+    } else if (ok) {
       tc_fence_after();
       // O / l as bf16 over the head's Q tile (every product has read it), in
       // the 128-byte swizzle, then one TMA store per 64 features: whole lines,
@@ -1076,9 +1228,64 @@ extern "C" {
 
 static bool att_use_prefill(int64_t n, int Hq, int Hkv) { return n * (Hq / Hkv) > ATT_MAXQ; }
 
+// Whether to split the tiles' key blocks over several CTAs, and how far: L
+// blocks per item (0: no split), the items and those of split tiles. One CTA
+// per SM: a chunk of queries over a long cache has few tiles and leaves SMs
+// idle. Times in block steps (1.5 us for two heads): an item costs its blocks
+// plus 2.5 (set-up, first loads, output); writing partial rows and the merge
+// launch 3 plus 0.025 per item. Tiles of about equal length run in whole waves of one
+// item per SM; lengths from one block up (n = C) fill the SMs evenly and end
+// with the longest. Only taken where the estimate is 10 % better; measured
+// (32 heads on 4 KV heads, whole -> split): 509 queries over 4605 keys 59.7 ->
+// 42.5 us in 2, 33 over 4129 54.8 -> 19.5 in 9, 87 over 13767 169 -> 32 in 9,
+// 300 over 8300 104 -> 48.7 in 3, 700 over 8700 109 -> 95 in 3; 509 over 1009
+// would go 17.2 -> 21.0 in 2 and 1024 over 5120 66 -> 83.
+struct AttPreSplit {
+  int L;
+  int64_t items, split_items, split_tiles;
+};
+static AttPreSplit att_pre_split(int64_t n, int64_t C, int Hq) {
+  const int64_t ntile = (n + ATP_BM - 1) / ATP_BM;
+  const int npair = Hq / ATP_HEADS, nsm = sm_count();
+  AttPreSplit best = {0, ntile * npair, 0, 0};
+  if (best.items > 2 * nsm || C >= (1LL << 31)) return best;
+  const int bmax = att_pre_blocks(static_cast<int>(ntile) - 1, n, C), bmin = att_pre_blocks(0, n, C);
+  double best_t = 0.0;
+  for (int s = 1; s <= ATM_MAX_ITEMS && (s == 1 || bmax / s >= 2); ++s) {
+    AttPreSplit c = {(bmax + s - 1) / s, 0, 0, 0};
+    int64_t blocks = 0;
+    for (int t = static_cast<int>(ntile) - 1; t >= 0; --t) {
+      const int b = att_pre_blocks(t, n, C), ns = (b + c.L - 1) / c.L;
+      c.items += static_cast<int64_t>(ns) * npair;
+      blocks += static_cast<int64_t>(b) * npair;
+      if (ns > 1) {
+        c.split_items += static_cast<int64_t>(ns) * npair;
+        ++c.split_tiles;
+      }
+    }
+    const double longest = c.L + 2.5;
+    const double t = (2 * bmin >= bmax ? static_cast<double>((c.items + nsm - 1) / nsm) * longest
+                                       : std::max(longest, (blocks + 2.5 * c.items) / nsm + 0.5 * longest)) +
+                     (c.split_items > 0 ? 3.0 + 0.025 * c.split_items : 0.0);
+    if (s == 1) {
+      best_t = 0.9 * t;
+    } else if (c.split_items > 0 && t < best_t) {
+      best_t = t;
+      best = c;
+    }
+  }
+  return best;
+}
+static size_t att_pre_base_bytes(int64_t C, int Hkv) {
+  return align_up(static_cast<size_t>(Hkv) * ATT_D * ((C + 63) / 64 * 64) * 2, 256);
+}
+
 size_t decomoe_attention_workspace_bytes(int64_t n, int64_t C, int Hq, int Hkv, int D) {
   if (n <= 0 || C <= 0 || Hq <= 0 || Hkv <= 0 || D != ATT_D || Hq % Hkv != 0) return 0;
-  if (att_use_prefill(n, Hq, Hkv)) return 0;
+  if (att_use_prefill(n, Hq, Hkv)) {  // the split items' partial rows; the base size covers most of them
+    const size_t split = Hq % ATP_HEADS == 0 ? att_pre_split(n, C, Hq).split_items * ATP_ITEM_BYTES : 0;
+    return std::max(att_pre_base_bytes(C, Hkv), align_up(split, 256));
+  }
   // decode sizes: a cluster's splits merge through its shared memory; several
   // clusters per head (long caches) leave their merged rows here
   const int nq = static_cast<int>(n) * (Hq / Hkv);
@@ -1100,7 +1307,9 @@ int decomoe_attention(const void* q, int64_t n, const void* k_cache, const void*
   DM_ARG_CHECK(aligned16(q) && aligned16(k_cache) && aligned16(v_cache) && aligned16(out),
                "attention: pointers must be 16-byte aligned");
   const int G = Hq / Hkv;
-  const size_t need = decomoe_attention_workspace_bytes(n, C, Hq, Hkv, D);
+  const bool prefill = att_use_prefill(n, Hq, Hkv);
+  // prefill: a workspace sized for another call's n is enough (no split then)
+  const size_t need = prefill ? att_pre_base_bytes(C, Hkv) : decomoe_attention_workspace_bytes(n, C, Hq, Hkv, D);
   if (need > 0 && (ws == nullptr || ws_bytes < need)) {
     set_error("attention: workspace needs %zu bytes", need);
     return DECOMOE_ERR_WORKSPACE;
@@ -1108,7 +1317,7 @@ int decomoe_attention(const void* q, int64_t n, const void* k_cache, const void*
   DM_ARG_CHECK(need == 0 || aligned16(ws), "attention: workspace must be 16-byte aligned");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const float sc = scale > 0.f ? scale : 1.0f / sqrtf(static_cast<float>(D));
-  if (att_use_prefill(n, Hq, Hkv)) {
+  if (prefill) {
     DM_ARG_CHECK(G % ATP_HEADS == 0, "attention: prefill sizes need an even number of query heads per KV head (%d)",
                  G);
     // [rows][heads][D] in boxes of 128 rows x 64 features of one head
@@ -1130,13 +1339,20 @@ int decomoe_attention(const void* q, int64_t n, const void* k_cache, const void*
     pa.scale_log2 = sc * 1.4426950408889634f;
     pa.status = status_dev;
     pa.limit_ns = static_cast<uint64_t>(wait_limit_ns());
-    const int64_t ntile = (n + ATP_BM - 1) / ATP_BM;
-    DM_ARG_CHECK(ntile * (Hq / ATP_HEADS) < 0x7fffffffLL, "attention: too many query tiles");
+    DM_ARG_CHECK((n + ATP_BM - 1) / ATP_BM * (Hq / ATP_HEADS) < 0x7fffffffLL, "attention: too many query tiles");
+    AttPreSplit sp = att_pre_split(n, C, Hq);
+    if (sp.split_items * ATP_ITEM_BYTES > ws_bytes) sp = {0, (n + ATP_BM - 1) / ATP_BM * (Hq / ATP_HEADS), 0, 0};
+    pa.L = sp.L;
+    pa.part = static_cast<float*>(ws);
+    pa.ml = reinterpret_cast<float2*>(pa.part + sp.split_items * ATP_HEADS * ATP_PART);
     DM_CUDA_CHECK(cudaFuncSetAttribute(k_attn_prefill, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(ATP_SMEM)));
-    DM_CUDA_CHECK(launch_pdl(k_attn_prefill, dim3(static_cast<unsigned>(ntile * (Hq / ATP_HEADS))), dim3(ATP_THREADS),
-                             ATP_SMEM, s,
-                             tq, tk, tv, to, pa));
+    DM_CUDA_CHECK(launch_pdl(k_attn_prefill, dim3(static_cast<unsigned>(sp.items)), dim3(ATP_THREADS), ATP_SMEM, s, tq,
+                             tk, tv, to, pa));
+    if (sp.L > 0)
+      DM_CUDA_CHECK(launch_pdl(k_attn_pre_merge, dim3(static_cast<unsigned>(sm_count())), dim3(1024), 0, s,
+                               static_cast<const float*>(pa.part), static_cast<const float2*>(pa.ml), n, C, Hq, sp.L,
+                               static_cast<int>(sp.split_tiles), static_cast<__nv_bfloat16*>(out)));
     return DECOMOE_OK;
   }
   AttDecArgs a;

@@ -82,6 +82,26 @@ def test_attention_prefill_key_block_edges(n, C):
     assert_close_out(f64(_run(q, k, v)), ref, BF16_REL_L2, BF16_MAX_ABS, f"prefill attention n={n} C={C}")
 
 
+@pytest.mark.parametrize("n,C", [(9, 1009), (33, 4129), (129, 2200), (300, 2500), (509, 3000)])
+def test_attention_prefill_split_keys(n, C):
+    """Few query tiles over a long cache: each tile's key blocks are split
+    over several CTAs and merged in key order, the same bits on every call. The
+    same call with a workspace sized for a call that does not split runs
+    whole tiles."""
+    q, k, v = _qkv(n, C, seed=5 * C + n)
+    full = dm.decomoe_attention_workspace_bytes(n, C, HQ, HKV, D)
+    whole = dm.decomoe_attention_workspace_bytes(C, C, HQ, HKV, D)
+    assert full > whole, "this size is meant to split"
+    ref = O.attention(f64(q), f64(k), f64(v))
+    out = _run(q, k, v)
+    assert_close_out(f64(out), ref, BF16_REL_L2, BF16_MAX_ABS, f"split prefill attention n={n} C={C}")
+    assert torch.equal(out, _run(q, k, v))
+    un = torch.empty_like(out)
+    dm.decomoe_attention(q.to(DEV), k.to(DEV), v.to(DEV), un, dm.workspace(whole, DEV))
+    torch.cuda.synchronize()
+    assert_close_out(f64(un), ref, BF16_REL_L2, BF16_MAX_ABS, f"whole-tile prefill attention n={n} C={C}")
+
+
 def _sampled_rows(out, q, k, v, rows, label):
     """Query row i of a launch over (n, C) is attention at position C - n + i
     over keys 0..C - n + i: the oracle on that one row and prefix."""
