@@ -25,6 +25,7 @@
 #include <cudaTypedefs.h>
 
 #include "decomoe_internal.cuh"
+#include "simt_rows.cuh"
 
 // Kernel choice for the bf16 expert GEMMs: the weights-stationary k_moe_ws
 // when the average expert gets at most DECOMOE_WS_MAX_AVG_ROWS rows (decode
@@ -2245,11 +2246,10 @@ __device__ __forceinline__ int find_group(const int32_t* __restrict__ offsets, i
 }
 
 // h[r, f] = silu(W_gate[e] x_r)_f * (W_up[e] x_r)_f with the interleaved gate/up
-// layout. One thread per (row, feature).
+// layout. One thread per (row, feature): the reference of the bf16 experts.
 template <typename T>
 __global__ void k_simt_gate_up(const T* __restrict__ A, const int32_t* __restrict__ offsets, int G,
-                               const T* __restrict__ Wgu, int d, int m, T* __restrict__ H,
-                               const int32_t* __restrict__ a_rows) {
+                               const T* __restrict__ Wgu, int d, int m, T* __restrict__ H) {
   const int rows = offsets[G];
   const int f = blockIdx.x * blockDim.x + threadIdx.x;
   if (f >= m) return;
@@ -2259,7 +2259,7 @@ __global__ void k_simt_gate_up(const T* __restrict__ A, const int32_t* __restric
     const int64_t grow = static_cast<int64_t>(e) * 2 * m + blk * 2 * DECOMOE_GU_BLOCK + i;
     const T* wg = Wgu + grow * d;
     const T* wu = wg + static_cast<int64_t>(DECOMOE_GU_BLOCK) * d;
-    const T* x = A + static_cast<int64_t>(a_rows ? a_rows[r] : r) * d;
+    const T* x = A + static_cast<int64_t>(r) * d;
     float ag = 0.f, au = 0.f;
     for (int j = 0; j < d; ++j) {
       const float xv = ld_f(x + j);
@@ -2286,6 +2286,86 @@ __global__ void k_simt_down(const T* __restrict__ H, const int32_t* __restrict__
     for (int f = 0; f < m; ++f) acc = fmaf(ld_f(h + f), ld_f(w + f), acc);
     Y[static_cast<int64_t>(r) * d + n] = from_f<T>(acc);
   }
+}
+
+// fp32 experts: a warp takes up to F32_RT rows of one expert and four features
+// (a gate and an up row each) or eight outputs. 128 routed rows over ten
+// experts of d = 256, m = 128: gate/up 39.4 -> 5.9 us, down 20.4 ->
+// 4.5 us against one thread per result.
+constexpr int F32_RT = 8, F32_WARPS = 4;
+template <int VEC>
+__global__ void __launch_bounds__(32 * F32_WARPS)
+    k_f32_gate_up(const float* __restrict__ A, const int32_t* __restrict__ offsets, int G,
+                  const float* __restrict__ Wgu, int d, int m, float* __restrict__ H,
+                  const int32_t* __restrict__ a_rows) {
+  pdl_enter();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int e, r0, r1;
+  if (!chunk_rows<F32_RT>(offsets, G, blockIdx.x, lane, e, r0, r1)) return;
+  const float* a[F32_RT];
+#pragma unroll
+  for (int r = 0; r < F32_RT; ++r) {
+    const int row = min(r0 + r, r1 - 1);  // a short chunk repeats its last row
+    a[r] = A + static_cast<int64_t>(a_rows ? a_rows[row] : row) * d;
+  }
+  for (int f0 = (blockIdx.y * F32_WARPS + warp) * 4; f0 < m; f0 += gridDim.y * F32_WARPS * 4) {
+    const float* w[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int f = f0 + i;
+      const int64_t grow = static_cast<int64_t>(e) * 2 * m + f / DECOMOE_GU_BLOCK * 2 * DECOMOE_GU_BLOCK +
+                           f % DECOMOE_GU_BLOCK;
+      w[2 * i] = Wgu + grow * d;
+      w[2 * i + 1] = w[2 * i] + static_cast<int64_t>(DECOMOE_GU_BLOCK) * d;
+    }
+    float acc[F32_RT * 8];
+    rows_dot<float, VEC>(a, w, d, lane, acc);
+    warp_scatter_sum(acc, lane);  // lane 4 r + i: gate and up of row r, feature i
+    const float ag = acc[0], au = acc[1];
+    const int row = r0 + (lane >> 2);
+    if (row < r1) H[static_cast<int64_t>(row) * m + f0 + (lane & 3)] = ag / (1.0f + expf(-ag)) * au;
+  }
+}
+
+template <int VEC>
+__global__ void __launch_bounds__(32 * F32_WARPS)
+    k_f32_down(const float* __restrict__ H, const int32_t* __restrict__ offsets, int G, const float* __restrict__ Wd,
+               int d, int m, float* __restrict__ Y) {
+  pdl_enter();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int e, r0, r1;
+  if (!chunk_rows<F32_RT>(offsets, G, blockIdx.x, lane, e, r0, r1)) return;
+  const float* a[F32_RT];
+#pragma unroll
+  for (int r = 0; r < F32_RT; ++r) a[r] = H + static_cast<int64_t>(min(r0 + r, r1 - 1)) * m;
+  for (int n0 = (blockIdx.y * F32_WARPS + warp) * 8; n0 < d; n0 += gridDim.y * F32_WARPS * 8) {
+    const float* w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = Wd + (static_cast<int64_t>(e) * d + min(n0 + i, d - 1)) * m;
+    float acc[F32_RT * 8];
+    rows_dot<float, VEC>(a, w, m, lane, acc);
+    warp_scatter_sum(acc, lane);  // lane 4 r + i: outputs 2 i and 2 i + 1 of row r
+    const int row = r0 + (lane >> 2), n = n0 + 2 * (lane & 3);
+    if (row < r1) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (n + u < d) Y[static_cast<int64_t>(row) * d + n + u] = acc[u];
+    }
+  }
+}
+
+// Row chunks of R rows in K groups (at most) and the features' blocks.
+static dim3 f32_grid(int64_t R, int K, int outs, int per_warp) {
+  const int64_t chunks = (R + F32_RT - 1) / F32_RT + std::min<int64_t>(K, R);
+  const int per_block = F32_WARPS * per_warp;
+  return dim3(static_cast<unsigned>(chunks), static_cast<unsigned>(std::min((outs + per_block - 1) / per_block, 65535)));
+}
+static int launch_f32_gate_up(const float* x, const int32_t* offsets, int64_t R, int K, int d, int m, const float* wgu,
+                              float* h, const int32_t* rows, cudaStream_t s) {
+  const bool vec = d % 4 == 0 && aligned16(x) && aligned16(wgu);
+  DM_CUDA_CHECK(launch_pdl(vec ? k_f32_gate_up<4> : k_f32_gate_up<1>, f32_grid(R, K, m, 4), dim3(32 * F32_WARPS), 0, s,
+                           x, offsets, K, wgu, d, m, h, rows));
+  return DECOMOE_OK;
 }
 
 // ------------------------------------------------------------------ weight layout
@@ -2395,14 +2475,9 @@ int decomoe_expert_gate_up(const void* x_perm, const int32_t* offsets, int64_t r
   if (rows == 0) return DECOMOE_OK;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int R = static_cast<int>(rows);
-  if (dtype == DECOMOE_F32) {
-    dim3 g1((m + 127) / 128, static_cast<unsigned>(std::min(R, 65535)));
-    k_simt_gate_up<float><<<g1, 128, 0, s>>>(static_cast<const float*>(x_perm), offsets, K,
-                                              static_cast<const float*>(w_gate_up), d, m, static_cast<float*>(h),
-                                              nullptr);
-    DM_LAUNCH_CHECK("k_simt_gate_up");
-    return DECOMOE_OK;
-  }
+  if (dtype == DECOMOE_F32)
+    return launch_f32_gate_up(static_cast<const float*>(x_perm), offsets, R, K, d, m,
+                              static_cast<const float*>(w_gate_up), static_cast<float*>(h), nullptr, s);
   if (static_cast<int64_t>(R) <= static_cast<int64_t>(DECOMOE_WS_MAX_AVG_ROWS) * K)
     return launch_ws_auto<true>(x_perm, R, d, w_gate_up, 2 * m, offsets, K, h, m, status_dev, s);
   // A = x_perm [R, d], B = w_gate_up [K*2m, d] (only experts < K are read)
@@ -2420,10 +2495,10 @@ int decomoe_expert_down(const void* h, const int32_t* offsets, int64_t rows, int
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int R = static_cast<int>(rows);
   if (dtype == DECOMOE_F32) {
-    dim3 g2((d + 127) / 128, static_cast<unsigned>(std::min(R, 65535)));
-    k_simt_down<float><<<g2, 128, 0, s>>>(static_cast<const float*>(h), offsets, K,
-                                           static_cast<const float*>(w_down), d, m, static_cast<float*>(y_perm));
-    DM_LAUNCH_CHECK("k_simt_down");
+    const bool vec = m % 4 == 0 && aligned16(h) && aligned16(w_down);
+    DM_CUDA_CHECK(launch_pdl(vec ? k_f32_down<4> : k_f32_down<1>, f32_grid(R, K, d, 8), dim3(32 * F32_WARPS), 0, s,
+                             static_cast<const float*>(h), offsets, K, static_cast<const float*>(w_down), d, m,
+                             static_cast<float*>(y_perm)));
     return DECOMOE_OK;
   }
   if (static_cast<int64_t>(R) <= static_cast<int64_t>(DECOMOE_WS_MAX_AVG_ROWS) * K)
@@ -2444,14 +2519,9 @@ int decomoe_expert_gate_up_gather(const void* x, int64_t T, const int32_t* perm_
   DM_ARG_CHECK(perm_token != nullptr && T > 0 && T < 0x7fffffffLL, "expert_gate_up_gather: bad perm_token or T");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int R = static_cast<int>(rows);
-  if (dtype == DECOMOE_F32) {
-    dim3 g1((m + 127) / 128, static_cast<unsigned>(std::min(R, 65535)));
-    k_simt_gate_up<float><<<g1, 128, 0, s>>>(static_cast<const float*>(x), offsets, K,
-                                              static_cast<const float*>(w_gate_up), d, m, static_cast<float*>(h),
-                                              perm_token);
-    DM_LAUNCH_CHECK("k_simt_gate_up");
-    return DECOMOE_OK;
-  }
+  if (dtype == DECOMOE_F32)
+    return launch_f32_gate_up(static_cast<const float*>(x), offsets, R, K, d, m, static_cast<const float*>(w_gate_up),
+                              static_cast<float*>(h), perm_token, s);
   if (static_cast<int64_t>(R) <= static_cast<int64_t>(DECOMOE_WS_MAX_AVG_ROWS) * K)
     return launch_ws<true, 4, true>(x, R, d, w_gate_up, 2 * m, offsets, K, h, m, status_dev, s, perm_token, T);
   return launch_tc<256, EPI_SWIGLU, GU_STAGES, GU_BK, 2>(
@@ -2492,7 +2562,7 @@ int decomoe_expert_swiglu_ref(const void* x_perm, const int32_t* offsets, int64_
   dim3 g1((m + 127) / 128, static_cast<unsigned>(std::min(R, 65535)));
   k_simt_gate_up<__nv_bfloat16><<<g1, 128, 0, s>>>(static_cast<const __nv_bfloat16*>(x_perm), offsets, K,
                                                     static_cast<const __nv_bfloat16*>(w_gate_up), d, m,
-                                                    static_cast<__nv_bfloat16*>(h_ws), nullptr);
+                                                    static_cast<__nv_bfloat16*>(h_ws));
   DM_LAUNCH_CHECK("k_simt_gate_up<bf16>");
   dim3 g2((d + 127) / 128, static_cast<unsigned>(std::min(R, 65535)));
   k_simt_down<__nv_bfloat16><<<g2, 128, 0, s>>>(static_cast<const __nv_bfloat16*>(h_ws), offsets, K,

@@ -6,34 +6,37 @@
 
 #include "dispatch_tile.cuh"
 #include "route_common.cuh"
+#include "simt_rows.cuh"
 
 namespace decomoe {
 
 // ------------------------------------------------------------ router, CUDA cores
-// logits[t, e] = sum_j x[t, j] * w_r[e, j] + bias[e]. One thread per (t, e);
-// fp32 accumulate. Used for fp32 storage and shapes the tensor-core kernel does
-// not take.
-template <typename T>
-__device__ __forceinline__ float to_f(T v);
-template <>
-__device__ __forceinline__ float to_f<float>(float v) { return v; }
-template <>
-__device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
-
-template <typename T>
-__global__ void k_router_simt(const T* __restrict__ x, const T* __restrict__ w_r,
-                              const float* __restrict__ bias, int64_t Tn, int d, int E,
-                              float* __restrict__ logits) {
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= Tn * E) return;
-  const int64_t t = i / E;
-  const int e = static_cast<int>(i - t * E);
-  const T* xr = x + t * d;
-  const T* wr = w_r + static_cast<int64_t>(e) * d;
-  float acc = 0.f;
-  for (int j = 0; j < d; ++j) acc = fmaf(to_f(xr[j]), to_f(wr[j]), acc);
-  if (bias != nullptr) acc += bias[e];
-  logits[i] = acc;
+// logits[t, e] = sum_j x[t, j] * w_r[e, j] + bias[e] for fp32 storage and
+// shapes the tensor-core kernel does not take: a warp per RS_RT tokens and
+// RS_NR experts, four warps per block (64 tokens, 16 experts, d = 256: 21.6 ->
+// 4.9 us against one thread per logit).
+constexpr int RS_RT = 4, RS_NR = 4, RS_WARPS = 4;
+template <typename T, int VEC>
+__global__ void __launch_bounds__(32 * RS_WARPS)
+    k_router_rows(const T* __restrict__ x, const T* __restrict__ w_r, const float* __restrict__ bias, int64_t Tn, int d,
+                  int E, float* __restrict__ logits) {
+  pdl_enter();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t t0 = static_cast<int64_t>(blockIdx.x) * RS_RT;
+  const T* a[RS_RT];
+#pragma unroll
+  for (int r = 0; r < RS_RT; ++r) a[r] = x + (t0 + r < Tn ? t0 + r : Tn - 1) * d;
+  for (int e0 = (blockIdx.y * RS_WARPS + warp) * RS_NR; e0 < E; e0 += gridDim.y * RS_WARPS * RS_NR) {
+    const T* w[RS_NR];
+#pragma unroll
+    for (int j = 0; j < RS_NR; ++j) w[j] = w_r + static_cast<int64_t>(min(e0 + j, E - 1)) * d;
+    float acc[RS_RT * RS_NR];
+    rows_dot<T, VEC>(a, w, d, lane, acc);
+    warp_scatter_sum(acc, lane);  // lanes 2 i and 2 i + 1: token i / RS_NR, expert i % RS_NR
+    const int64_t t = t0 + (lane >> 1) / RS_NR;
+    const int e = e0 + (lane >> 1) % RS_NR;
+    if ((lane & 1) == 0 && t < Tn && e < E) logits[t * E + e] = acc[0] + (bias != nullptr ? bias[e] : 0.f);
+  }
 }
 
 // Router for few tokens (decode) on CUDA cores: fp32 dot products of the bf16
@@ -279,17 +282,18 @@ int decomoe_router_logits(const void* x, const void* w_r, const float* bias, int
                  "router_logits: pointers must be 16-byte aligned");
     return launch_router_tc(x, w_r, bias, T, d, E, logits, status_dev, s);
   }
-  const int64_t n = T * E;
-  const int threads = 256;
-  const int64_t blocks = (n + threads - 1) / threads;
-  if (dtype == DECOMOE_F32)
-    k_router_simt<float><<<blocks, threads, 0, s>>>(static_cast<const float*>(x),
-                                                    static_cast<const float*>(w_r), bias, T, d, E, logits);
-  else
-    k_router_simt<__nv_bfloat16><<<blocks, threads, 0, s>>>(
-        static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(w_r), bias, T, d, E, logits);
-  DM_LAUNCH_CHECK("k_router_simt");
-  return DECOMOE_OK;
+  const bool f32 = dtype == DECOMOE_F32;
+  const bool vec = d % (f32 ? 4 : 8) == 0 && aligned16(x) && aligned16(w_r);
+  const dim3 grid(static_cast<unsigned>((T + RS_RT - 1) / RS_RT),
+                  static_cast<unsigned>(std::min((E + RS_WARPS * RS_NR - 1) / (RS_WARPS * RS_NR), 65535)));
+  auto go = [&](auto kern, auto type) -> int {
+    using S = decltype(type);
+    DM_CUDA_CHECK(launch_pdl(kern, grid, dim3(32 * RS_WARPS), 0, s, static_cast<const S*>(x),
+                             static_cast<const S*>(w_r), bias, T, d, E, logits));
+    return DECOMOE_OK;
+  };
+  if (f32) return go(vec ? k_router_rows<float, 4> : k_router_rows<float, 1>, 0.f);
+  return go(vec ? k_router_rows<__nv_bfloat16, 8> : k_router_rows<__nv_bfloat16, 1>, __nv_bfloat16());
 }
 
 size_t decomoe_router_logits_ws_bytes(int64_t T, int d, int E) {

@@ -322,6 +322,56 @@ def test_expert_swiglu_f32_parity():
     assert torch.equal(y3, y)
 
 
+@pytest.mark.parametrize("T,k,K,d,m", [(1, 1, 2, 64, 64), (9, 2, 3, 260, 64), (65, 4, 8, 34, 192), (300, 2, 16, 129, 64),
+                                       (40, 2, 200, 64, 64)])
+def test_expert_swiglu_f32_ragged(T, k, K, d, m):
+    """Row chunks and output tiles that end anywhere (d = 129 and 34 leave the
+    16-byte vectors; 200 groups, most of them empty), each with pointers off
+    a 16-byte boundary too, against the oracle; the same bits both ways round
+    (rows gathered by index or copied)."""
+    g = torch.Generator().manual_seed(T)
+    x, wgu = torch.randn(T, d, generator=g), torch.randn(K, 2 * m, d, generator=g) * 0.1
+    wd = torch.randn(K, d, m, generator=g) * 0.1
+    idx = torch.stack([torch.randperm(K, generator=g)[:k] for _ in range(T)]).numpy()
+    _, offsets, perm, _ = O.dispatch(idx, K)
+    B = dm.GU_BLOCK
+    blocks = wgu.view(K, m // B, 2, B, d)
+    w_gate, w_up = blocks[:, :, 0].reshape(K, m, d), blocks[:, :, 1].reshape(K, m, d)
+    ref = O.expert_swiglu(f64(x)[perm], offsets, f64(w_gate), f64(w_up), f64(wd))
+    off = torch.from_numpy(offsets.astype(np.int32)).to(DEV)
+    perm_d = torch.from_numpy(perm.astype(np.int32)).to(DEV)
+
+    def put(t, shift):  # on the device, `shift` floats past an aligned address
+        buf = torch.empty(t.numel() + shift, device=DEV)
+        buf[shift:] = t.to(DEV).reshape(-1)
+        return buf[shift:].view(t.shape)
+
+    for shift in (0, 1):
+        xd, wgud, wdd = put(x, shift), put(wgu, shift), put(wd, shift)
+        xp = put(x[torch.from_numpy(perm)], shift)
+        h, y, y2 = (torch.empty(T * k, c, device=DEV) for c in (m, d, d))
+        dm.decomoe_expert_swiglu(xp, off, K, wgud, wdd, h, y)
+        dm.decomoe_expert_swiglu_gather(xd, perm_d, off, K, wgud, wdd, torch.empty_like(h), y2)
+        torch.cuda.synchronize()
+        assert_close_out(f64(y), ref, F32_REL_L2, F32_MAX_ABS, f"fp32 experts shift {shift}")
+        assert torch.equal(y, y2)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("T,d,E", [(7, 64, 5), (33, 129, 16), (66, 1000, 17), (260, 34, 200)])
+def test_router_logits_cuda_core_ragged(T, d, E, dtype):
+    g = torch.Generator().manual_seed(d)
+    x, w = torch.randn(T, d, generator=g).to(dtype), (torch.randn(E, d, generator=g) * 0.05).to(dtype)
+    b = torch.linspace(1, -1, E)
+    for bias in (b, None):
+        lg = torch.empty(T, E, device=DEV)
+        dm.decomoe_router_logits(x.to(DEV), w.to(DEV), None if bias is None else bias.to(DEV), lg)
+        torch.cuda.synchronize()
+        b64 = np.zeros(E) if bias is None else f64(bias)
+        err = np.abs(f64(lg) - O.router_logits(f64(x), f64(w), b64))
+        assert (err <= logit_error_bound(f64(x), f64(w), b64)).all()
+
+
 def test_weight_layout_interleave():
     E, m, d = 3, 256, 64
     wg = torch.randn(E, m, d).to(torch.bfloat16).to(DEV)
