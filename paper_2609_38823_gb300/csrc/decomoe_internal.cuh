@@ -145,6 +145,10 @@ int route_prefix_src(const float* logits, const RouteSrc& src, int64_t T, int E,
                      int32_t* topk_idx, float* topk_w, double* mass_out, void* ws, size_t ws_bytes,
                      bool defer_finalize, int* mass_blocks, cudaStream_t s, const int32_t* K_dev = nullptr,
                      const RouteDispatch* rd = nullptr, int32_t* zero_ints = nullptr, int n_zero = 0);
+// The deferred activated mass of a routing launch (part: nblocks partials of E)
+// added up into mass, and the prefix it selects (Eq. 12) into K_dev.
+int launch_mass_select(const double* part, int nblocks, int E, double* mass, int k, double p, int32_t* K_dev,
+                       cudaStream_t s);
 // The row gather of decomoe_dispatch: x_perm[r] = x[perm_token[r]] for the
 // offsets[K] routed rows (N = T*k rows at most).
 int launch_gather_rows(const void* x, const int32_t* perm_token, const int32_t* offsets, int K, size_t row_bytes,

@@ -96,9 +96,13 @@ static int route_dispatch_src(const float* logits, const RouteSrc& src, int64_t 
   if (device_k) {
     // mass pass, Eq. 12 on the device, routing over [0, *K_dev) (from the
     // summed logits when the first pass read the router's partials)
-    DM_RET(route_prefix_src(logits, src, T, E, E, E, k, nullptr, nullptr, mass_out, route_ws, rbytes, false, nullptr,
-                            s, nullptr, nullptr, zero_ints, n_zero));
-    DM_RET(decomoe_select_prefix_device(mass_out, E, k, p, K_dev, stream));
+    DM_RET(route_prefix_src(logits, src, T, E, E, E, k, nullptr, nullptr, mass_out, route_ws, rbytes, true,
+                            &mass_blocks, s, nullptr, nullptr, zero_ints, n_zero));
+    if (mass_blocks > 0)  // the partial masses are added up by the selecting launch
+      DM_RET(launch_mass_select(static_cast<const double*>(route_ws), mass_blocks, E, mass_out, k, p, K_dev, s));
+    else
+      DM_RET(decomoe_select_prefix_device(mass_out, E, k, p, K_dev, stream));
+    mass_blocks = 0;
     DM_RET(route_prefix_src(src.logits_out != nullptr ? src.logits_out : logits, RouteSrc{}, T, E, E, E, k, topk_idx,
                             topk_w, nullptr, nullptr, 0, false, nullptr, s, K_dev, one_block ? &rd : nullptr));
   } else {

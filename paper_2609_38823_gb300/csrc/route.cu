@@ -234,11 +234,151 @@ __global__ void __launch_bounds__(256)
   mass_finalize_block(part, nblocks, E, static_cast<int>(blockIdx.x), mass);
 }
 
-// Eq. 12 on the device, one thread (bit-identical to decomoe_select_prefix).
-__global__ void k_select_prefix(const double* __restrict__ mass, int E, int k, double p, int32_t* __restrict__ K_dev) {
+// Eq. 12 by one block of DECOMOE_MAX_E threads on the mass in shared memory,
+// thread e on the sum of the first e + 1 masses: the K of
+// decomoe_select_prefix bit for bit. fp64 is what this costs (a dependent add
+// takes tens of cycles here: one thread adding and dividing took 13.4 us for
+// 128 experts), so the sums are formed as integers where that is exact: the
+// masses are sums of fp32 weights, and when all of them are multiples of
+// 2^-sh with a total below 2^(53 - sh) every sequential fp64 sum is exact, in
+// whatever order it is formed. Otherwise one thread adds them up in order. A
+// ratio is divided out only where the product p * total leaves it open.
+// s_cum: E doubles of scratch.
+__device__ __forceinline__ int select_prefix_block(const double* s_mass, double* s_cum, int E, int k, double p) {
+  constexpr int NW = DECOMOE_MAX_E / 32;
+  __shared__ float s_tf[NW];
+  __shared__ uint64_t s_wsum[NW];
+  __shared__ int s_first;
+  const int e = threadIdx.x, warp = e >> 5, lane = e & 31;
+  const uint64_t bits = e < E ? static_cast<uint64_t>(__double_as_longlong(s_mass[e])) : 0ull;
+  const int ex = static_cast<int>(bits >> 52);  // sign and exponent
+  // the total, to fix the scale (truncated to fp32 by hand; other exponents
+  // than fp32's are left to the sequential sum)
+  bool odd = bits != 0 && (ex < 1023 - 126 || ex > 1023 + 100);
+  float tf = (odd || bits == 0) ? 0.f
+                                : __uint_as_float((static_cast<uint32_t>(ex - 1023 + 127) << 23) |
+                                                  static_cast<uint32_t>((bits >> 29) & 0x7FFFFFu));
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) tf += __shfl_xor_sync(0xffffffffu, tf, off);
+  if (lane == 0) s_tf[warp] = tf;
+  if (e == 0) s_first = E;  // none reaches p (or p >= 1): the whole pool
+  __syncthreads();
+  tf = 0.f;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) tf += s_tf[w];
+  const int te = static_cast<int>(__float_as_uint(tf) >> 23) - 127;  // total < 2^(te + 2)
+  const int shift = ex - 1075 + (51 - te);                           // scale sh = 51 - te
+  uint64_t v = 0;
+  if (!odd && bits != 0) {
+    const uint64_t mant = (bits & ((1ull << 52) - 1)) | (1ull << 52);
+    if (shift >= 0) {
+      v = mant << shift;  // below 2^53, as the total is
+    } else if (shift > -53) {
+      v = mant >> -shift;
+      odd = (v << -shift) != mant;
+    } else {
+      odd = true;
+    }
+  }
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const uint64_t u = __shfl_up_sync(0xffffffffu, v, off);
+    if (lane >= off) v += u;
+  }
+  if (lane == 31) s_wsum[warp] = v;
+  double cum, tot;
+  if (!__syncthreads_or(odd)) {
+    uint64_t all = 0, before = 0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+      if (w == warp) before = all;
+      all += s_wsum[w];
+    }
+    cum = __ull2double_rn(v + before);
+    tot = __ull2double_rn(all);
+  } else {
+    if (e == 0) {
+      double acc = 0.0;
+      for (int i = 0; i < E; ++i) {
+        acc = __dadd_rn(acc, s_mass[i]);
+        s_cum[i] = acc;
+      }
+    }
+    __syncthreads();
+    cum = e < E ? s_cum[e] : 0.0;
+    tot = s_cum[E - 1];
+  }
+  if (p < 1.0 && e < E) {
+    // |p * tot rounded - p * tot| <= 2^-53 of it, and the quotient is rounded
+    // by as little: outside 2^-50 of p * tot the comparison is decided
+    const double t = p * tot;
+    bool reached;
+    if (p > 1e-280 && t < 1e280 && tot > 1e-280 && cum > fma(t, 0x1p-50, t))
+      reached = true;
+    else if (p > 1e-280 && t < 1e280 && tot > 1e-280 && cum < fma(t, -0x1p-50, t))
+      reached = false;
+    else
+      reached = __ddiv_rn(cum, tot) >= p;
+    if (reached) atomicMin(&s_first, e + 1);
+  }
+  __syncthreads();
+  return tot > 0.0 && s_first > k ? s_first : k;
+}
+
+__global__ void __launch_bounds__(DECOMOE_MAX_E)
+    k_select_prefix(const double* __restrict__ mass, int E, int k, double p, int32_t* __restrict__ K_dev) {
   pdl_enter();
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  *K_dev = select_prefix_seq(mass, E, k, p);
+  __shared__ double s_mass[DECOMOE_MAX_E], s_cum[DECOMOE_MAX_E];
+  if (E > DECOMOE_MAX_E) {  // larger than any pool routed here: one thread
+    if (threadIdx.x == 0) *K_dev = select_prefix_seq(mass, E, k, p);
+    return;
+  }
+  for (int e = threadIdx.x; e < E; e += blockDim.x) s_mass[e] = mass[e];
+  __syncthreads();
+  const int K = select_prefix_block(s_mass, s_cum, E, k, p);
+  if (threadIdx.x == 0) *K_dev = K;
+}
+
+// k_mass_finalize and k_select_prefix in one block, for at most MS_MAX_BLOCKS
+// routing blocks: a thread per expert holds the partials that threads 0, 1,
+// ... of mass_finalize_block would, and adds them in the same tree (its other
+// leaves are zero, which change nothing), so the bits are the same. fp64 adds
+// are the cost (an SM issues about two a cycle, so a warp's takes 16 cycles
+// whatever its lanes do): a warp per expert with shuffles took 33 us at 17
+// blocks of 128 experts, and above 64 blocks E blocks of their own are faster.
+constexpr int MS_MAX_BLOCKS = 64;
+__global__ void __launch_bounds__(DECOMOE_MAX_E)
+    k_mass_select(const double* __restrict__ part, int nblocks, int E, double* __restrict__ mass, int k, double p,
+                  int32_t* __restrict__ K_dev) {
+  pdl_enter();
+  __shared__ double s_mass[DECOMOE_MAX_E], s_cum[DECOMOE_MAX_E];
+  const int e = threadIdx.x;
+  if (e < E) {
+    double a[MS_MAX_BLOCKS];
+#pragma unroll
+    for (int b = 0; b < MS_MAX_BLOCKS; ++b)
+      if (b < nblocks) a[b] = part[static_cast<int64_t>(b) * E + e];
+#pragma unroll
+    for (int w = MS_MAX_BLOCKS / 2; w > 0; w >>= 1)
+#pragma unroll
+      for (int i = 0; i < w; ++i)
+        if (i + w < nblocks) a[i] += a[i + w];
+    mass[e] = a[0];
+    s_mass[e] = a[0];
+  }
+  __syncthreads();
+  const int K = select_prefix_block(s_mass, s_cum, E, k, p);
+  if (threadIdx.x == 0) *K_dev = K;
+}
+
+int launch_mass_select(const double* part, int nblocks, int E, double* mass, int k, double p, int32_t* K_dev,
+                       cudaStream_t s) {
+  if (nblocks > MS_MAX_BLOCKS) {
+    DM_CUDA_CHECK(launch_pdl(k_mass_finalize, dim3(E), dim3(256), 0, s, part, nblocks, E, mass));
+    return decomoe_select_prefix_device(mass, E, k, p, K_dev, reinterpret_cast<decomoe_stream_t>(s));
+  }
+  DM_CUDA_CHECK(launch_pdl(k_mass_select, dim3(1), dim3(DECOMOE_MAX_E), 0, s, part, nblocks, E, mass, k, p, K_dev));
+  return DECOMOE_OK;
 }
 
 // Activated mass (Eq. 11) over n tokens whose logit rows skip a block:
@@ -403,7 +543,7 @@ int decomoe_select_prefix_device(const double* mass, int E, int k, double p, int
   DM_ARG_CHECK(mass && K_dev, "select_prefix_device: null pointer");
   DM_ARG_CHECK(E >= 1 && k >= 1 && k <= E, "select_prefix_device: need 1 <= k <= E");
   DM_ARG_CHECK(p > 0.0 && p <= 1.0, "select_prefix_device: p must lie in (0, 1]");
-  DM_CUDA_CHECK(launch_pdl(k_select_prefix, dim3(1), dim3(32), 0, reinterpret_cast<cudaStream_t>(stream), mass, E, k,
+  DM_CUDA_CHECK(launch_pdl(k_select_prefix, dim3(1), dim3(DECOMOE_MAX_E), 0, reinterpret_cast<cudaStream_t>(stream), mass, E, k,
                            p, K_dev));
   return DECOMOE_OK;
 }

@@ -322,6 +322,45 @@ def test_expert_swiglu_f32_parity():
     assert torch.equal(y3, y)
 
 
+@pytest.mark.parametrize("E,k,p", [(1, 1, 0.5), (16, 2, 1.0), (100, 8, 0.37), (128, 8, 0.9), (256, 1, 0.999),
+                                   (300, 3, 0.8)])
+def test_select_prefix_device_equals_host(E, k, p):
+    """The block form (up to 256 experts) and the one-thread form beyond, on
+    masses with zeros, ties and none at all, against the host (which refuses
+    masses that are not finite)."""
+    g = torch.Generator().manual_seed(E)
+    mass = torch.rand(E, generator=g, dtype=torch.float64) ** 6
+    zeros = mass.clone()
+    zeros[::3] = 0.0
+    for m in (mass, zeros, torch.full((E,), 0.1, dtype=torch.float64), torch.zeros(E, dtype=torch.float64)):
+        K = torch.zeros(1, dtype=torch.int32, device=DEV)
+        dm.decomoe_select_prefix_device(m.to(DEV), k, p, K)
+        assert int(K.item()) == dm.decomoe_select_prefix(m.numpy(), k, p)
+
+
+@pytest.mark.parametrize("T,E,k", [(9, 128, 8), (17, 16, 2), (256, 256, 4), (257, 100, 8), (512, 128, 8), (513, 128, 8),
+                                   (2049, 128, 8)])
+def test_device_prefix_in_one_call_equals_separate_calls(T, E, k):
+    """Up to 512 tokens one launch adds the routing blocks' masses and
+    selects; its mass has the bits of the separate finalize."""
+    lg = W.make_logits(T, E, bias=_zipf_bias(E), seed=T).to(DEV)
+    i32 = dict(dtype=torch.int32, device=DEV)
+    mass, mass2 = (torch.empty(E, dtype=torch.float64, device=DEV) for _ in range(2))
+    idx, w = torch.empty(T, k, **i32), torch.empty(T, k, device=DEV)
+    Kd = torch.zeros(1, **i32)
+    ws = dm.workspace(dm.decomoe_route_dispatch_workspace_bytes(T, k, E), DEV)
+    dm.decomoe_route_dispatch(lg, -1, k, idx, w, None, torch.empty(E, **i32), torch.empty(E + 1, **i32),
+                              torch.empty(T * k, **i32), torch.empty(T * k, **i32), None, ws, p=0.83, mass_out=mass,
+                              K_dev=Kd)
+    dm.decomoe_route_prefix(lg, E, k, mass_out=mass2, ws=dm.workspace(dm.decomoe_route_workspace_bytes(T, E), DEV))
+    K = dm.decomoe_select_prefix(mass2.cpu().numpy(), k, 0.83)
+    idx2, w2 = torch.empty_like(idx), torch.empty_like(w)
+    dm.decomoe_route_prefix(lg, K, k, topk_idx=idx2, topk_w=w2)
+    torch.cuda.synchronize()
+    assert torch.equal(mass, mass2) and int(Kd.item()) == K
+    assert torch.equal(idx, idx2) and torch.equal(w, w2)
+
+
 @pytest.mark.parametrize("T,k,K,d,m", [(1, 1, 2, 64, 64), (9, 2, 3, 260, 64), (65, 4, 8, 34, 192), (300, 2, 16, 129, 64),
                                        (40, 2, 200, 64, 64)])
 def test_expert_swiglu_f32_ragged(T, k, K, d, m):
