@@ -186,6 +186,36 @@ def test_dispatch_parity(T, k, K, d, dt, pattern):
     assert torch.equal(xp2, xp)
 
 
+@pytest.mark.parametrize("T,k,K", [(1025, 1, 3), (205, 5, 200), (4096, 1, 64), (4097, 1, 256), (513, 8, 128),
+                                   (16384, 1, 17), (16385, 1, 17)])
+def test_dispatch_cluster_sizes(T, k, K):
+    """One launch of a cluster up to 16384 pairs (two, four and eight 32-pair
+    rounds per warp, the last warps partly or wholly empty), the two-launch form
+    above; ids out of range, -2 among them, are dropped and reported."""
+    idx = np.random.default_rng(T).integers(0, K, size=(T, k)).astype(np.int32)
+    bad = idx.copy()
+    bad[T // 2, 0], bad[T - 1, k - 1], bad[3, 0] = -2, K, -1
+    for ids in (idx, bad):
+        i32 = dict(dtype=torch.int32, device=DEV)
+        counts, offsets = torch.empty(K, **i32), torch.empty(K + 1, **i32)
+        perm, inv = torch.full((T * k,), -7, **i32), torch.full((T * k,), -7, **i32)
+        status = torch.zeros(1, **i32)
+        dm.decomoe_dispatch(torch.from_numpy(ids).to(DEV), K, None, counts, offsets, perm, inv, None,
+                            dm.workspace(dm.decomoe_dispatch_workspace_bytes(T, k, K), DEV), status)
+        torch.cuda.synchronize()
+        assert dm.decomoe_read_status(status) == (dm.DECOMOE_ERR_BAD_INPUT if ids is bad else 0)
+        flat = ids.reshape(-1)
+        ok = np.flatnonzero((flat >= 0) & (flat < K))
+        order = ok[np.argsort(flat[ok], kind="stable")]
+        want = np.full(T * k, -1)
+        want[order] = np.arange(order.size)
+        assert np.array_equal(inv.cpu().numpy(), want)
+        assert np.array_equal(perm.cpu().numpy()[:order.size], order // k)
+        c = np.bincount(flat[ok], minlength=K)
+        assert np.array_equal(counts.cpu().numpy(), c)
+        assert np.array_equal(offsets.cpu().numpy(), np.concatenate([[0], np.cumsum(c)]))
+
+
 def test_dispatch_flags_bad_expert_id():
     T, k, K = 50, 2, 8
     idx = np.random.default_rng(0).integers(0, K, size=(T, k))
