@@ -13,6 +13,7 @@ raises.
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 from typing import Optional
 
@@ -131,16 +132,22 @@ def _check(name, code):
         raise DecomoeError(name, code, msg.decode() if msg else "")
 
 
+# Marshalling costs a call more host time than its launches do where it makes
+# objects on the way (a Stream, c_void_p boxes, tensor views): pointers and the
+# stream go over as plain integers.
 def _ptr(t: Optional[torch.Tensor]):
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream=None):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _dt(t: torch.Tensor) -> int:
@@ -153,11 +160,8 @@ def _dt(t: torch.Tensor) -> int:
 
 def _need_cuda(*ts):
     for t in ts:
-        if t is not None:
-            if not t.is_cuda:
-                raise ValueError("device tensors expected")
-            if not t.is_contiguous():
-                raise ValueError("contiguous tensors expected")
+        if t is not None and not (t.is_cuda and t.is_contiguous()):
+            raise ValueError("contiguous tensors expected" if t.is_cuda else "device tensors expected")
 
 
 # ----------------------------------------------------------------- host-only calls
@@ -537,7 +541,9 @@ def decomoe_combine_drop_visual_block(y_perm, inv_slot, topk_w, out, text_out, v
 def _drop_geometry(src, dst, nv):
     if src.dim() >= 3:
         nbatch, rows = src.shape[0], src.shape[1]
-        row_bytes = src[0, 0].numel() * src.element_size()
+        if nbatch == 0 or rows == 0:
+            raise IndexError("no rows to take the row size from")
+        row_bytes = math.prod(src.shape[2:]) * src.element_size()
         sstride = src.stride(0) * src.element_size()
         dstride = dst.stride(0) * dst.element_size()
     else:
