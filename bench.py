@@ -298,9 +298,9 @@ def algo_bytes_ffn(wl, R, D, T=None):
     row gather in the launch the T token rows x, each read once), h written
     once (an output of the call) and y written. The read of h back by the
     down tiles is not counted: in the one-launch form it follows the write
-    within microseconds and is served from L2. With the row gather the launch
-    also writes the gathered rows to its x_perm scratch: that is not
-    algorithmic traffic (the DRAM counters show it)."""
+    within microseconds and is served from L2. The separate call also writes the
+    gathered rows to its x_perm argument: that is not algorithmic traffic (the
+    DRAM counters show it)."""
     act = (T if T is not None else R) * wl.d * 2
     return D * 3 * wl.m * wl.d * 2 + act + R * wl.m * 2 + R * wl.d * 2
 
@@ -418,8 +418,8 @@ def ours(args, ws, rank, local):
     else:
         roof = {"bound": "hbm", "achieved": round(ffn_gbs, 1), "peak": pk["hbm_gbs"], "unit": "GB/s",
                 "frac": round(ffn_gbs / pk["hbm_gbs"], 4), "traffic": traffic}
-    roof.update({"kernel": "k_ffn_tc as the layer launches it (row gather, gate/up + SwiGLU, down in one "
-                           "persistent launch)",
+    roof.update({"kernel": "k_ffn_pair as the layer launches it (rows read by index, gate/up + SwiGLU, down in "
+                           "one persistent launch), plus the grouped copy of the rows that the layer leaves out",
                  "peak_source": f"{pk['source']} burst", "ms_per_launch": round(ffn_ms, 4),
                  "flops_per_launch": ffn_flops, "algo_bytes_per_launch": ffn_bytes,
                  "tensor_frac": round(ffn_tflops / pk["bf16_tflops"], 4),
@@ -1053,22 +1053,17 @@ def only_decode(args, local):
 
 
 def _kernel_hash():
-    """Hash of the one-launch expert FFN's own source: the tcgen05 GEMM and
-    fused prefill FFN sections of expert_gemm.cu and the device-side helpers
-    they use, so edits elsewhere leave the recorded DRAM traffic valid."""
+    """Hash of the one-launch expert FFN's own source (ffn_pair.cuh) and the
+    device-side helpers it uses, so edits elsewhere leave the recorded DRAM
+    traffic valid."""
     import hashlib
 
     csrc = os.path.join(ROOT, "paper_2609_38823_gb300", "csrc")
-    g = open(os.path.join(csrc, "expert_gemm.cu")).read()
-    a = g.index("// ------------------------------------------------------------------ tcgen05 GEMM")
-    b = g.index("// ------------------------------------------------------------------ weights-stationary")
-    c = g.index("// ------------------------------------------------------------------ fused prefill FFN")
-    e = g.index("// ------------------------------------------------------------------ CUDA-core paths")
+    g = open(os.path.join(csrc, "ffn_pair.cuh")).read()
     hdr = open(os.path.join(csrc, "decomoe_internal.cuh")).read()
     hdr = hdr[hdr.index("// ---------------------------------------------------------------- device side"):]
     h = hashlib.sha256()
-    h.update(g[a:b].encode())
-    h.update(g[c:e].encode())
+    h.update(g.encode())
     h.update(hdr.encode())
     return h.hexdigest()[:16]
 

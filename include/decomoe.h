@@ -285,11 +285,8 @@ DECOMOE_API int decomoe_weight_layout(const void* w_gate, const void* w_up, void
  * d % 256 == 0 and 16-byte aligned pointers (DECOMOE_ERR_INVALID_ARG
  * otherwise, before any launch).
  * status_dev: optional device int32 collecting bounded-wait timeouts.
- * sched_dev: optional device int32 (4 bytes, caller-owned). Given, the
- * tensor-core kernels hand tiles out dynamically from this counter (the call
- * zeroes it first) instead of a fixed round robin, which balances the mix of
- * weight-streaming and weight-reusing tiles. Launches that may overlap on the
- * GPU need distinct counters. NULL keeps the static order.
+ * sched_dev: optional device int32 (4 bytes, caller-owned); accepted and not
+ * used (the tiles are handed out in a fixed order).
  * ------------------------------------------------------------------------ */
 DECOMOE_API int decomoe_expert_swiglu(const void* x_perm, const int32_t* offsets, int64_t rows, int K, int d,
                           int m, int dtype, const void* w_gate_up, const void* w_down, void* h_ws,
@@ -298,7 +295,7 @@ DECOMOE_API int decomoe_expert_swiglu(const void* x_perm, const int32_t* offsets
 /* decomoe_expert_swiglu with both GEMMs in one persistent launch where that
  * is faster (bf16, 16 to 32768 rows): the down tiles of an expert (decode
  * sizes) or of a 128-row tile (larger) start as soon as the gate/up tiles
- * they read have stored h, published through per-expert or per-tile counters
+ * they read have stored h, published through per-expert or per-row-tile counters
  * with release/acquire ordering. ready: decomoe_expert_swiglu_ready_ints(rows,
  * K) int32, all zero at the call (decomoe_moe_layer clears its own); the call
  * leaves them non-zero. Outside that range the call runs the two launches of
@@ -311,16 +308,16 @@ DECOMOE_API int decomoe_expert_swiglu_fused(const void* x_perm, const int32_t* o
                                             void* y_perm, int32_t* ready, int32_t* status_dev,
                                             decomoe_stream_t stream);
 
-/* The same one launch as decomoe_moe_layer runs it from 8192 routed rows: the
- * dispatch's row gather inside the expert launch (Algorithm 2, dispatch and
- * expert evaluation). x: [T, d] token rows; perm_token: [rows] from
- * decomoe_dispatch (called without x_perm); x_perm: [rows, d] scratch the
- * launch fills with x[perm_token[r]] on its way to the tiles (caller-owned,
- * 16-byte aligned). Other arguments as decomoe_expert_swiglu_fused; ready
- * needs decomoe_expert_swiglu_ready_ints(rows, K) zeroed int32. Only for
- * sizes the one-launch tokens-as-M form takes (bf16, 8*K < rows <= 32768):
- * DECOMOE_ERR_INVALID_ARG otherwise, nothing launched. Outputs equal those of
- * decomoe_dispatch with x_perm followed by decomoe_expert_swiglu, bit for bit. */
+/* The same one launch reading its rows from the token-ordered x by index, as
+ * decomoe_moe_layer runs it (Algorithm 2, dispatch and expert evaluation). x:
+ * [T, d] token rows; perm_token: [rows] from decomoe_dispatch (called without
+ * x_perm); x_perm: [rows, d], filled with x[perm_token[r]] on the way
+ * (caller-owned, 16-byte aligned; the layer leaves that copy out). Other
+ * arguments as decomoe_expert_swiglu_fused; ready needs
+ * decomoe_expert_swiglu_ready_ints(rows, K) zeroed int32. Only for 8*K < rows
+ * <= 32768 and bf16: DECOMOE_ERR_INVALID_ARG otherwise, nothing launched.
+ * Outputs equal those of decomoe_dispatch with x_perm followed by
+ * decomoe_expert_swiglu, bit for bit. */
 DECOMOE_API int decomoe_expert_swiglu_fused_gather(const void* x, int64_t T, const int32_t* perm_token,
                                                    const int32_t* offsets, int64_t rows, int K, int d, int m,
                                                    int dtype, const void* w_gate_up, const void* w_down,
@@ -338,13 +335,11 @@ DECOMOE_API int decomoe_expert_down(const void* h, const int32_t* offsets, int64
                                     int32_t* sched_dev, decomoe_stream_t stream);
 
 /* Gather forms: the expert rows are read straight from the token-ordered
- * hidden state, row r of the grouped order being x[perm_token[r], :] (TMA
- * tile::gather4 on the tensor cores), so dispatch need not materialise x_perm
- * (saves T*k*d elements of memory). Same results bit for bit as the x_perm
- * forms; slower at prefill sizes, where the four-row gathers, not the tensor
- * cores, bound the gate/up GEMM. x: [T, d] dtype; perm_token: [rows] int32
- * from decomoe_dispatch; other arguments and rules as decomoe_expert_gate_up /
- * decomoe_expert_swiglu. */
+ * hidden state, row r of the grouped order being x[perm_token[r], :], so
+ * dispatch need not materialise x_perm (saves T*k*d elements of memory and the
+ * copy). Same results bit for bit as the x_perm forms. x: [T, d] dtype;
+ * perm_token: [rows] int32 from decomoe_dispatch; other arguments and rules as
+ * decomoe_expert_gate_up / decomoe_expert_swiglu. */
 DECOMOE_API int decomoe_expert_gate_up_gather(const void* x, int64_t T, const int32_t* perm_token,
                                               const int32_t* offsets, int64_t rows, int K, int d, int m,
                                               int dtype, const void* w_gate_up, void* h, int32_t* status_dev,
@@ -523,9 +518,9 @@ DECOMOE_API int decomoe_moe_layer_exit(const void* x, const void* w_r, const flo
 /* Offsets (bytes) of the intermediates inside the decomoe_moe_layer workspace,
  * for inspection: logits, topk_idx, topk_w, mass, counts, offsets, perm_token,
  * inv_slot, x_perm, h, y_perm, device K (12 entries written to offs_host).
- * The layer's scratch rows are dropped from L2 after their last read (see
- * decomoe_set_discard_scratch): turn that off before a call whose y_perm is
- * to be inspected. */
+ * The layer's scratch rows are dropped from L2 after their last read, and
+ * above 8*K routed rows x_perm is not made (see decomoe_set_discard_scratch):
+ * turn that off before a call whose x_perm or y_perm is to be inspected. */
 DECOMOE_API int decomoe_moe_layer_workspace_layout(int64_t T, int d, int E, int k, int m, int dtype,
                                        size_t* offs_host);
 
@@ -590,8 +585,10 @@ DECOMOE_API int decomoe_selftest_wait(int32_t* status_dev, int64_t limit_ns, dec
  * decomoe_moe_layer_exit drop the L2 lines of their workspace's y_perm rows
  * once the combine has read them (discard.global.L2): the rows are not
  * written back to HBM, and the next layer's writes find clean lines to
- * evict. Those workspace rows are undefined after the call. on == 0 keeps
- * them (for inspection). Process-wide; applies to later calls.
+ * evict; and where the experts read x by index (more than 8*K routed rows) the
+ * grouped copy x_perm is not written. Those workspace rows are undefined after
+ * the call. on == 0 makes and keeps them (for inspection). Process-wide;
+ * applies to later calls.
  * ------------------------------------------------------------------------ */
 DECOMOE_API int decomoe_set_discard_scratch(int on);
 

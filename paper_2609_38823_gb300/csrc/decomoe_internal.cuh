@@ -181,15 +181,15 @@ int moe_layer_impl(const void* x, const void* w_r, const float* bias, const void
 // Both expert GEMMs in one launch (bf16): ready holds
 // expert_ffn_sync_ints(rows, K) int32, zero at launch. Sets *launched = false
 // (and launches nothing) where the two-launch form is kept. With gather_x and
-// perm (tokens-as-M form only) the launch also fills x_perm[r] =
-// gather_x[perm[r]] itself.
-enum { FFN_FUSED_NONE = 0, FFN_FUSED_WS = 1, FFN_FUSED_TC = 2 };
-int expert_ffn_fused_kind(int64_t rows, int K, int m, int dtype);
+// perm (pair form only) the gate/up rows are gather_x[perm[r]] and x_perm is
+// not read; copy_rows: it receives those rows.
+enum { FFN_FUSED_NONE = 0, FFN_FUSED_WS = 1, FFN_FUSED_PAIR = 2 };
+int expert_ffn_fused_kind(int64_t rows, int K, int dtype);
 size_t expert_ffn_sync_ints(int64_t rows, int E);
 int launch_expert_ffn_fused(const void* x_perm, const int32_t* offsets, int64_t rows, int K, int d, int m, int dtype,
                             const void* w_gate_up, const void* w_down, void* h, void* y_perm, int32_t* ready,
                             int32_t* status, cudaStream_t s, bool* launched, const void* gather_x = nullptr,
-                            const int32_t* perm = nullptr);
+                            const int32_t* perm = nullptr, bool copy_rows = false);
 // One launch for a whole decode-size layer (router, routing, dispatch,
 // experts, combine, and with text_out the visual-block removal of the
 // output; fixed or device-selected prefix). sync: decode_layer_sync_ints(T, d, E) int32 of the caller's

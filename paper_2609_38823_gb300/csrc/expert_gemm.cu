@@ -20,6 +20,7 @@
 // bf16, few rows per expert (decode): the weights-stationary tcgen05 kernel
 // k_moe_ws (expert weights as M, the expert's tokens as N).
 // f32: CUDA-core kernels (exact fp32 products, fp32 accumulation).
+#include <atomic>
 #include <mutex>
 
 #include <cudaTypedefs.h>
@@ -175,6 +176,10 @@ __device__ __forceinline__ void tile_coords(int tile, int NT, const int* s_mt, i
   grp = lo;
   mt = mtg - s_mt[lo];
 }
+
+}  // namespace decomoe
+#include "ffn_pair.cuh"
+namespace decomoe {
 
 // EW epilogue warps (4 or 8): with 8, two warps share each 32-lane TMEM
 // quarter and split its column chunks, so the epilogue's latency is hidden.
@@ -1547,507 +1552,77 @@ static int launch_ffn_ws(const void* x_perm, int rows, int d, int m, const void*
                                                          status, s);
 }
 
-// ------------------------------------------------------------------ fused prefill FFN
-// Gate/up and down of the tokens-as-M path in one persistent launch, with
-// k_gemm_tc's tiles (128 rows x 256, 4-stage ring, two TMEM accumulators,
-// 8 epilogue warps). Work items: every gate/up tile (tile_coords order),
-// then every down tile (same order); static round robin. A down tile of
-// M-tile j reads the h rows that the 2m/256 gate/up tiles of j store: those
-// bump ready[j] after their stores (release); the down tile issues its
-// weight k-blocks first, polls ready[j] (acquire, bounded), then requests the
-// h rows. The early CTAs of the down phase start while the last gate/up
-// tiles still run, instead of after a launch boundary. Deadlock-free as
-// k_ffn_ws (gate/up items never wait; one CTA per SM, grid <= SMs). ready[]
-// (one int per M-tile) is zero at launch.
-//
-// With x set, the launch also performs the dispatch's row gather: each CTA's
-// epilogue warps copy, for every gate/up item of the CTA in work order, one
-// 1/NT1 share of that item's M-tile rows x_perm[r] = x[perm[r]] and publish
-// it (stores, proxy fence, barrier, release add on gathered[M-tile]); they
-// copy shares while the accumulator they need next is still being computed. A gate/up item's A rows are requested once all NT1
-// shares of its M-tile are in (acquire, bounded; its weight k-blocks go out
-// first), as a down item waits for h. The gathers wait on nothing, so this
-// adds no cycle; the first wave's rows are in after one share per CTA
-// instead of after a separate gather launch.
-// Non-blocking: has the phase with this parity completed?
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
+// ------------------------------------------------------------------ experts on SM pairs
+// Clusters of two that the device keeps resident at once (per device ordinal):
+// the down tiles wait for gate/up tiles of other clusters.
+static std::atomic<int> g_pair_clusters[64];
+static int pair_clusters() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  int v = g_pair_clusters[dev].load();
+  if (v != 0) return v > 0 ? v : 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2);
+  cfg.blockDim = dim3(PF_THREADS);
+  cfg.dynamicSmemBytes = PF_SMEM;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaFuncSetAttribute(k_ffn_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(PF_SMEM)) !=
+          cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&v, k_ffn_pair, &cfg) != cudaSuccess)
+    v = 0;
+  cudaGetLastError();  // a refused query leaves no error behind
+  g_pair_clusters[dev].store(v > 0 ? v : -1);
+  return v;
 }
 
-struct TcFfnArgs {
-  const int32_t* offsets;  // [G + 1]
-  int G;
-  int rows;
-  int d, m;
-  void* h;  // [rows, m] bf16
-  void* y;  // [rows, d] bf16
-  int32_t* ready;
-  int32_t* status;
-  uint64_t limit_ns;
-  const uint4* x;      // gather source [tokens, d / 8] (16-byte vectors), or null: x_perm is filled
-  const int32_t* perm;  // [rows] token of each dispatched row
-  uint4* x_perm;        // [rows, d / 8], written by the gather
-  int32_t* gathered;    // per M-tile: shares copied (zero at launch)
-};
-
-constexpr int FFN_BN = 256, FFN_BK = 64, FFN_STAGES = 4, FFN_EW = 8;
-using FfnCfg = TcCfg<FFN_BN, FFN_STAGES, FFN_BK, 1, 1>;
-
-__global__ void __launch_bounds__(64 + 32 * FFN_EW, 1)
-    k_ffn_tc(const __grid_constant__ CUtensorMap tma_a1, const __grid_constant__ CUtensorMap tma_b1,
-             const __grid_constant__ CUtensorMap tma_a2, const __grid_constant__ CUtensorMap tma_b2,
-             const TcFfnArgs g) {
-  using C = FfnCfg;
-  constexpr int BN = FFN_BN, STAGES = FFN_STAGES, EW = FFN_EW;
-  __shared__ int s_gperm[C::BM + 1];  // token rows of the share being gathered; [BM]: a broadcast flag
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t raw = smem_u32(smem_raw);
-  const uint32_t pad = (1024u - (raw & 1023u)) & 1023u;
-  uint8_t* smem = smem_raw + pad;
-  const uint32_t sA = raw + pad;
-  const uint32_t sB = sA + STAGES * C::A_BYTES;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * C::STAGE_BYTES);
-  int* s_off = reinterpret_cast<int*>(bars + C::NBARS);
-  int* s_mt = s_off + (C::MAXG + 1);
-  volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(s_mt + (C::MAXG + 1));
-  volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t bar0 = smem_u32(bars);
-#define FULL_BAR(s) (bar0 + 8u * (s))
-#define EMPTY_BAR(s) (bar0 + 8u * (STAGES + (s)))
-#define TFULL_BAR(a) (bar0 + 8u * (2 * STAGES + (a)))
-#define TEMPTY_BAR(a) (bar0 + 8u * (2 * STAGES + 2 + (a)))
-#define DRAIN_BAR (bar0 + 8u * (2 * STAGES + 4))
-
-  const int G = g.G;
-  if (threadIdx.x == 0) {
-    *s_abort = 0;
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(FULL_BAR(s), 1);
-      mbar_init(EMPTY_BAR(s), 1);
-    }
-    for (int a = 0; a < 2; ++a) {
-      mbar_init(TFULL_BAR(a), 1);
-      mbar_init(TEMPTY_BAR(a), 32 * EW);
-    }
-    mbar_init(DRAIN_BAR, 1);
-    fence_mbar_init();
-  }
-  pdl_wait();
-  for (int i = threadIdx.x; i <= G; i += blockDim.x) s_off[i] = g.offsets[i];
-  __syncthreads();
-  if (warp == 2) {
-    // exclusive scan of M-tiles per group: s_mt[e] = first M-tile of e
-    const int per = (G + 31) / 32;  // <= 8
-    int loc[8];
-    int sum = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      loc[i] = 0;
-      const int gi = lane * per + i;
-      if (i < per && gi < G) {
-        const int n = s_off[gi + 1] - s_off[gi];
-        loc[i] = n > 0 ? (n + C::BM - 1) / C::BM : 0;
-      }
-      sum += loc[i];
-    }
-    int incl = sum;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, off);
-      if (lane >= off) incl += v;
-    }
-    int run = incl - sum;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int gi = lane * per + i;
-      if (i < per && gi < G) s_mt[gi] = run;
-      run += loc[i];
-    }
-    if (lane == 31) s_mt[G] = incl;
-  }
-  __syncthreads();
-  const int NT1 = 2 * g.m / BN, NT2 = g.d / BN;
-  const int total1 = s_mt[G] * NT1, total2 = s_mt[G] * NT2;
-  const int total = total1 + total2;
-  if (static_cast<int>(blockIdx.x) >= total) return;  // before any TMEM or TMA use
-
-  if (warp == 1) {
-    tmem_alloc(smem_u32(const_cast<uint32_t*>(s_tmem)), C::TMEM_COLS);
-    tmem_relinquish();
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *s_tmem;
-  // work item t -> (down?, group, M-tile of the group, N-tile, M-tile index)
-  struct Item {
-    bool dn;
-    int grp, mt, nb, mtg;
-  };
-  auto item = [&](int t) -> Item {
-    Item r;
-    r.dn = t >= total1;
-    const int tl = r.dn ? t - total1 : t;
-    tile_coords(tl, r.dn ? NT2 : NT1, s_mt, G, r.grp, r.mt, r.nb);
-    r.mtg = s_mt[r.grp] + r.mt;
-    return r;
-  };
-
-  if (warp == 0) {
-    // ------------------------------------------------ TMA producer (lane 0)
-    if (lane == 0) {
-      tma_prefetch_desc(&tma_a1);
-      tma_prefetch_desc(&tma_b1);
-      tma_prefetch_desc(&tma_a2);
-      tma_prefetch_desc(&tma_b2);
-    }
-    int stage = 0;
-    uint32_t ph = 0;
-    bool ok = true;
-    uint32_t armed = 0, armed_ph = 0;
-    // what an item's A rows wait for: a down item for its M-tile's h, a
-    // gate/up item (with the gather) for its M-tile's rows; NT1 counts each.
-    // Acquire-loaded one item ahead (as k_ffn_ws).
-    auto dep_of = [&](const Item& it) -> const int32_t* {
-      return it.dn ? g.ready : (g.x != nullptr ? g.gathered : nullptr);
-    };
-    auto flag_of = [&](int t) -> int {
-      if (t >= total) return 0;
-      const Item it = item(t);
-      const int32_t* dp = dep_of(it);
-      return dp != nullptr ? ld_acquire_gpu(dp + it.mtg) : 0;
-    };
-    int flag_cur = lane == 0 ? flag_of(static_cast<int>(blockIdx.x)) : 0;
-    const uint64_t pol_once = policy_evict_first();
-    for (int t = blockIdx.x; t < total; t += gridDim.x) {
-      const Item it = item(t);
-      const int flag = flag_cur;
-      if (lane == 0) flag_cur = flag_of(t + static_cast<int>(gridDim.x));
-      if (lane == 0) {
-        const CUtensorMap* ta = it.dn ? &tma_a2 : &tma_a1;
-        const CUtensorMap* tb = it.dn ? &tma_b2 : &tma_b1;
-        const int row0 = s_off[it.grp] + it.mt * C::BM;
-        const int brow = it.grp * (it.dn ? g.d : 2 * g.m) + it.nb * BN;
-        const int KB = (it.dn ? g.m : g.d) / FFN_BK;
-        const int32_t* dp = dep_of(it);
-        // an expert of one M-tile reads its weights once: they go to L2 as
-        // evict-first, leaving room for the weights that later M-tiles reuse
-        const bool once = s_mt[it.grp + 1] - s_mt[it.grp] == 1;
-        int pre = 0;  // k-blocks whose weights go out before the dependency is met
-        // already met (the usual case once the first wave is under way): the
-        // ordinary pipeline, A rows and weights together
-        const bool met = dp == nullptr || flag >= NT1;
-        if (dp != nullptr && met) fence_proxy_async_all();  // rows written by generic stores, read through TMA
-        if (!met) {
-          pre = KB < STAGES ? KB : STAGES;
-          const int st0 = stage;
-          for (int kb = 0; kb < pre; ++kb) {
-            if (!mbar_wait(EMPTY_BAR(stage), ph ^ 1u, g.limit_ns, s_abort)) {
-              ok = false;
-              break;
-            }
-            mbar_arrive_expect_tx(FULL_BAR(stage), C::A_BYTES + C::B_BYTES);
-            if (once)
-              tma_load_2d_hint(sB + stage * C::B_BYTES, tb, FULL_BAR(stage), kb * FFN_BK, brow, pol_once);
-            else
-              tma_load_2d(sB + stage * C::B_BYTES, tb, FULL_BAR(stage), kb * FFN_BK, brow);
-            armed |= 1u << stage;
-            armed_ph = (armed_ph & ~(1u << stage)) | (ph << stage);
-            if (++stage == STAGES) {
-              stage = 0;
-              ph ^= 1u;
-            }
-          }
-          if (ok) {
-            // every gate/up tile of this M-tile has stored its h columns (down
-            // item), or every share of its rows is gathered (gate/up item)
-            const volatile int32_t* rp = dp + it.mtg;
-            const uint64_t t0 = globaltimer_ns();
-            while (*rp < NT1) {
-              if (*s_abort || globaltimer_ns() - t0 > g.limit_ns) {
-                ok = false;
-                break;
-              }
-            }
-            __threadfence();
-            fence_proxy_async_all();  // rows written by generic stores, read through the tensor map
-          }
-          if (ok) {
-            int st = st0;
-            for (int kb = 0; kb < pre; ++kb) {
-              tma_load_2d(sA + st * C::A_BYTES, ta, FULL_BAR(st), kb * FFN_BK, row0);
-              if (++st == STAGES) st = 0;
-            }
-          }
-        }
-        for (int kb = pre; ok && kb < KB; ++kb) {
-          if (!mbar_wait(EMPTY_BAR(stage), ph ^ 1u, g.limit_ns, s_abort)) {
-            ok = false;
-            break;
-          }
-          mbar_arrive_expect_tx(FULL_BAR(stage), C::A_BYTES + C::B_BYTES);
-          tma_load_2d(sA + stage * C::A_BYTES, ta, FULL_BAR(stage), kb * FFN_BK, row0);
-          if (once)
-            tma_load_2d_hint(sB + stage * C::B_BYTES, tb, FULL_BAR(stage), kb * FFN_BK, brow, pol_once);
-          else
-            tma_load_2d(sB + stage * C::B_BYTES, tb, FULL_BAR(stage), kb * FFN_BK, brow);
-          armed |= 1u << stage;
-          armed_ph = (armed_ph & ~(1u << stage)) | (ph << stage);
-          if (++stage == STAGES) {
-            stage = 0;
-            ph ^= 1u;
-          }
-        }
-      }
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!ok) break;
-    }
-    if (lane == 0 && !ok) {
-      *s_abort = 1;
-      report_status(g.status, DECOMOE_ERR_TIMEOUT);
-      int no_abort = 0;
-      for (int s = 0; s < STAGES; ++s)
-        if ((armed >> s) & 1u) mbar_wait(FULL_BAR(s), (armed_ph >> s) & 1u, g.limit_ns, &no_abort);
-    }
-  } else if (warp == 1 && lane == 0) {
-    // ------------------------------------------------ MMA issuer
-    constexpr uint32_t IDESC = idesc_bf16_f32(C::BM, BN);
-    int stage = 0;
-    uint32_t ph = 0;
-    bool ok = true, issued = false;
-    int n = 0;
-    for (int t = blockIdx.x; t < total; t += gridDim.x, ++n) {
-      const bool dn = t >= total1;
-      const int KB = (dn ? g.m : g.d) / FFN_BK;
-      const int acc = n & 1;
-      const uint32_t aph = (n >> 1) & 1;
-      if (!mbar_wait(TEMPTY_BAR(acc), aph ^ 1u, g.limit_ns, s_abort)) {
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      const uint32_t dt = tmem_base + static_cast<uint32_t>(acc * BN);
-      for (int kb = 0; kb < KB; ++kb) {
-        if (!mbar_wait(FULL_BAR(stage), ph, g.limit_ns, s_abort)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint64_t ad = smem_desc_kmajor<FFN_BK>(sA + stage * C::A_BYTES);
-        const uint64_t bd = smem_desc_kmajor<FFN_BK>(sB + stage * C::B_BYTES);
-#pragma unroll
-        for (int kk = 0; kk < FFN_BK / 16; ++kk)
-          tc_mma_f16(dt, ad + 2u * kk, bd + 2u * kk, IDESC, (kb | kk) != 0 ? 1u : 0u);
-        tc_commit(EMPTY_BAR(stage));
-        issued = true;
-        if (++stage == STAGES) {
-          stage = 0;
-          ph ^= 1u;
-        }
-      }
-      if (!ok) break;
-      tc_commit(TFULL_BAR(acc));
-    }
-    if (!ok) {
-      *s_abort = 1;
-      report_status(g.status, DECOMOE_ERR_TIMEOUT);
-      if (issued) {
-        int no_abort = 0;
-        tc_commit(DRAIN_BAR);
-        mbar_wait(DRAIN_BAR, 0, g.limit_ns, &no_abort);
-      }
-    }
-  } else if (warp >= 2) {
-    // ------------------------------------------------ row gather (with g.x):
-    // one share of each of this CTA's gate/up M-tiles, in work order, copied
-    // while the accumulator the epilogue needs next is still being computed
-    const int et = static_cast<int>(threadIdx.x) - 64;  // 0 .. 32*EW-1
-    int gshare = g.x != nullptr ? static_cast<int>(blockIdx.x) : total1;  // next share's work item
-    auto gather_share = [&](int t) {
-      const int vec = g.d / 8;
-      constexpr int U = 8;  // 16-byte loads in flight per thread
-      const Item it = item(t);
-      const int r0 = s_off[it.grp] + it.mt * C::BM;
-      const int r1 = min(r0 + C::BM, s_off[it.grp + 1]);
-      const int per = (r1 - r0 + NT1 - 1) / NT1;
-      const int a = min(r0 + it.nb * per, r1), b = min(a + per, r1);
-      for (int i = et; i < b - a; i += 32 * EW) s_gperm[i] = g.perm[a + i];
-      named_bar_sync(1, 32 * EW);
-      const int nv = (b - a) * vec;
-      for (int i0 = et; i0 < nv; i0 += 32 * EW * U) {
-        uint4 v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int i = i0 + u * 32 * EW;
-          if (i < nv) {
-            const int r = i / vec;
-            v[u] = __ldg(g.x + static_cast<int64_t>(s_gperm[r]) * vec + (i - r * vec));
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int i = i0 + u * 32 * EW;
-          if (i < nv) {
-            const int r = i / vec;
-            g.x_perm[static_cast<int64_t>(a + r) * vec + (i - r * vec)] = v[u];
-          }
-        }
-      }
-      // publish the share to the gate/up tiles of this M-tile (and free
-      // s_gperm for the next share)
-      fence_proxy_async_all();
-      named_bar_sync(1, 32 * EW);
-      if (warp == 2 && lane == 0) {
-        __threadfence();
-        atomicAdd(g.gathered + it.mtg, 1);
-      }
-    };
-    // ------------------------------------------------ epilogue (k_gemm_tc's)
-    const int q = warp & 3;
-    const int wp = (warp - 2) >> 2;
-    constexpr int WPQ = EW / 4;
-    bool ok = true;
-    int n = 0;
-    for (int t = blockIdx.x; t < total; t += gridDim.x, ++n) {
-      const Item it = item(t);
-      const int acc = n & 1;
-      const uint32_t aph = (n >> 1) & 1;
-      const int row0 = s_off[it.grp] + it.mt * C::BM;
-      const int row_end = s_off[it.grp + 1];
-      // gather shares until this tile's accumulator is complete (one thread
-      // tests the barrier, all epilogue threads follow its answer); while
-      // shares remain the warps never block here, so every share gets copied
-      while (gshare < total1) {
-        if (et == 0) s_gperm[C::BM] = mbar_test(TFULL_BAR(acc), aph) ? 1 : 0;
-        named_bar_sync(1, 32 * EW);
-        const bool full = s_gperm[C::BM] != 0;
-        named_bar_sync(1, 32 * EW);
-        if (full) break;
-        gather_share(gshare);
-        gshare += gridDim.x;
-      }
-      if (!mbar_wait(TFULL_BAR(acc), aph, g.limit_ns, s_abort)) {
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      const int grow = row0 + q * 32 + lane;
-      const bool valid = grow < row_end;
-      const uint32_t tb = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * BN);
-      if (!it.dn) {
-        constexpr int GU = DECOMOE_GU_BLOCK;
-        __nv_bfloat16* out = static_cast<__nv_bfloat16*>(g.h);
-#pragma unroll 1
-        for (int cc = 32 * wp; cc < BN / 2; cc += 32 * WPQ) {
-          const int half = cc / GU, c = cc % GU;
-          uint32_t gr[32], ur[32];
-          tmem_ld32(tb + half * 2 * GU + c, gr);
-          tmem_ld32(tb + half * 2 * GU + GU + c, ur);
-          tc_wait_ld();
-          uint32_t pk[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const float g0 = __uint_as_float(gr[2 * i]), g1 = __uint_as_float(gr[2 * i + 1]);
-            const float u0 = __uint_as_float(ur[2 * i]), u1 = __uint_as_float(ur[2 * i + 1]);
-            pk[i] = pack_bf16x2(silu_f(g0) * u0, silu_f(g1) * u1);
-          }
-          if (valid) {
-            uint4* dst = reinterpret_cast<uint4*>(out + static_cast<int64_t>(grow) * g.m + it.nb * (BN / 2) + cc);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) dst[v] = make_uint4(pk[4 * v], pk[4 * v + 1], pk[4 * v + 2], pk[4 * v + 3]);
-          }
-        }
-      } else {
-        __nv_bfloat16* out = static_cast<__nv_bfloat16*>(g.y);
-#pragma unroll 1
-        for (int c = 32 * wp; c < BN; c += 32 * WPQ) {
-          uint32_t r[32];
-          tmem_ld32(tb + c, r);
-          tc_wait_ld();
-          uint32_t pk[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) pk[i] = pack_bf16x2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
-          if (valid) {
-            uint4* dst = reinterpret_cast<uint4*>(out + static_cast<int64_t>(grow) * g.d + it.nb * BN + c);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) dst[v] = make_uint4(pk[4 * v], pk[4 * v + 1], pk[4 * v + 2], pk[4 * v + 3]);
-          }
-        }
-      }
-      tc_fence_before();
-      mbar_arrive(TEMPTY_BAR(acc));
-      if (!it.dn) {
-        // this tile's h columns are stored: publish them to the down tiles
-        fence_proxy_async_all();
-        named_bar_sync(1, 32 * EW);
-        if (warp == 2 && lane == 0) {
-          __threadfence();
-          atomicAdd(g.ready + it.mtg, 1);
-        }
-      }
-    }
-    if (!ok) {
-      *s_abort = 1;
-      report_status(g.status, DECOMOE_ERR_TIMEOUT);
+// Gate/up (h given w_gu), down (w_down) or both over rows grouped by expert:
+// a: x_perm, or with perm the token-ordered x (x_copy: receives the grouped
+// rows then, or null); see k_ffn_pair.
+static int launch_ffn_pair(const void* a, const int32_t* perm, void* x_copy, int64_t rows, int d, int m, const void* w_gu,
+                           const void* w_down, const int32_t* offsets, int G, void* h, void* y, int32_t* ready,
+                           int32_t* status, cudaStream_t s) {
+  const bool gu = w_gu != nullptr, dn = w_down != nullptr;
+  CUtensorMap ta1, ta1s, tb1, ta2, ta2s, tb2;
+  if (gu) {
+    DM_RET(make_tmap_bf16(&tb1, w_gu, static_cast<uint64_t>(d), static_cast<uint64_t>(G) * 2 * m, 128, PF_BK));
+    if (perm == nullptr) {
+      DM_RET(make_tmap_bf16(&ta1, a, static_cast<uint64_t>(d), static_cast<uint64_t>(rows), PF_BM, PF_BK));
+      DM_RET(make_tmap_bf16(&ta1s, a, static_cast<uint64_t>(d), static_cast<uint64_t>(rows), PF_BM / 2, PF_BK));
+    } else {
+      ta1 = ta1s = tb1;  // rows gathered by index: not used
     }
   }
-  pdl_trigger();
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 1) {
-    __syncwarp();
-    tc_fence_after();
-    tmem_dealloc(tmem_base, C::TMEM_COLS);
+  if (dn) {
+    DM_RET(make_tmap_bf16(&ta2, h, static_cast<uint64_t>(m), static_cast<uint64_t>(rows), PF_BM, PF_BK));
+    DM_RET(make_tmap_bf16(&ta2s, h, static_cast<uint64_t>(m), static_cast<uint64_t>(rows), PF_BM / 2, PF_BK));
+    DM_RET(make_tmap_bf16(&tb2, w_down, static_cast<uint64_t>(m), static_cast<uint64_t>(G) * d, 128, PF_BK));
   }
-#undef FULL_BAR
-#undef EMPTY_BAR
-#undef TFULL_BAR
-#undef TEMPTY_BAR
-#undef DRAIN_BAR
-}
-
-// gather_x / perm given: the launch fills x_perm itself (see k_ffn_tc);
-// the gathered counters follow the ready counters in the same array.
-static int launch_ffn_tc(const void* x_perm, int rows, int d, int m, const void* w_gu, const void* w_down,
-                         const int32_t* offsets, int G, void* h, void* y, int32_t* ready, int32_t* status,
-                         cudaStream_t s, const void* gather_x = nullptr, const int32_t* perm = nullptr) {
-  using C = FfnCfg;
-  CUtensorMap ta1, tb1, ta2, tb2;
-  DM_RET(make_tmap_bf16(&ta1, x_perm, static_cast<uint64_t>(d), static_cast<uint64_t>(rows), C::BM, FFN_BK));
-  DM_RET(make_tmap_bf16(&tb1, w_gu, static_cast<uint64_t>(d), static_cast<uint64_t>(G) * 2 * m, FFN_BN, FFN_BK));
-  DM_RET(make_tmap_bf16(&ta2, h, static_cast<uint64_t>(m), static_cast<uint64_t>(rows), C::BM, FFN_BK));
-  DM_RET(make_tmap_bf16(&tb2, w_down, static_cast<uint64_t>(m), static_cast<uint64_t>(G) * d, FFN_BN, FFN_BK));
-  TcFfnArgs g;
+  if (!gu) ta1 = ta2, ta1s = ta2s, tb1 = tb2;
+  if (!dn) ta2 = ta1, ta2s = ta1s, tb2 = tb1;
+  PairArgs g;
   g.offsets = offsets;
   g.G = G;
-  g.rows = rows;
   g.d = d;
   g.m = m;
+  g.gu = gu;
+  g.dn = dn;
   g.h = h;
   g.y = y;
   g.ready = ready;
   g.status = status;
   g.limit_ns = static_cast<uint64_t>(wait_limit_ns());
-  g.x = static_cast<const uint4*>(gather_x);
+  g.x = perm != nullptr ? static_cast<const uint8_t*>(a) : nullptr;
   g.perm = perm;
-  g.x_perm = static_cast<uint4*>(const_cast<void*>(x_perm));
-  g.gathered = ready + (rows / C::BM + G + 1);
-  static_assert(C::SMEM + sizeof(int) * (C::BM + 1) <= 232448, "shared memory budget");
-  static_assert(C::SMEM > 232448 / 2, "one CTA per SM: the dependency waits need every CTA resident");
-  DM_CUDA_CHECK(cudaFuncSetAttribute(k_ffn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(C::SMEM)));
-  const int64_t ub = (static_cast<int64_t>(rows) / C::BM + G) * static_cast<int64_t>((2 * m + d) / FFN_BN);
-  const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(sm_count(), ub)));
-  DM_CUDA_CHECK(launch_pdl(k_ffn_tc, dim3(grid), dim3(64 + 32 * FFN_EW), C::SMEM, s, ta1, tb1, ta2, tb2, g));
+  g.x_copy = static_cast<uint8_t*>(x_copy);
+  const int64_t ub = (rows / (2 * PF_BM) + std::min<int64_t>(G, rows)) * ((gu ? 2 * m : 0) + (dn ? d : 0)) / PF_BN;
+  const int ncl = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(pair_clusters(), ub)));
+  DM_CUDA_CHECK(cudaFuncSetAttribute(k_ffn_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(PF_SMEM)));
+  DM_CUDA_CHECK(launch_pdl(k_ffn_pair, dim3(2 * ncl), dim3(PF_THREADS), PF_SMEM, s, ta1, tb1, ta2, tb2, ta1s, ta2s, g));
   return DECOMOE_OK;
 }
 
@@ -2430,43 +2005,6 @@ static int expert_check(const char* name, const void* a, const int32_t* offsets,
   return DECOMOE_OK;
 }
 
-// Pipeline shape of the two expert GEMMs: k-block depth (64 -> 128-byte
-// swizzle, 32 -> 64-byte swizzle) and the number of shared-memory stages.
-#ifndef DECOMOE_GU_BK
-#define DECOMOE_GU_BK 64
-#endif
-#ifndef DECOMOE_GU_STAGES
-#define DECOMOE_GU_STAGES 4
-#endif
-#ifndef DECOMOE_DN_BK
-#define DECOMOE_DN_BK 64
-#endif
-#ifndef DECOMOE_GU_MP
-#define DECOMOE_GU_MP 1
-#endif
-#ifndef DECOMOE_GU_OCC
-#define DECOMOE_GU_OCC 1
-#endif
-#ifndef DECOMOE_DN_OCC
-#define DECOMOE_DN_OCC 1
-#endif
-#ifndef DECOMOE_GU_EW
-#define DECOMOE_GU_EW 8
-#endif
-#ifndef DECOMOE_DN_EW
-#define DECOMOE_DN_EW 8
-#endif
-#ifndef DECOMOE_DN_MP
-#define DECOMOE_DN_MP 1
-#endif
-#ifndef DECOMOE_DN_STAGES
-#define DECOMOE_DN_STAGES 4
-#endif
-constexpr int GU_BK = DECOMOE_GU_BK, GU_STAGES = DECOMOE_GU_STAGES;
-constexpr int DN_BK = DECOMOE_DN_BK, DN_STAGES = DECOMOE_DN_STAGES;
-constexpr int GU_MP = DECOMOE_GU_MP, DN_MP = DECOMOE_DN_MP;
-constexpr int GU_OCC = DECOMOE_GU_OCC, DN_OCC = DECOMOE_DN_OCC, GU_EW = DECOMOE_GU_EW, DN_EW = DECOMOE_DN_EW;
-
 int decomoe_expert_gate_up(const void* x_perm, const int32_t* offsets, int64_t rows, int K, int d, int m,
                            int dtype, const void* w_gate_up, void* h, int32_t* status_dev, int32_t* sched_dev,
                            decomoe_stream_t stream) {
@@ -2480,10 +2018,8 @@ int decomoe_expert_gate_up(const void* x_perm, const int32_t* offsets, int64_t r
                               static_cast<const float*>(w_gate_up), static_cast<float*>(h), nullptr, s);
   if (static_cast<int64_t>(R) <= static_cast<int64_t>(DECOMOE_WS_MAX_AVG_ROWS) * K)
     return launch_ws_auto<true>(x_perm, R, d, w_gate_up, 2 * m, offsets, K, h, m, status_dev, s);
-  // A = x_perm [R, d], B = w_gate_up [K*2m, d] (only experts < K are read)
-  return launch_tc<256, EPI_SWIGLU, GU_STAGES, GU_BK, false, GU_MP, GU_EW, GU_OCC>(
-      x_perm, R, d, w_gate_up, static_cast<int64_t>(K) * 2 * m, offsets, K, 2 * m, h, m, nullptr, status_dev, s, 0,
-      nullptr, 0, sched_dev);
+  (void)sched_dev;  // the pair kernel hands its tiles out in a fixed order
+  return launch_ffn_pair(x_perm, nullptr, nullptr, R, d, m, w_gate_up, nullptr, offsets, K, h, nullptr, nullptr, status_dev, s);
 }
 
 int decomoe_expert_down(const void* h, const int32_t* offsets, int64_t rows, int K, int d, int m, int dtype,
@@ -2503,10 +2039,9 @@ int decomoe_expert_down(const void* h, const int32_t* offsets, int64_t rows, int
   }
   if (static_cast<int64_t>(R) <= static_cast<int64_t>(DECOMOE_WS_MAX_AVG_ROWS) * K)
     return launch_ws_auto<false>(h, R, m, w_down, d, offsets, K, y_perm, d, status_dev, s);
-  // A = h [R, m], B = w_down [K*d, m]
-  return launch_tc<256, EPI_BF16, DN_STAGES, DN_BK, false, DN_MP, DN_EW, DN_OCC>(h, R, m, w_down, static_cast<int64_t>(K) * d, offsets,
-                                                                  K, d, y_perm, d, nullptr, status_dev, s, 0,
-                                                                  nullptr, 0, sched_dev);
+  (void)sched_dev;
+  return launch_ffn_pair(nullptr, nullptr, nullptr, R, d, m, nullptr, w_down, offsets, K, const_cast<void*>(h), y_perm, nullptr,
+                           status_dev, s);
 }
 
 int decomoe_expert_gate_up_gather(const void* x, int64_t T, const int32_t* perm_token, const int32_t* offsets,
@@ -2524,9 +2059,7 @@ int decomoe_expert_gate_up_gather(const void* x, int64_t T, const int32_t* perm_
                               static_cast<float*>(h), perm_token, s);
   if (static_cast<int64_t>(R) <= static_cast<int64_t>(DECOMOE_WS_MAX_AVG_ROWS) * K)
     return launch_ws<true, 4, true>(x, R, d, w_gate_up, 2 * m, offsets, K, h, m, status_dev, s, perm_token, T);
-  return launch_tc<256, EPI_SWIGLU, GU_STAGES, GU_BK, 2>(
-      x, R, d, w_gate_up, static_cast<int64_t>(K) * 2 * m, offsets, K, 2 * m, h, m, nullptr, status_dev, s, 0,
-      perm_token, T);
+  return launch_ffn_pair(x, perm_token, nullptr, R, d, m, w_gate_up, nullptr, offsets, K, h, nullptr, nullptr, status_dev, s);
 }
 
 int decomoe_expert_swiglu_gather(const void* x, int64_t T, const int32_t* perm_token, const int32_t* offsets,
@@ -2577,39 +2110,26 @@ int decomoe_expert_swiglu_ref(const void* x_perm, const int32_t* offsets, int64_
 namespace decomoe {
 
 // Rows from which the fused launch is taken (with fewer, the gate/up tiles
-// leave SMs idle and the fused form gains nothing), and up to which the
-// tokens-as-M form is fused (measured per layer: 7 us faster at 2048 and
-// 16384 rows, 1-2 us at 8192 and 32768, 5 and 20 us slower at 65536 and
-// 131072 rows).
+// leave SMs idle and the fused form gains nothing).
 #ifndef DECOMOE_FFN_FUSED_MIN_ROWS
 #define DECOMOE_FFN_FUSED_MIN_ROWS 16
 #endif
-#ifndef DECOMOE_FFN_FUSED_TC_MAX_ROWS
-#define DECOMOE_FFN_FUSED_TC_MAX_ROWS 32768
-#endif
-// Both expert GEMMs in one launch: k_ffn_ws at decode sizes (bf16, at most 8
-// rows per expert on average), k_ffn_tc above up to
-// DECOMOE_FFN_FUSED_TC_MAX_ROWS rows; nothing launched (and *launched false)
-// for fp32, fewer than DECOMOE_FFN_FUSED_MIN_ROWS rows or more than that.
-// Which one-launch form the expert FFN takes: FFN_FUSED_NONE (two launches),
-// FFN_FUSED_WS (decode sizes) or FFN_FUSED_TC (tokens as M).
-int expert_ffn_fused_kind(int64_t rows, int K, int m, int dtype) {
+// Which one-launch form the expert FFN takes: FFN_FUSED_NONE (two launches:
+// fp32 and fewer than DECOMOE_FFN_FUSED_MIN_ROWS rows), FFN_FUSED_WS (at most 8
+// rows per expert on average) or FFN_FUSED_PAIR (above, any size).
+int expert_ffn_fused_kind(int64_t rows, int K, int dtype) {
   constexpr int64_t min_rows = DECOMOE_FFN_FUSED_MIN_ROWS;
-  constexpr int64_t tc_max_rows = DECOMOE_FFN_FUSED_TC_MAX_ROWS;
   if (dtype != DECOMOE_BF16 || rows < min_rows || rows <= 0 || K <= 0) return FFN_FUSED_NONE;
-  if (rows <= static_cast<int64_t>(DECOMOE_WS_MAX_AVG_ROWS) * K) return FFN_FUSED_WS;
-  // the tokens-as-M kernel tiles gate/up in whole 256-column blocks
-  if (rows > tc_max_rows || (2 * m) % FFN_BN != 0) return FFN_FUSED_NONE;
-  return FFN_FUSED_TC;
+  return rows <= static_cast<int64_t>(DECOMOE_WS_MAX_AVG_ROWS) * K ? FFN_FUSED_WS : FFN_FUSED_PAIR;
 }
 
 int launch_expert_ffn_fused(const void* x_perm, const int32_t* offsets, int64_t rows, int K, int d, int m, int dtype,
                             const void* w_gate_up, const void* w_down, void* h, void* y_perm, int32_t* ready,
                             int32_t* status, cudaStream_t s, bool* launched, const void* gather_x,
-                            const int32_t* perm) {
+                            const int32_t* perm, bool copy_rows) {
   *launched = false;
-  const int kind = expert_ffn_fused_kind(rows, K, m, dtype);
-  DM_ARG_CHECK(gather_x == nullptr || kind == FFN_FUSED_TC, "expert ffn: the row gather needs the tokens-as-M form");
+  const int kind = expert_ffn_fused_kind(rows, K, dtype);
+  DM_ARG_CHECK(gather_x == nullptr || kind == FFN_FUSED_PAIR, "expert ffn: the row gather needs the pair form");
   if (kind == FFN_FUSED_NONE) return DECOMOE_OK;
   DM_RET(expert_check("expert_gate_up", x_perm, offsets, rows, K, d, m, dtype, w_gate_up, h));
   DM_RET(expert_check("expert_down", h, offsets, rows, K, d, m, dtype, w_down, y_perm));
@@ -2620,15 +2140,16 @@ int launch_expert_ffn_fused(const void* x_perm, const int32_t* offsets, int64_t 
     DM_RET(launch_ffn_ws(x_perm, static_cast<int>(rows), d, m, w_gate_up, w_down, offsets, K, h, y_perm, ready,
                          status, s));
   else
-    DM_RET(launch_ffn_tc(x_perm, static_cast<int>(rows), d, m, w_gate_up, w_down, offsets, K, h, y_perm, ready,
-                         status, s, gather_x, perm));
+    DM_RET(launch_ffn_pair(gather_x != nullptr ? gather_x : x_perm, gather_x != nullptr ? perm : nullptr,
+                           copy_rows ? const_cast<void*>(x_perm) : nullptr, rows, d, m, w_gate_up, w_down, offsets, K, h, y_perm, ready, status, s));
   *launched = true;
   return DECOMOE_OK;
 }
 
 // int32 counters the fused expert launch needs (zero at launch): one per
-// expert (decode kernel) or two per M-tile (prefill kernel: h stored, rows
-// gathered).
+// expert (decode kernel) or two per 256-row tile (pair kernel).
+// Rows that decomoe_expert_swiglu_fused runs as one launch (its contract).
+constexpr int64_t PUBLIC_FUSED_MAX_ROWS = 32768;
 size_t expert_ffn_sync_ints(int64_t rows, int E) { return 2 * static_cast<size_t>(rows / 128 + E + 1); }
 
 }  // namespace decomoe
@@ -2645,8 +2166,9 @@ int decomoe_expert_swiglu_fused(const void* x_perm, const int32_t* offsets, int6
   using namespace decomoe;
   clear_error();
   bool fused = false;
-  DM_RET(launch_expert_ffn_fused(x_perm, offsets, rows, K, d, m, dtype, w_gate_up, w_down, h_ws, y_perm, ready,
-                                 status_dev, reinterpret_cast<cudaStream_t>(stream), &fused));
+  if (rows <= PUBLIC_FUSED_MAX_ROWS)
+    DM_RET(launch_expert_ffn_fused(x_perm, offsets, rows, K, d, m, dtype, w_gate_up, w_down, h_ws, y_perm, ready,
+                                   status_dev, reinterpret_cast<cudaStream_t>(stream), &fused));
   if (fused) return DECOMOE_OK;
   return decomoe_expert_swiglu(x_perm, offsets, rows, K, d, m, dtype, w_gate_up, w_down, h_ws, y_perm, status_dev,
                                nullptr, stream);
@@ -2659,12 +2181,12 @@ int decomoe_expert_swiglu_fused_gather(const void* x, int64_t T, const int32_t* 
   using namespace decomoe;
   clear_error();
   DM_ARG_CHECK(x != nullptr && perm_token != nullptr && T >= 0, "expert_swiglu_fused_gather: null pointer");
-  DM_ARG_CHECK(expert_ffn_fused_kind(rows, K, m, dtype) == FFN_FUSED_TC,
+  DM_ARG_CHECK(rows <= PUBLIC_FUSED_MAX_ROWS && expert_ffn_fused_kind(rows, K, dtype) == FFN_FUSED_PAIR,
                "expert_swiglu_fused_gather: %lld rows at K=%d take no one-launch tokens-as-M form",
                (long long)rows, K);
   bool fused = false;
   DM_RET(launch_expert_ffn_fused(x_perm, offsets, rows, K, d, m, dtype, w_gate_up, w_down, h_ws, y_perm, ready,
-                                 status_dev, reinterpret_cast<cudaStream_t>(stream), &fused, x, perm_token));
+                                 status_dev, reinterpret_cast<cudaStream_t>(stream), &fused, x, perm_token, true));
   return fused ? DECOMOE_OK : DECOMOE_ERR_UNSUPPORTED;
 }
 

@@ -344,16 +344,11 @@ int moe_layer_impl(const void* x, const void* w_r, const float* bias, const void
                                topk_idx, topk_w, mass, counts, offsets, perm, inv, x_perm, h, y_perm, K_dev,
                                reinterpret_cast<int32_t*>(base + L.off[WS_DSYNC]), status_dev, s);
   }
-  // Where the experts take the one-launch tokens-as-M form on at least
-  // gather_min_rows routed rows, that launch copies the
-  // dispatched rows itself (per M-tile, while its accumulators fill) and the
-  // dispatch skips its gather launch (measured: T=2048 K=64 0.2258 -> 0.2244
-  // ms, end to end 8.80 -> 9.00 M tokens/s; at 1024 rows 3.4 us slower, the
-  // shares being a few rows each).
-  constexpr int64_t gather_min_rows = 8192;
-  auto ffn_gathers = [&](int K_groups) {
-    return T * k >= gather_min_rows && expert_ffn_fused_kind(T * k, K_groups, m, dtype) == FFN_FUSED_TC;
-  };
+  // Where the experts take the pair form, its gate/up reads x by index and the
+  // dispatch has no rows to gather (T = 131, K = 64 99.8 -> 95.9 us, T = 777 181.8
+  // -> 173.9, T = 16384 1144 -> 1057 against a gather launch). Their grouped copy
+  // in the workspace is then left only for inspection (scratch not discarded).
+  auto ffn_gathers = [&](int K_groups) { return expert_ffn_fused_kind(T * k, K_groups, dtype) == FFN_FUSED_PAIR; };
   bool gathers = false;
   if (K_fixed != 0) {
     // a1-a5: router logits over all E reordered experts, full-pool mass
@@ -397,7 +392,8 @@ int moe_layer_impl(const void* x, const void* w_r, const float* bias, const void
   // keeps them chained programmatically)
   bool fused = false;
   DM_RET(launch_expert_ffn_fused(x_perm, offsets, T * k, K, d, m, dtype, w_gate_up, w_down, h, y_perm, sync,
-                                 status_dev, s, &fused, gathers ? x : nullptr, gathers ? perm : nullptr));
+                                 status_dev, s, &fused, gathers ? x : nullptr, gathers ? perm : nullptr,
+                                 !discard_scratch()));
   if (!fused)
     DM_RET(decomoe_expert_swiglu(x_perm, offsets, T * k, K, d, m, dtype, w_gate_up, w_down, h, y_perm, status_dev,
                                  nullptr, stream));
