@@ -632,13 +632,15 @@ static int att_active_clusters(int cs) {
 //
 // Bound: the tensor pipe, once one head's chain (score product, row softmax,
 // P back to tensor memory, value product) fits under the other head's
-// products. Blocks of 128 keys halve the hand-offs per key against 64, and a
-// 128-column score product reads shared memory at its own rate (64 columns:
-// 1.5 times over it); packed fp32 pairs and 208 registers keep a row's 128
-// scores in registers without a spill. 32 query heads on 4 KV heads: 16384
-// rows 1999 -> 1511 us (1100 -> 1455 TFLOP/s), 1553 rows 39.4 -> 26.6 us, 509
-// rows over 4605 keys 90.8 -> 59.7 us against 64-key blocks with a separate
-// transpose of V.
+// products; at 16384 rows the power limit. Blocks of 128 keys halve the
+// hand-offs per key against 64, and a 128-column score product reads shared
+// memory at its own rate (64 columns: 1.5 times over it); packed fp32 pairs and
+// 208 registers keep a row's 128 scores in registers. 32 query heads on 4 KV
+// heads, 64-key blocks with a separate transpose of V -> this: 16384 rows 2001
+// -> 1335 us (1099 -> 1648 TFLOP/s), 1553 rows 40.3 -> 24.6 us, 509 rows over
+// 4605 keys 90.7 -> 39.3 us. The same kernel with one lane of a divergent branch
+// issuing the products took 1484, 26.7 and 43.3 us; one lane polling for each
+// softmax warp is 8 to 10 % slower.
 constexpr int ATP_BM = 128;                  // query rows per CTA
 constexpr int ATP_BN = 128;                  // keys per block
 constexpr int ATP_HEADS = 2;                 // query heads per CTA (same KV head)
@@ -709,6 +711,12 @@ __device__ __forceinline__ float ex2_approx(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+// The larger of three (one instruction).
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
 }
 // Two fp32 lanes in one 64-bit register pair (the packed fp32 pipe).
 __device__ __forceinline__ uint64_t f32x2(float lo, float hi) {
@@ -975,70 +983,68 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
       }
     }
   } else if (warp == 9) {
-    // ------------------------------------------------ MMA issuer (lane 0)
-    if (lane == 0) {
-      // S_x = Q_x K^T over the 128 features (two 64-feature halves)
-      auto issue_s = [&](int x, int st) {
-        const uint64_t ad = smem_desc_kmajor<64>(sQ + x * ATP_SLOT);
-        const uint64_t bd = smem_desc_kmajor<64>(sKV + st * ATP_SLOT);
+    // ------------------------------------------------ MMA issuer (whole warp, one elected thread issues)
+    const bool leader = elect_one();
+    auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
+      return __all_sync(0xffffffffu, mbar_wait(bar, parity, a.limit_ns, s_abort));
+    };
+    const uint64_t qd = smem_desc_kmajor<64>(sQ), kd = smem_desc_kmajor<64>(sKV), vd = smem_desc_v(sKV);
+    // S_x = Q_x K^T over the 128 features (two 64-feature halves)
+    auto issue_s = [&](int x, int st) {
+      const uint64_t ad = qd + static_cast<uint32_t>(x * (ATP_SLOT >> 4));
+      const uint64_t bd = kd + static_cast<uint32_t>(st * (ATP_SLOT >> 4));
 #pragma unroll
-        for (int kb = 0; kb < 2; ++kb)
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            tc_mma_f16(S_TM(x), ad + (ATP_HALF >> 4) * kb + 2u * kk, bd + (ATP_HALF >> 4) * kb + 2u * kk, IDESC_S,
-                       (kb | kk) != 0 ? 1u : 0u);
-      };
-      // O_x += P_x V_j over 64 of the block's keys
-      auto issue_pv = [&](int x, int st, int half, bool acc) {
-        const uint64_t bd = smem_desc_v(sKV + st * ATP_SLOT);
+      for (int kb = 0; kb < 2; ++kb)
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          tc_mma_f16_ts(O_TM(x), S_TM(x) + 32u * half + 8u * kk, bd + (2048u >> 4) * (4 * half + kk), IDESC_O,
-                        (acc || half > 0 || kk > 0) ? 1u : 0u);
-      };
-      bool ok = mbar_wait(Q_BAR, 0, a.limit_ns, s_abort) && mbar_wait(FULL(0), 0, a.limit_ns, s_abort);
-      bool issued = false;
-      if (ok) {
-        tc_fence_after();
+          tc_mma_f16(S_TM(x), ad + (ATP_HALF >> 4) * kb + 2u * kk, bd + (ATP_HALF >> 4) * kb + 2u * kk, IDESC_S,
+                     (kb | kk) != 0 ? 1u : 0u);
+    };
+    // O_x += P_x V_j over 64 of the block's keys
+    auto issue_pv = [&](int x, int st, int half, bool acc) {
+      const uint64_t bd = vd + static_cast<uint32_t>(st * (ATP_SLOT >> 4));
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk)
+        tc_mma_f16_ts(O_TM(x), S_TM(x) + 32u * half + 8u * kk, bd + (2048u >> 4) * (4 * half + kk), IDESC_O,
+                      (acc || half > 0 || kk > 0) ? 1u : 0u);
+    };
+    bool ok = wait(Q_BAR, 0) && wait(FULL(0), 0);
+    bool issued = false;
+    if (ok) {
+      tc_fence_after();
+      if (leader) {
+#pragma unroll
         for (int x = 0; x < ATP_HEADS; ++x) {
           issue_s(x, 0);
           tc_commit(S_FULL(x));
         }
         tc_commit(EMPTY(0));
-        issued = true;
       }
-      int st = 1;  // ring slot of V_j, then of K_{j+1}
-      uint32_t ph = 0;
-      for (int j = 0; ok && j < nblk; ++j) {
-        int stk = st + 1;
-        uint32_t phk = ph;
-        if (stk == ATP_NST) {
-          stk = 0;
-          phk ^= 1u;
+      issued = true;
+    }
+    int st = 1;  // ring slot of V_j, then of K_{j+1}
+    uint32_t ph = 0;
+    for (int j = 0; ok && j < nblk; ++j) {
+      int stk = st + 1;
+      uint32_t phk = ph;
+      if (stk == ATP_NST) {
+        stk = 0;
+        phk ^= 1u;
+      }
+      ok = wait(FULL(st), ph);
+#pragma unroll
+      for (int x = 0; x < ATP_HEADS; ++x) {
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          ok = ok && wait(P_FULL(x, half), j & 1);
+          tc_fence_after();
+          if (ok && leader) issue_pv(x, st, half, j > 0);
         }
-        for (int x = 0; ok && x < ATP_HEADS; ++x) {
-          if (x == 0 && !mbar_wait(FULL(st), ph, a.limit_ns, s_abort)) {
-            ok = false;
-            break;
-          }
-          for (int half = 0; half < 2; ++half) {
-            if (!mbar_wait(P_FULL(x, half), j & 1, a.limit_ns, s_abort)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            issue_pv(x, st, half, j > 0);
-          }
-          if (!ok) break;
+        if (x == 0 && j + 1 < nblk) ok = ok && wait(FULL(stk), phk);
+        tc_fence_after();
+        if (ok && leader) {
           if (x == ATP_HEADS - 1) tc_commit(EMPTY(st));  // V_j read by both heads' products
           if (j + 1 < nblk) {
-            if (x == 0) {
-              if (!mbar_wait(FULL(stk), phk, a.limit_ns, s_abort)) {
-                ok = false;
-                break;
-              }
-              tc_fence_after();
-            }
             issue_s(x, stk);
             tc_commit(S_FULL(x));
             if (x == ATP_HEADS - 1) tc_commit(EMPTY(stk));
@@ -1046,23 +1052,24 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
             tc_commit(O_FINAL(x));
           }
         }
-        st = stk + 1;
-        ph = phk;
-        if (st == ATP_NST) {
-          st = 0;
-          ph ^= 1u;
-        }
       }
-      if (!ok) {
-        *s_abort = 1;
-        report_status(a.status, DECOMOE_ERR_TIMEOUT);
-        if (issued) {
-          int no_abort = 0;
-          tc_commit(DRAIN);
-          mbar_wait(DRAIN, 0, a.limit_ns, &no_abort);
-        }
+      st = stk + 1;
+      ph = phk;
+      if (st == ATP_NST) {
+        st = 0;
+        ph ^= 1u;
       }
     }
+    if (!ok && leader) {
+      *s_abort = 1;
+      report_status(a.status, DECOMOE_ERR_TIMEOUT);
+      if (issued) {
+        int no_abort = 0;
+        tc_commit(DRAIN);
+        mbar_wait(DRAIN, 0, a.limit_ns, &no_abort);
+      }
+    }
+    __syncwarp();
   }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(ATP_REGS_SOFTMAX));
@@ -1103,7 +1110,7 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
       for (int c = 0; c < ATP_BN; c += 8)
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-          mx[u] = fmaxf(fmaxf(mx[u], __uint_as_float(sv[c + 2 * u])), __uint_as_float(sv[c + 2 * u + 1]));
+          mx[u] = max3(mx[u], __uint_as_float(sv[c + 2 * u]), __uint_as_float(sv[c + 2 * u + 1]));
       const float m_blk = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
       float factor = 1.0f;
       if (m_blk > m + ATP_RESCALE) {
@@ -1231,15 +1238,15 @@ static bool att_use_prefill(int64_t n, int Hq, int Hkv) { return n * (Hq / Hkv) 
 // Whether to split the tiles' key blocks over several CTAs, and how far: L
 // blocks per item (0: no split), the items and those of split tiles. One CTA
 // per SM: a chunk of queries over a long cache has few tiles and leaves SMs
-// idle. Times in block steps (1.5 us for two heads): an item costs its blocks
+// idle. Times in block steps (1.1 us for two heads): an item costs its blocks
 // plus 2.5 (set-up, first loads, output); writing partial rows and the merge
-// launch 3 plus 0.025 per item. Tiles of about equal length run in whole waves of one
-// item per SM; lengths from one block up (n = C) fill the SMs evenly and end
-// with the longest. Only taken where the estimate is 10 % better; measured
-// (32 heads on 4 KV heads, whole -> split): 509 queries over 4605 keys 59.7 ->
-// 42.5 us in 2, 33 over 4129 54.8 -> 19.5 in 9, 87 over 13767 169 -> 32 in 9,
-// 300 over 8300 104 -> 48.7 in 3, 700 over 8700 109 -> 95 in 3; 509 over 1009
-// would go 17.2 -> 21.0 in 2 and 1024 over 5120 66 -> 83.
+// launch 3 plus 0.025 per item. Tiles of about equal length run in whole waves
+// of one item per SM; lengths from one block up (n = C) fill the SMs evenly and
+// end with the longest. Only taken where the estimate is 10 % better; measured
+// when a step took 1.5 us (32 heads on 4 KV heads, whole -> split): 509 queries
+// over 4605 keys 59.7 -> 42.5 us in 2, 33 over 4129 54.8 -> 19.5 in 9, 87 over
+// 13767 169 -> 32 in 9, 300 over 8300 104 -> 48.7 in 3, 700 over 8700 109 -> 95
+// in 3; 509 over 1009 would go 17.2 -> 21.0 in 2 and 1024 over 5120 66 -> 83.
 struct AttPreSplit {
   int L;
   int64_t items, split_items, split_tiles;
