@@ -2,23 +2,10 @@
 // only the first K physically contiguous expert MLPs; gate, up and down
 // matmuls, Appendix C_expert = 6Kdm) and the bf16 router projection.
 //
-// bf16, many rows: a persistent warp-specialised tcgen05 kernel.
-//   warp 0      TMA producer: A tile (128 rows x 64) and B tile (BN rows x 64)
-//               per k-block into a STAGES-deep shared-memory ring (128-byte
-//               swizzle), completion on mbarriers.
-//   warp 1      TMEM allocator and MMA issuer: one thread issues
-//               tcgen05.mma.cta_group::1.kind::f16 (M=128, N=BN, K=16) into a
-//               double-buffered fp32 accumulator in tensor memory.
-//   warps 2..   epilogue (EW warps, 8 by default: two per TMEM lane
-//               quarter, each on half of the tile's columns): tcgen05.ld of
-//               the accumulator, one row per thread, fused SwiGLU / bf16 /
-//               fp32+bias conversion, stores to global.
-// Tiles: for every group (expert) g, ceil(rows_g / 128) M-tiles times
-// N / BN N-tiles; see tile_coords for the order. Rows past the group's end are
-// computed on whatever TMA loaded (zeros past the tensor end) and never
-// stored.
+// bf16, many rows: the tcgen05 kernel on pairs of SMs (ffn_pair.cuh).
 // bf16, few rows per expert (decode): the weights-stationary tcgen05 kernel
-// k_moe_ws (expert weights as M, the expert's tokens as N).
+// k_moe_ws (expert weights as M, the expert's tokens as N) and its one-launch
+// form k_ffn_ws. Router: k_router_tc (router rows as M, tokens as N).
 // f32: CUDA-core kernels (exact fp32 products, fp32 accumulation).
 #include <atomic>
 #include <mutex>
@@ -28,10 +15,10 @@
 #include "decomoe_internal.cuh"
 #include "simt_rows.cuh"
 
-// Kernel choice for the bf16 expert GEMMs: the weights-stationary k_moe_ws
-// when the average expert gets at most DECOMOE_WS_MAX_AVG_ROWS rows (decode
-// sizes: every tile streams its own weight slice), the tokens-as-M k_gemm_tc
-// otherwise (prefill: faster when many rows share an expert's weights).
+// Kernel choice for the bf16 expert GEMMs: the weights-stationary kernels when
+// the average expert gets at most DECOMOE_WS_MAX_AVG_ROWS rows (decode sizes:
+// every tile streams its own weight slice), the pair kernel otherwise (prefill:
+// faster when many rows share an expert's weights).
 #ifndef DECOMOE_WS_MAX_AVG_ROWS
 #define DECOMOE_WS_MAX_AVG_ROWS 8
 #endif
@@ -104,53 +91,7 @@ int make_tmap_bf16_3d(CUtensorMap* m, const void* base, const uint64_t dims[3], 
   return DECOMOE_OK;
 }
 
-// ------------------------------------------------------------------ tcgen05 GEMM
-// EPI_SWIGLU: columns [0, BN/2) gate, [BN/2, BN) up -> bf16 silu(g)*u.
-// EPI_BF16: bf16 store. EPI_F32_BIAS: fp32 + bias[col]. EPI_F32_BIAS_T: the
-// accumulator is the transpose of the output (A = router rows, B = tokens):
-// out[col * ld + row] = acc + bias[row], columns >= n_valid skipped.
-enum { EPI_SWIGLU = 0, EPI_BF16 = 1, EPI_F32_BIAS = 2, EPI_F32_BIAS_T = 3 };
-
-struct TcArgs {
-  const int32_t* offsets;  // [ngroups + 1] row offsets (device) or null: one group [0, rows)
-  int ngroups;
-  int rows;
-  int n_per_group;  // B rows per group
-  int kdim;
-  void* out;
-  int64_t out_ld;  // elements
-  const float* bias;
-  int32_t* status;
-  uint64_t limit_ns;
-  int n_valid;  // EPI_F32_BIAS_T: number of valid output columns (tokens)
-  const int32_t* a_rows;  // GA != 0: A row r is row a_rows[r] of the A tensor (rows entries)
-  const uint8_t* a_ptr;   // GA == 2: the A tensor itself (rows of kdim bf16)
-  int* sched;             // dynamic scheduling: tile counter, zero at launch (null: static round robin)
-  int64_t split_stride;   // KS > 1: elements between the k slices' partial outputs
-};
-
-// MP = M-tiles per work item. MP = 1: one 128-row A tile per B tile, two
-// accumulator buffers (epilogue overlaps the next tile's MMAs). MP = 2: two
-// M-tiles of the same group share each B tile (two M=128 MMAs per k-step,
-// 2/3 of the shared-memory traffic per MMA), one buffer of two accumulators.
-// OCC = resident CTAs per SM. OCC = 2 halves each CTA's shared memory and
-// TMEM (one accumulator, no double buffer): two tiles then share an SM, so
-// one CTA's weight streaming overlaps the other's tensor-core work.
-template <int BN, int STAGES, int BK_, int MP_ = 1, int OCC_ = 1>
-struct TcCfg {
-  static constexpr int BM = 128, BK = BK_, MP = MP_, OCC = OCC_;
-  static constexpr int A_BYTES = BM * BK * 2;  // one M-tile
-  static constexpr int B_BYTES = BN * BK * 2;
-  static constexpr int STAGE_BYTES = MP * A_BYTES + B_BYTES;
-  static constexpr int NBUF = (MP == 1 && OCC == 1) ? 2 : 1;  // accumulator buffers
-  static constexpr int TMEM_COLS = NBUF * MP * BN;             // power of two for BN in {128, 256}
-  static constexpr int MAXG = DECOMOE_MAX_E;
-  static constexpr int TQ = 4;  // depth of the tile-id queue (dynamic scheduling)
-  static constexpr int NBARS = 2 * STAGES + 5 + 2 * TQ;
-  static constexpr size_t SMEM =
-      1024 + static_cast<size_t>(STAGES) * STAGE_BYTES + NBARS * 8 + 2 * (MAXG + 1) * 4 + 16 + TQ * 4;
-};
-
+// ------------------------------------------------------------------ tile order
 // Work item -> (group, M-tile inside the group, N-tile). M-tiles are visited
 // alternately from the two ends of the group-ordered list (first, last,
 // second, second-to-last, ...), each with all its N-tiles back to back. With
@@ -181,458 +122,202 @@ __device__ __forceinline__ void tile_coords(int tile, int NT, const int* s_mt, i
 #include "ffn_pair.cuh"
 namespace decomoe {
 
-// EW epilogue warps (4 or 8): with 8, two warps share each 32-lane TMEM
-// quarter and split its column chunks, so the epilogue's latency is hidden.
-// GA: how A tiles reach shared memory. 0: tiled TMA of rows [row0, row0+128)
-// of A. 2: four extra warps, one A row per thread, 16-byte cp.async of the
-// rows a_rows[row0 ..] into the 128-byte-swizzled layout the TMA would
-// produce; each thread's copies complete on the stage's full barrier.
-// KS: split of the k loop. Work item = (output tile, k slice); slice s runs
-// k-blocks [s*KB/KS, (s+1)*KB/KS) and writes its partial sums to
-// out + s * split_stride (EPI_F32_BIAS_T only; the caller adds the slices).
-template <int BN, int EPI, int STAGES, int BK, int GA = 0, int MP = 1, int EW = 8, int OCC = 1, int KS = 1>
-__global__ void __launch_bounds__(64 + 32 * EW + (GA == 2 ? 128 : 0), OCC)
-    k_gemm_tc(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUtensorMap tma_b,
-              const TcArgs g) {
-  using C = TcCfg<BN, STAGES, BK, MP, OCC>;
-  static_assert(GA == 0 || GA == 2, "A rows by tiled TMA (0) or by cp.async gather (2)");
-  static_assert(!(GA != 0 && MP != 1), "gathered A takes one M-tile per work item");
-  static_assert(GA != 2 || BK == 64, "the cp.async gather writes 128-byte swizzled rows");
-  static_assert(KS == 1 || (EPI == EPI_F32_BIAS_T && MP == 1 && GA == 0), "k split: transposed fp32 partials only");
+// ------------------------------------------------------------------ tensor-core router
+// logits[t, e] = sum_k x[t, k] w_r[e, k] (+ bias[e]) with router rows as M (128
+// per tile), BN tokens as N and the k loop split into KS slices: work item =
+// (128 router rows, BN tokens, slice). Slice s runs k-blocks [s KB, (s + 1) KB)
+// and writes its partial sums to out + s * split_stride without the bias; the
+// caller adds the slices. Persistent, one CTA per SM: warp 0 streams both
+// operands by TMA through an eight-stage ring, warp 1 issues the products,
+// eight epilogue warps (two per 32-lane TMEM quarter) store the transposed
+// accumulator. Bound by latency up to 4096 tokens, by reading x above. With the
+// slices' reduction, d = 2048, E = 128 (the shared GEMM kernel before -> this):
+// 131 tokens 7.2 -> 5.7 us, 2048 9.7 -> 8.0, 16384 20.3 -> 15.1.
+constexpr int RT_BM = 128, RT_BK = 64, RT_STAGES = 8, RT_EW = 8;
+template <int BN>
+struct RtCfg {
+  static constexpr int A_BYTES = RT_BM * RT_BK * 2;
+  static constexpr int B_BYTES = BN * RT_BK * 2;
+  static constexpr int ACC_COLS = BN < 32 ? 32 : BN;  // tensor-memory columns per accumulator
+  static constexpr int NBARS = 2 * RT_STAGES + 5;
+  static constexpr size_t SMEM = 1024 + static_cast<size_t>(RT_STAGES) * (A_BYTES + B_BYTES) + NBARS * 8 + 16;
+};
+struct RouterArgs {
+  int E, n, npad;        // router rows, tokens, tokens rounded up to BN
+  int kdim;
+  float* out;            // [n, E], slice s at + s * split_stride
+  int64_t split_stride;
+  const float* bias;     // KS == 1 only
+  int32_t* status;
+  uint64_t limit_ns;
+};
+
+template <int BN, int KS>
+__global__ void __launch_bounds__(64 + 32 * RT_EW, 1)
+    k_router_tc(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUtensorMap tma_b,
+                const RouterArgs g) {
+  using C = RtCfg<BN>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t pad = (1024u - (raw & 1023u)) & 1023u;
   uint8_t* smem = smem_raw + pad;
   const uint32_t sA = raw + pad;
-  const uint32_t sB = sA + STAGES * MP * C::A_BYTES;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * C::STAGE_BYTES);
-  int* s_off = reinterpret_cast<int*>(bars + C::NBARS);
-  int* s_mt = s_off + (C::MAXG + 1);
-  volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(s_mt + (C::MAXG + 1));
+  const uint32_t sB = sA + RT_STAGES * C::A_BYTES;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + RT_STAGES * (C::A_BYTES + C::B_BYTES));
+  volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(bars + C::NBARS);
   volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
-  volatile int* s_tq = reinterpret_cast<volatile int*>(s_tmem + 4);  // [TQ] tile ids
-
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t bar0 = smem_u32(bars);
-  // barrier slots: full[STAGES] | empty[STAGES] | tfull[2] | tempty[2] | drain | tqfull[TQ] | tqempty[TQ]
-#define FULL_BAR(s) (bar0 + 8u * (s))
-#define EMPTY_BAR(s) (bar0 + 8u * (STAGES + (s)))
-#define TFULL_BAR(a) (bar0 + 8u * (2 * STAGES + (a)))
-#define TEMPTY_BAR(a) (bar0 + 8u * (2 * STAGES + 2 + (a)))
-#define DRAIN_BAR (bar0 + 8u * (2 * STAGES + 4))
-#define TQF_BAR(i) (bar0 + 8u * (2 * STAGES + 5 + (i)))
-#define TQE_BAR(i) (bar0 + 8u * (2 * STAGES + 5 + C::TQ + (i)))
+  auto FULL = [&](int s) { return bar0 + 8u * s; };
+  auto EMPTY = [&](int s) { return bar0 + 8u * (RT_STAGES + s); };
+  auto TFULL = [&](int a) { return bar0 + 8u * (2 * RT_STAGES + a); };
+  auto TEMPTY = [&](int a) { return bar0 + 8u * (2 * RT_STAGES + 2 + a); };
+  const uint32_t DRAIN = bar0 + 8u * (2 * RT_STAGES + 4);
 
-  const int G = g.ngroups;
   if (threadIdx.x == 0) {
     *s_abort = 0;
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(FULL_BAR(s), GA == 2 ? 1 + 128 : 1);  // + one arrival per cp.async A-row thread
-      mbar_init(EMPTY_BAR(s), 1);
+    for (int s = 0; s < RT_STAGES; ++s) {
+      mbar_init(FULL(s), 1);
+      mbar_init(EMPTY(s), 1);
     }
     for (int a = 0; a < 2; ++a) {
-      mbar_init(TFULL_BAR(a), 1);
-      mbar_init(TEMPTY_BAR(a), 32 * EW);
+      mbar_init(TFULL(a), 1);
+      mbar_init(TEMPTY(a), 32 * RT_EW);
     }
-    mbar_init(DRAIN_BAR, 1);
-    for (int i = 0; i < C::TQ; ++i) {
-      mbar_init(TQF_BAR(i), 1);
-      mbar_init(TQE_BAR(i), 1 + EW);  // the MMA thread and lane 0 of every epilogue warp
-    }
+    mbar_init(DRAIN, 1);
     fence_mbar_init();
+  }
+  if (warp == 1) {
+    tmem_alloc(smem_u32(const_cast<uint32_t*>(s_tmem)), 2 * C::ACC_COLS);
+    tmem_relinquish();
   }
   // wait for the earlier kernels' results; the next kernel is released only
   // at the end (its CTAs would otherwise sit resident through this one)
   pdl_wait();
-  for (int i = threadIdx.x; i <= G; i += blockDim.x)
-    s_off[i] = (g.offsets != nullptr) ? g.offsets[i] : (i == 0 ? 0 : g.rows);
-  __syncthreads();
-  if (warp == 2) {
-    // exclusive scan of work units (MP M-tiles) per group: s_mt[g] = first unit of g
-    const int per = (G + 31) / 32;  // <= 8
-    int loc[8];
-    int sum = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      loc[i] = 0;
-      const int gi = lane * per + i;
-      if (i < per && gi < G) {
-        const int n = s_off[gi + 1] - s_off[gi];
-        loc[i] = n > 0 ? (n + C::BM * MP - 1) / (C::BM * MP) : 0;
-      }
-      sum += loc[i];
-    }
-    int incl = sum;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, off);
-      if (lane >= off) incl += v;
-    }
-    int run = incl - sum;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int gi = lane * per + i;
-      if (i < per && gi < G) s_mt[gi] = run;
-      run += loc[i];
-    }
-    if (lane == 31) s_mt[G] = incl;
-  }
-  __syncthreads();
-  const int NT = g.n_per_group / BN;
-  const int total = s_mt[G] * NT * KS;
-  if (static_cast<int>(blockIdx.x) >= total) return;  // before any TMEM or TMA use
-
-  if (warp == 1) {
-    tmem_alloc(smem_u32(const_cast<uint32_t*>(s_tmem)), C::TMEM_COLS);
-    tmem_relinquish();
-  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
-  const int KB = g.kdim / C::BK / KS;  // k-blocks per work item
-
-  // Tile sequence of this CTA. Static: blockIdx.x, + gridDim.x, ... Dynamic:
-  // the producer takes the next id from the global counter and passes it to
-  // the MMA and epilogue warps through a TQ-deep shared-memory queue; -1 ends.
-  const bool dyn = GA == 0 && g.sched != nullptr;
-  auto static_tile = [&](int i) -> int {
-    const int t = static_cast<int>(blockIdx.x) + i * static_cast<int>(gridDim.x);
-    return t < total ? t : -1;
-  };
-  auto produce_tile = [&](int i) -> int {  // producer thread; returns -2 on timeout
-    if (!dyn) return static_tile(i);
-    const int slot = i % C::TQ;
-    const uint32_t qph = (i / C::TQ) & 1;
-    if (!mbar_wait(TQE_BAR(slot), qph ^ 1u, g.limit_ns, s_abort)) return -2;
-    int t = atomicAdd(g.sched, 1);
-    if (t >= total) t = -1;
-    s_tq[slot] = t;
-    mbar_arrive(TQF_BAR(slot));
-    return t;
-  };
-  auto consume_tile = [&](int i, bool arrive) -> int {  // returns -2 on timeout
-    if (!dyn) return static_tile(i);
-    const int slot = i % C::TQ;
-    const uint32_t qph = (i / C::TQ) & 1;
-    if (!mbar_wait(TQF_BAR(slot), qph, g.limit_ns, s_abort)) return -2;
-    const int t = s_tq[slot];
-    if (arrive) mbar_arrive(TQE_BAR(slot));
-    return t;
-  };
+  const int MT = g.E / RT_BM, total = MT * (g.npad / BN) * KS;
+  const int KB = g.kdim / RT_BK / KS;  // k-blocks per work item
 
   if (warp == 0) {
-    // ------------------------------------------------ TMA producer (lane 0 issues)
+    // ------------------------------------------------ TMA producer (lane 0)
     if (lane == 0) {
       tma_prefetch_desc(&tma_a);
       tma_prefetch_desc(&tma_b);
-    }
-    int stage = 0;
-    uint32_t ph = 0;
-    bool ok = true;
-    uint32_t armed = 0;  // bit s: stage s was ever filled
-    uint32_t armed_ph = 0;
-    for (int ti = 0;; ++ti) {
-      int tile = 0;
-      if (lane == 0) tile = produce_tile(ti);
-      tile = __shfl_sync(0xffffffffu, tile, 0);
-      if (tile == -2) {
-        ok = false;
-        break;
-      }
-      if (tile < 0) break;
-      int grp, mt, nb;
-      tile_coords(tile / KS, NT, s_mt, G, grp, mt, nb);
-      const int row0 = s_off[grp] + mt * MP * C::BM;
-      const int brow = grp * g.n_per_group + nb * BN;
-      const int kbase = (tile % KS) * KB;  // first k-block of this work item's slice
-      const bool has2 = MP == 2 && row0 + C::BM < s_off[grp + 1];  // second M-tile has rows
-      if (lane == 0) {
+      int stage = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      uint32_t armed = 0, armed_ph = 0;
+      for (int t = blockIdx.x; ok && t < total; t += gridDim.x) {
+        const int row0 = t / KS % MT * RT_BM, col0 = t / KS / MT * BN, k0 = t % KS * KB;
         for (int kb = 0; kb < KB; ++kb) {
-          if (!mbar_wait(EMPTY_BAR(stage), ph ^ 1u, g.limit_ns, s_abort)) {
+          if (!mbar_wait(EMPTY(stage), ph ^ 1u, g.limit_ns, s_abort)) {
             ok = false;
             break;
           }
-          mbar_arrive_expect_tx(FULL_BAR(stage), (GA == 2 ? 0 : (has2 ? 2 : 1) * C::A_BYTES) + C::B_BYTES);
-          if constexpr (GA == 0) {
-            tma_load_2d(sA + stage * MP * C::A_BYTES, &tma_a, FULL_BAR(stage), (kbase + kb) * C::BK, row0);
-            if (has2)
-              tma_load_2d(sA + (stage * MP + 1) * C::A_BYTES, &tma_a, FULL_BAR(stage), (kbase + kb) * C::BK,
-                          row0 + C::BM);
-          }
-          tma_load_2d(sB + stage * C::B_BYTES, &tma_b, FULL_BAR(stage), (kbase + kb) * C::BK, brow);
+          mbar_arrive_expect_tx(FULL(stage), C::A_BYTES + C::B_BYTES);
+          tma_load_2d(sA + stage * C::A_BYTES, &tma_a, FULL(stage), (k0 + kb) * RT_BK, row0);
+          tma_load_2d(sB + stage * C::B_BYTES, &tma_b, FULL(stage), (k0 + kb) * RT_BK, col0);
           armed |= 1u << stage;
           armed_ph = (armed_ph & ~(1u << stage)) | (ph << stage);
-          if (++stage == STAGES) {
+          if (++stage == RT_STAGES) {
             stage = 0;
             ph ^= 1u;
           }
         }
       }
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!ok) break;
+      if (!ok) {
+        *s_abort = 1;
+        report_status(g.status, DECOMOE_ERR_TIMEOUT);
+        // let every copy this thread started land before the CTA can exit
+        int no_abort = 0;
+        for (int s = 0; s < RT_STAGES; ++s)
+          if ((armed >> s) & 1u) mbar_wait(FULL(s), (armed_ph >> s) & 1u, g.limit_ns, &no_abort);
+      }
     }
-    if (lane == 0 && !ok) {
-      *s_abort = 1;
-      report_status(g.status, DECOMOE_ERR_TIMEOUT);
-      // let every copy this thread started land before the CTA can exit
-      int no_abort = 0;
-      for (int s = 0; s < STAGES; ++s)
-        if ((armed >> s) & 1u) mbar_wait(FULL_BAR(s), (armed_ph >> s) & 1u, g.limit_ns, &no_abort);
-    }
-  } else if (warp == 1 && lane == 0) {
-    // ------------------------------------------------ MMA issuer
-    constexpr uint32_t IDESC = idesc_bf16_f32(C::BM, BN);
+  } else if (warp == 1) {
+    // ------------------------------------------------ MMA issuer (whole warp, one elected thread issues)
+    constexpr uint32_t IDESC = idesc_bf16_f32(RT_BM, BN);
+    const bool leader = elect_one();
     int stage = 0;
     uint32_t ph = 0;
     bool ok = true, issued = false;
-    for (int it = 0;; ++it) {
-      const int tile = consume_tile(it, true);
-      if (tile == -2) {
-        ok = false;
-        break;
-      }
-      if (tile < 0) break;
-      const int acc = it % C::NBUF;
-      const uint32_t aph = (it / C::NBUF) & 1;
-      bool has2 = false;
-      if constexpr (MP == 2) {
-        int grp, mt, nb;
-        tile_coords(tile / KS, NT, s_mt, G, grp, mt, nb);
-        has2 = s_off[grp] + (mt * 2 + 1) * C::BM < s_off[grp + 1];
-      }
-      if (!mbar_wait(TEMPTY_BAR(acc), aph ^ 1u, g.limit_ns, s_abort)) {
+    int n = 0;
+    for (int t = blockIdx.x; ok && t < total; t += gridDim.x, ++n) {
+      const int acc = n & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(TEMPTY(acc), ((n >> 1) & 1) ^ 1u, g.limit_ns, s_abort))) {
         ok = false;
         break;
       }
       tc_fence_after();
-      const uint32_t dt = tmem_base + static_cast<uint32_t>(acc * BN);
+      const uint32_t dt = tmem_base + static_cast<uint32_t>(acc * C::ACC_COLS);
       for (int kb = 0; kb < KB; ++kb) {
-        if (!mbar_wait(FULL_BAR(stage), ph, g.limit_ns, s_abort)) {
+        if (!__all_sync(0xffffffffu, mbar_wait(FULL(stage), ph, g.limit_ns, s_abort))) {
           ok = false;
           break;
         }
         tc_fence_after();
-        if constexpr (GA == 2) fence_proxy_async_smem();  // A rows came through the generic proxy
-        const uint64_t ad = smem_desc_kmajor<BK>(sA + stage * MP * C::A_BYTES);
-        const uint64_t bd = smem_desc_kmajor<BK>(sB + stage * C::B_BYTES);
+        const uint64_t ad = smem_desc_kmajor<RT_BK>(sA + stage * C::A_BYTES);
+        const uint64_t bd = smem_desc_kmajor<RT_BK>(sB + stage * C::B_BYTES);
+        if (leader) {
 #pragma unroll
-        for (int kk = 0; kk < C::BK / 16; ++kk) {
-          tc_mma_f16(dt, ad + 2u * kk, bd + 2u * kk, IDESC, (kb | kk) != 0 ? 1u : 0u);
-          if (MP == 2 && has2)
-            tc_mma_f16(tmem_base + BN, ad + static_cast<uint64_t>(C::A_BYTES >> 4) + 2u * kk, bd + 2u * kk, IDESC,
-                       (kb | kk) != 0 ? 1u : 0u);
+          for (int kk = 0; kk < RT_BK / 16; ++kk)
+            tc_mma_f16(dt, ad + 2u * kk, bd + 2u * kk, IDESC, (kb | kk) != 0 ? 1u : 0u);
+          tc_commit(EMPTY(stage));
+          if (kb == KB - 1) tc_commit(TFULL(acc));
         }
-        tc_commit(EMPTY_BAR(stage));
         issued = true;
-        if (++stage == STAGES) {
+        if (++stage == RT_STAGES) {
           stage = 0;
           ph ^= 1u;
         }
       }
-      if (!ok) break;
-      tc_commit(TFULL_BAR(acc));
     }
-    if (!ok) {
+    if (!ok && leader) {
       *s_abort = 1;
       report_status(g.status, DECOMOE_ERR_TIMEOUT);
       if (issued) {
         int no_abort = 0;
-        tc_commit(DRAIN_BAR);
-        mbar_wait(DRAIN_BAR, 0, g.limit_ns, &no_abort);
+        tc_commit(DRAIN);
+        mbar_wait(DRAIN, 0, g.limit_ns, &no_abort);
       }
     }
-  } else if (GA == 2 && warp >= 2 + EW) {
-    // ------------------------------------------------ A rows by cp.async:
-    // the 128 threads copy the tile's 128 A rows (token rows a_rows[row0 +
-    // i] of the A tensor), 8 x 16 bytes per row per k-block, eight lanes per
-    // row so each warp instruction reads four whole 128-byte row segments.
-    // Chunk c of tile row i lands at i*128 + ((c ^ (i & 7)) * 16): the
-    // 128-byte-swizzled layout the TMA would write.
-    const int t = threadIdx.x - 32 * (2 + EW);
-    const int c = lane & 7;                      // 16-byte chunk of the row
-    const int i0 = (t >> 5) * 32 + (lane >> 3);  // rows i0 + 4j, j < 8
-    int stage = 0;
-    uint32_t ph = 0;
+    __syncwarp();
+  } else {
+    // ------------------------------------------------ epilogue: lane = router row
+    const int q = warp & 3;          // TMEM lanes [32q, 32q + 32)
+    const int wp = (warp - 2) >> 2;  // which of the quarter's two warps
     bool ok = true;
-    for (int ti = 0;; ++ti) {
-      const int tile = static_tile(ti);
-      if (tile < 0) break;
-      int grp, mt, nb;
-      tile_coords(tile / KS, NT, s_mt, G, grp, mt, nb);
-      const int row0 = s_off[grp] + mt * C::BM;
-      const uint8_t* src[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int r = row0 + i0 + 4 * j;
-        const int src_row = (r < g.rows) ? g.a_rows[r] : 0;  // rows past the end: any valid row, never stored
-        src[j] = g.a_ptr + static_cast<int64_t>(src_row) * g.kdim * 2 + c * 16;
-      }
-      for (int kb = 0; kb < KB; ++kb) {
-        bool got = true;
-        if (lane == 0) got = mbar_wait(EMPTY_BAR(stage), ph ^ 1u, g.limit_ns, s_abort);
-        got = __shfl_sync(0xffffffffu, got, 0);
-        if (!got) {
-          ok = false;
-          break;
-        }
-        const uint32_t dst = sA + stage * C::A_BYTES;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int i = i0 + 4 * j;
-          cp_async16(dst + static_cast<uint32_t>(i) * 128u + (static_cast<uint32_t>(c ^ (i & 7)) << 4),
-                     src[j] + kb * (C::BK * 2));
-        }
-        cp_async_mbar_arrive_noinc(FULL_BAR(stage));
-        if (++stage == STAGES) {
-          stage = 0;
-          ph ^= 1u;
-        }
-      }
-      if (!ok) break;
-    }
-    cp_async_wait_all();  // every copy lands before the CTA can exit
-    if (!ok && lane == 0) {
-      *s_abort = 1;
-      report_status(g.status, DECOMOE_ERR_TIMEOUT);
-    }
-  } else if (warp >= 2) {
-    // ------------------------------------------------ epilogue
-    const int q = warp & 3;            // TMEM lanes [32q, 32q + 32) belong to this warp
-    const int wp = (warp - 2) >> 2;    // which of the quarter's warps (0 .. EW/4 - 1)
-    constexpr int WPQ = EW / 4;        // warps per quarter: column chunks are dealt round robin
-    bool ok = true;
-    for (int it = 0;; ++it) {
-      int tile = 0;
-      if (lane == 0) tile = consume_tile(it, true);
-      tile = __shfl_sync(0xffffffffu, tile, 0);
-      if (tile == -2) {
-        ok = false;
-        break;
-      }
-      if (tile < 0) break;
-      const int acc = it % C::NBUF;
-      const uint32_t aph = (it / C::NBUF) & 1;
-      int grp, mt, nb;
-      tile_coords(tile / KS, NT, s_mt, G, grp, mt, nb);
-      const int row_end = s_off[grp + 1];
-      if (!mbar_wait(TFULL_BAR(acc), aph, g.limit_ns, s_abort)) {
+    int n = 0;
+    for (int t = blockIdx.x; t < total; t += gridDim.x, ++n) {
+      const int e = t / KS % MT * RT_BM + q * 32 + lane, n0 = t / KS / MT * BN;
+      const int acc = n & 1;
+      if (!mbar_wait(TFULL(acc), (n >> 1) & 1, g.limit_ns, s_abort)) {
         ok = false;
         break;
       }
       tc_fence_after();
-#pragma unroll 1
-      for (int sub = 0; sub < MP; ++sub) {
-      const int row0 = s_off[grp] + (mt * MP + sub) * C::BM;
-      if (sub > 0 && row0 >= row_end) break;  // no second M-tile in this unit
-      const int grow = row0 + q * 32 + lane;
-      const bool valid = grow < row_end;
       const uint32_t tb =
-          tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>((acc + sub) * BN);
-      if constexpr (EPI == EPI_SWIGLU) {
-        // columns hold blocks of GU gate then GU up columns of the same
-        // features: features nb*BN/2 + half*GU + c
-        constexpr int GU = DECOMOE_GU_BLOCK;
-        static_assert(BN % (2 * GU) == 0, "N tile must hold whole gate/up blocks");
-        __nv_bfloat16* out = static_cast<__nv_bfloat16*>(g.out);
+          tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * C::ACC_COLS);
+      float* out = g.out + static_cast<int64_t>(t % KS) * g.split_stride + e;
+      const float bv = KS == 1 && g.bias != nullptr ? g.bias[e] : 0.f;
+      constexpr int CH = BN < 32 ? BN : 32;
 #pragma unroll 1
-        for (int cc = 32 * wp; cc < BN / 2; cc += 32 * WPQ) {
-          const int half = cc / GU, c = cc % GU;
-          uint32_t gr[32], ur[32];
-          tmem_ld32(tb + half * 2 * GU + c, gr);
-          tmem_ld32(tb + half * 2 * GU + GU + c, ur);
-          tc_wait_ld();
-          uint32_t pk[16];
+      for (int c0 = CH * wp; c0 < BN; c0 += 2 * CH) {
+        uint32_t r[CH];
+        if constexpr (CH == 16)
+          tmem_ld16(tb + c0, r);
+        else
+          tmem_ld32(tb + c0, r);
+        tc_wait_ld();
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const float g0 = __uint_as_float(gr[2 * i]), g1 = __uint_as_float(gr[2 * i + 1]);
-            const float u0 = __uint_as_float(ur[2 * i]), u1 = __uint_as_float(ur[2 * i + 1]);
-            pk[i] = pack_bf16x2(silu_f(g0) * u0, silu_f(g1) * u1);
-          }
-          if (valid) {
-            uint4* dst = reinterpret_cast<uint4*>(out + static_cast<int64_t>(grow) * g.out_ld +
-                                                  nb * (BN / 2) + cc);
-#pragma unroll
-            for (int v = 0; v < 4; ++v)
-              dst[v] = make_uint4(pk[4 * v], pk[4 * v + 1], pk[4 * v + 2], pk[4 * v + 3]);
-          }
-        }
-      } else if constexpr (EPI == EPI_BF16) {
-        __nv_bfloat16* out = static_cast<__nv_bfloat16*>(g.out);
-#pragma unroll 1
-        for (int c = 32 * wp; c < BN; c += 32 * WPQ) {
-          uint32_t r[32];
-          tmem_ld32(tb + c, r);
-          tc_wait_ld();
-          uint32_t pk[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i)
-            pk[i] = pack_bf16x2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
-          if (valid) {
-            uint4* dst =
-                reinterpret_cast<uint4*>(out + static_cast<int64_t>(grow) * g.out_ld + nb * BN + c);
-#pragma unroll
-            for (int v = 0; v < 4; ++v)
-              dst[v] = make_uint4(pk[4 * v], pk[4 * v + 1], pk[4 * v + 2], pk[4 * v + 3]);
-          }
-        }
-      } else if constexpr (EPI == EPI_F32_BIAS_T) {
-        // row = router row (expert), columns = tokens nb*BN + c; with a k
-        // split, slice (tile % KS) writes its partial sums without the bias
-        float* out = static_cast<float*>(g.out) + static_cast<int64_t>(tile % KS) * g.split_stride;
-        const float bv = (KS == 1 && valid && g.bias) ? g.bias[grow] : 0.f;
-        const int n0 = nb * BN;
-        if constexpr (BN == 16) {
-          if (wp == 0) {
-          uint32_t r[16];
-          tmem_ld16(tb, r);
-          tc_wait_ld();
-          if (valid) {
-#pragma unroll
-            for (int c = 0; c < 16; ++c)
-              if (n0 + c < g.n_valid) out[static_cast<int64_t>(n0 + c) * g.out_ld + grow] = __uint_as_float(r[c]) + bv;
-          }
-          }
-        } else {
-#pragma unroll 1
-          for (int c0 = 32 * wp; c0 < BN; c0 += 32 * WPQ) {
-            uint32_t r[32];
-            tmem_ld32(tb + c0, r);
-            tc_wait_ld();
-            if (valid) {
-#pragma unroll
-              for (int c = 0; c < 32; ++c)
-                if (n0 + c0 + c < g.n_valid)
-                  out[static_cast<int64_t>(n0 + c0 + c) * g.out_ld + grow] = __uint_as_float(r[c]) + bv;
-            }
-          }
-        }
-      } else {
-        float* out = static_cast<float*>(g.out);
-#pragma unroll 1
-        for (int c = 32 * wp; c < BN; c += 32 * WPQ) {
-          uint32_t r[32];
-          tmem_ld32(tb + c, r);
-          tc_wait_ld();
-          if (valid) {
-            float4* dst =
-                reinterpret_cast<float4*>(out + static_cast<int64_t>(grow) * g.out_ld + nb * BN + c);
-            const float* bptr = g.bias ? g.bias + nb * BN + c : nullptr;
-#pragma unroll
-            for (int v = 0; v < 8; ++v) {
-              float4 o;
-              o.x = __uint_as_float(r[4 * v + 0]) + (bptr ? bptr[4 * v + 0] : 0.f);
-              o.y = __uint_as_float(r[4 * v + 1]) + (bptr ? bptr[4 * v + 1] : 0.f);
-              o.z = __uint_as_float(r[4 * v + 2]) + (bptr ? bptr[4 * v + 2] : 0.f);
-              o.w = __uint_as_float(r[4 * v + 3]) + (bptr ? bptr[4 * v + 3] : 0.f);
-              dst[v] = o;
-            }
-          }
-        }
+        for (int c = 0; c < CH; ++c)
+          if (n0 + c0 + c < g.n) out[static_cast<int64_t>(n0 + c0 + c) * g.E] = __uint_as_float(r[c]) + bv;
       }
-      }  // sub
       tc_fence_before();
-      mbar_arrive(TEMPTY_BAR(acc));
+      mbar_arrive(TEMPTY(acc));
     }
     if (!ok) {
       *s_abort = 1;
@@ -645,58 +330,34 @@ __global__ void __launch_bounds__(64 + 32 * EW + (GA == 2 ? 128 : 0), OCC)
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem_base, C::TMEM_COLS);
+    tmem_dealloc(tmem_base, 2 * C::ACC_COLS);
   }
-#undef FULL_BAR
-#undef EMPTY_BAR
-#undef TFULL_BAR
-#undef TEMPTY_BAR
-#undef DRAIN_BAR
-#undef TQF_BAR
-#undef TQE_BAR
 }
 
-// A: [rows, kdim], or with GA == 2 the source tensor [a_tensor_rows, kdim]
-// whose row a_rows[r] is A row r.
-template <int BN, int EPI, int STAGES, int BK, int GA = 0, int MP = 1, int EW = 8, int OCC = 1, int KS = 1>
-static int launch_tc(const void* A, int rows, int kdim, const void* B, int64_t b_rows,
-                     const int32_t* offsets, int ngroups, int n_per_group, void* out,
-                     int64_t out_ld, const float* bias, int32_t* status, cudaStream_t s, int n_valid = 0,
-                     const int32_t* a_rows = nullptr, int64_t a_tensor_rows = 0, int* sched = nullptr,
-                     int64_t split_stride = 0) {
-  using C = TcCfg<BN, STAGES, BK, MP, OCC>;
+// Logits (KS == 1, with the bias) or KS slices of partial sums, T * E apart.
+template <int BN, int KS>
+static int launch_router_kernel(const void* x, const void* w_r, const float* bias, int64_t T, int d, int E, float* out,
+                                int32_t* status, cudaStream_t s) {
+  using C = RtCfg<BN>;
+  static_assert(C::SMEM <= 232448, "shared memory budget");
   CUtensorMap ta, tb;
-  if (GA == 2)
-    ta = CUtensorMap{};  // A is read with cp.async, not TMA
-  else
-    DM_RET(make_tmap_bf16(&ta, A, static_cast<uint64_t>(kdim), static_cast<uint64_t>(rows), C::BM, BK));
-  DM_RET(make_tmap_bf16(&tb, B, static_cast<uint64_t>(kdim), static_cast<uint64_t>(b_rows), BN, BK));
-  TcArgs g;
-  g.offsets = offsets;
-  g.ngroups = ngroups;
-  g.rows = rows;
-  g.n_per_group = n_per_group;
-  g.kdim = kdim;
+  DM_RET(make_tmap_bf16(&ta, w_r, static_cast<uint64_t>(d), static_cast<uint64_t>(E), RT_BM, RT_BK));
+  DM_RET(make_tmap_bf16(&tb, x, static_cast<uint64_t>(d), static_cast<uint64_t>(T), BN, RT_BK));
+  RouterArgs g;
+  g.E = E;
+  g.n = static_cast<int>(T);
+  g.npad = static_cast<int>((T + BN - 1) / BN) * BN;
+  g.kdim = d;
   g.out = out;
-  g.out_ld = out_ld;
+  g.split_stride = T * E;
   g.bias = bias;
   g.status = status;
   g.limit_ns = static_cast<uint64_t>(wait_limit_ns());
-  g.n_valid = n_valid;
-  g.a_rows = a_rows;
-  g.a_ptr = static_cast<const uint8_t*>(A);
-  g.sched = sched;
-  g.split_stride = split_stride;
-  if (sched != nullptr) DM_CUDA_CHECK(cudaMemsetAsync(sched, 0, sizeof(int), s));
-  auto kern = k_gemm_tc<BN, EPI, STAGES, BK, GA, MP, EW, OCC, KS>;
-  static_assert(C::SMEM <= 232448, "shared memory budget");
-  DM_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(C::SMEM)));
-  const int64_t ub_tiles =
-      (static_cast<int64_t>(rows) / C::BM + ngroups) * static_cast<int64_t>(n_per_group / BN) * KS;
-  const int64_t cap = static_cast<int64_t>(sm_count()) * OCC;
-  const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(cap, ub_tiles)));
-  DM_CUDA_CHECK(launch_pdl(kern, dim3(grid), dim3(64 + 32 * EW + (GA == 2 ? 128 : 0)), C::SMEM, s, ta, tb, g));
+  auto kern = k_router_tc<BN, KS>;
+  DM_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(C::SMEM)));
+  const int64_t total = static_cast<int64_t>(E / RT_BM) * (g.npad / BN) * KS;
+  const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(sm_count(), total)));
+  DM_CUDA_CHECK(launch_pdl(kern, dim3(grid), dim3(64 + 32 * RT_EW), C::SMEM, s, ta, tb, g));
   return DECOMOE_OK;
 }
 
@@ -706,13 +367,13 @@ static int launch_tc(const void* A, int rows, int kdim, const void* B, int64_t b
 // (up to 256 per tile, MMA width rounded up to 16). No M padding, so a ragged,
 // skewed expert population costs only what it routes; small experts (and the
 // decode sizes) become pure weight streaming with every tile reading its own
-// 128-row weight slice once. Roles as in k_gemm_tc (TMA warp, MMA warp, four
-// epilogue warps, double-buffered 256-column TMEM accumulators).
+// 128-row weight slice once. Roles: TMA warp, MMA warp, four epilogue warps;
+// double-buffered 256-column TMEM accumulators.
 //
 // Tiles: per expert e, (wrows / 128) weight blocks x ceil(n_e / 256) token
 // chunks, chunk innermost (consecutive tiles share a weight block, so it is
 // read from HBM once and from L2 after); the global list is visited
-// alternately from both ends, as in k_gemm_tc.
+// alternately from both ends (tile_coords).
 //
 // SwiGLU epilogue: with the 64-row gate/up interleave a weight block holds 64
 // gate rows (TMEM lanes 0..63) and the 64 up rows of the same features (lanes
@@ -956,8 +617,9 @@ __global__ void __launch_bounds__(192, 1)
       for (int s = 0; s < STAGES; ++s)
         if ((armed >> s) & 1u) mbar_wait(FULL_BAR(s), (armed_ph >> s) & 1u, g.limit_ns, &no_abort);
     }
-  } else if (warp == 1 && lane == 0) {
-    // ------------------------------------------------ MMA issuer
+  } else if (warp == 1) {
+    // ------------------------------------------------ MMA issuer (whole warp, one elected thread issues)
+    const bool leader = elect_one();
     int stage = 0;
     uint32_t ph = 0;
     bool ok = true, issued = false;
@@ -967,24 +629,26 @@ __global__ void __launch_bounds__(192, 1)
       const uint32_t idesc = idesc_bf16_f32(WS_BM, (T.ntok + 15) & ~15);
       const int acc = it & 1;
       const uint32_t aph = (it >> 1) & 1;
-      if (!mbar_wait(TEMPTY_BAR(acc), aph ^ 1u, g.limit_ns, s_abort)) {
+      if (!__all_sync(0xffffffffu, mbar_wait(TEMPTY_BAR(acc), aph ^ 1u, g.limit_ns, s_abort))) {
         ok = false;
         break;
       }
       tc_fence_after();
       const uint32_t dt = tmem_base + static_cast<uint32_t>(acc * WS_BN);
       for (int kb = 0; kb < KB; ++kb) {
-        if (!mbar_wait(FULL_BAR(stage), ph, g.limit_ns, s_abort)) {
+        if (!__all_sync(0xffffffffu, mbar_wait(FULL_BAR(stage), ph, g.limit_ns, s_abort))) {
           ok = false;
           break;
         }
         tc_fence_after();
         const uint64_t ad = smem_desc_kmajor<WS_BK>(sA + stage * C::A_BYTES);
         const uint64_t bd = smem_desc_kmajor<WS_BK>(sB + stage * C::B_BYTES);
+        if (leader) {
 #pragma unroll
-        for (int kk = 0; kk < WS_BK / 16; ++kk)
-          tc_mma_f16(dt, ad + 2u * kk, bd + 2u * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
-        tc_commit(EMPTY_BAR(stage));
+          for (int kk = 0; kk < WS_BK / 16; ++kk)
+            tc_mma_f16(dt, ad + 2u * kk, bd + 2u * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
+          tc_commit(EMPTY_BAR(stage));
+        }
         issued = true;
         if (++stage == STAGES) {
           stage = 0;
@@ -992,9 +656,9 @@ __global__ void __launch_bounds__(192, 1)
         }
       }
       if (!ok) break;
-      tc_commit(TFULL_BAR(acc));
+      if (leader) tc_commit(TFULL_BAR(acc));
     }
-    if (!ok) {
+    if (!ok && leader) {
       *s_abort = 1;
       report_status(g.status, DECOMOE_ERR_TIMEOUT);
       if (issued) {
@@ -1358,8 +1022,10 @@ __global__ void __launch_bounds__(192, 1)
       for (int s = 0; s < STAGES; ++s)
         if ((armed >> s) & 1u) mbar_wait(FULL_BAR(s), (armed_ph >> s) & 1u, g.limit_ns, &no_abort);
     }
-  } else if (warp == 1 && lane == 0) {
-    // ------------------------------------------------ MMA issuer
+  } else if (warp == 1) {
+    // ------------------------------------------------ MMA issuer (whole warp, one elected thread issues:
+    // against one lane of a divergent branch T=40 80.5 -> 76.9 us a layer, T=64 88.8 -> 85.2)
+    const bool leader = elect_one();
     int stage = 0;
     uint32_t ph = 0;
     bool ok = true, issued = false;
@@ -1371,24 +1037,26 @@ __global__ void __launch_bounds__(192, 1)
       const uint32_t idesc = idesc_bf16_f32(WS_BM, (T.ntok + 15) & ~15);
       const int acc = it & 1;
       const uint32_t aph = (it >> 1) & 1;
-      if (!mbar_wait(TEMPTY_BAR(acc), aph ^ 1u, g.limit_ns, s_abort)) {
+      if (!__all_sync(0xffffffffu, mbar_wait(TEMPTY_BAR(acc), aph ^ 1u, g.limit_ns, s_abort))) {
         ok = false;
         break;
       }
       tc_fence_after();
       const uint32_t dt = tmem_base + static_cast<uint32_t>(acc * BN);
       for (int kb = 0; kb < KB; ++kb) {
-        if (!mbar_wait(FULL_BAR(stage), ph, g.limit_ns, s_abort)) {
+        if (!__all_sync(0xffffffffu, mbar_wait(FULL_BAR(stage), ph, g.limit_ns, s_abort))) {
           ok = false;
           break;
         }
         tc_fence_after();
         const uint64_t ad = smem_desc_kmajor<WS_BK>(sA + stage * C::A_BYTES);
         const uint64_t bd = smem_desc_kmajor<WS_BK>(sB + stage * C::B_BYTES);
+        if (leader) {
 #pragma unroll
-        for (int kk = 0; kk < WS_BK / 16; ++kk)
-          tc_mma_f16(dt, ad + 2u * kk, bd + 2u * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
-        tc_commit(EMPTY_BAR(stage));
+          for (int kk = 0; kk < WS_BK / 16; ++kk)
+            tc_mma_f16(dt, ad + 2u * kk, bd + 2u * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
+          tc_commit(EMPTY_BAR(stage));
+        }
         issued = true;
         if (++stage == STAGES) {
           stage = 0;
@@ -1396,9 +1064,9 @@ __global__ void __launch_bounds__(192, 1)
         }
       }
       if (!ok) break;
-      tc_commit(TFULL_BAR(acc));
+      if (leader) tc_commit(TFULL_BAR(acc));
     }
-    if (!ok) {
+    if (!ok && leader) {
       *s_abort = 1;
       report_status(g.status, DECOMOE_ERR_TIMEOUT);
       if (issued) {
@@ -1686,14 +1354,6 @@ bool router_tc_supported(int d, int E) { return d % 64 == 0 && (E == 128 || E ==
 // or 256 rows, one or two M tiles) and the tokens as N tiles of BN columns, so
 // that T = 2048 already spreads over 128 CTAs; the epilogue writes the
 // transpose, logits[t, e], 32 experts of one token per warp store.
-template <int BN>
-static int launch_router_bn(const void* x, const void* w_r, const float* bias, int64_t T, int d, int E,
-                            float* logits, int32_t* status, cudaStream_t s) {
-  const int64_t npad = (T + BN - 1) / BN * BN;
-  return launch_tc<BN, EPI_F32_BIAS_T, 8, 64>(w_r, E, d, x, T, nullptr, 1, static_cast<int>(npad), logits, E,
-                                              bias, status, s, static_cast<int>(T));
-}
-
 int launch_router_tc(const void* x, const void* w_r, const float* bias, int64_t T, int d, int E,
                      float* logits, int32_t* status, cudaStream_t s) {
   if (T > 0x7fffff00LL) {
@@ -1701,9 +1361,9 @@ int launch_router_tc(const void* x, const void* w_r, const float* bias, int64_t 
     return DECOMOE_ERR_UNSUPPORTED;
   }
   const int64_t ctas = sm_count();
-  if (T <= 16 * ctas) return launch_router_bn<16>(x, w_r, bias, T, d, E, logits, status, s);
-  if (T <= 32 * ctas) return launch_router_bn<32>(x, w_r, bias, T, d, E, logits, status, s);
-  return launch_router_bn<64>(x, w_r, bias, T, d, E, logits, status, s);
+  if (T <= 16 * ctas) return launch_router_kernel<16, 1>(x, w_r, bias, T, d, E, logits, status, s);
+  if (T <= 32 * ctas) return launch_router_kernel<32, 1>(x, w_r, bias, T, d, E, logits, status, s);
+  return launch_router_kernel<64, 1>(x, w_r, bias, T, d, E, logits, status, s);
 }
 
 // k-split router: KS k slices of the router GEMM write partial logits
@@ -1751,11 +1411,8 @@ int router_split_ks(int64_t T, int d, int E) {
 template <int KS>
 static int launch_router_split_ks(const void* x, const void* w_r, const float* bias, int64_t T, int d, int E,
                                   float* logits, float* scratch, int32_t* status, cudaStream_t s) {
-  const int64_t npad = (T + 63) / 64 * 64;
   const int64_t n = T * E;
-  DM_RET((launch_tc<64, EPI_F32_BIAS_T, 8, 64, 0, 1, 8, 1, KS>(w_r, E, d, x, T, nullptr, 1, static_cast<int>(npad),
-                                                               scratch, E, nullptr, status, s, static_cast<int>(T),
-                                                               nullptr, 0, nullptr, n)));
+  DM_RET((launch_router_kernel<64, KS>(x, w_r, nullptr, T, d, E, scratch, status, s)));
   const int64_t n4 = n / 4;
   const int blocks = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((n4 + 255) / 256, sm_count())));
   DM_CUDA_CHECK(launch_pdl(k_router_reduce<KS>, dim3(blocks), dim3(256), 0, s,
@@ -1767,17 +1424,9 @@ int launch_router_parts(const void* x, const void* w_r, int64_t T, int d, int E,
                         cudaStream_t s, int* ks_out) {
   const int ks = router_split_ks(T, d, E);
   *ks_out = ks;
-  const int64_t npad = (T + 63) / 64 * 64;
-  const int64_t n = T * E;
   switch (ks) {
-    case 16:
-      return launch_tc<64, EPI_F32_BIAS_T, 8, 64, 0, 1, 8, 1, 16>(w_r, E, d, x, T, nullptr, 1, static_cast<int>(npad),
-                                                                  scratch, E, nullptr, status, s, static_cast<int>(T),
-                                                                  nullptr, 0, nullptr, n);
-    case 4:
-      return launch_tc<64, EPI_F32_BIAS_T, 8, 64, 0, 1, 8, 1, 4>(w_r, E, d, x, T, nullptr, 1, static_cast<int>(npad),
-                                                                 scratch, E, nullptr, status, s, static_cast<int>(T),
-                                                                 nullptr, 0, nullptr, n);
+    case 16: return launch_router_kernel<64, 16>(x, w_r, nullptr, T, d, E, scratch, status, s);
+    case 4: return launch_router_kernel<64, 4>(x, w_r, nullptr, T, d, E, scratch, status, s);
     default:
       return DECOMOE_OK;  // no split at this size: nothing launched
   }
