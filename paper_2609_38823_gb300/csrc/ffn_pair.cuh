@@ -9,13 +9,15 @@
 // x 256 columns. Why pairs: at 128 x 256 on one SM a 64-deep k-block moves 48 KB
 // into shared memory and the products read 48 KB back, 768 cycles of its 128
 // bytes a cycle against 512 of tensor work; half the weights per SM make that
-// 512 against 512, and the ring holds six k-blocks instead of four.
+// 512 against 512, and six k-blocks are on their way instead of four. Weights and
+// rows have rings of their own, filled by different threads: weights stream on
+// while rows wait for h or for their token numbers.
 //
 // Rows of the gate/up operand come from x by index (gather mode: four warps
 // copy them with cp.async, coalesced, in the swizzle the TMA would produce: no
 // gathered copy of x is written or read) or from grouped rows by TMA.
 //
-// Per stage each CTA's loads complete on its own barriers; a relay thread in
+// Per k-block each CTA's loads complete on its own barriers; a relay thread in
 // each passes them on to CTA 0's LOADED, the one barrier its MMA warp waits
 // for. The commits arrive on both CTAs' EMPTY and TFULL
 // barriers; both CTAs' epilogue warps arrive on CTA 0's TEMPTY. All waits are
@@ -25,13 +27,16 @@
 // still reach its shared memory.
 //
 // What bounds it: with weights in L2 and 4096 rows an expert (d = 2048, m = 768)
-// gate/up runs at 1789 TFLOP/s and down at 1551, against 1547 and 1148 of the
+// gate/up runs at 1805 TFLOP/s and down at 1560, against 1547 and 1148 of the
 // one-SM kernels before, near the power limit; with few rows an expert the
 // weight stream. The MMA warp's loop decides: issued by one thread of a divergent
 // branch with two barriers per k-block, the same kernel took 637 cycles per
 // k-block (gate/up 1576 TFLOP/s) instead of 512, and an arrival with cluster
-// release 1900. Layer at T = 2048, K = 64: 222 -> 203 us; 4096: 361 -> 307;
-// 16384, K = 128: 1237 -> 1057 (T = 131: 97.6 -> 95.9, 272: 113.7 -> 111.0).
+// release 1900. Layer against the one-SM kernels: T = 2048, K = 64 222 -> 192 us;
+// 4096 361 -> 295; 16384, K = 128 1237 -> 1027; 1552, K = 128 237 -> 219; 272, K =
+// 57 114 -> 105; 131, K = 64 97.6 -> 91.5. One ring for both operands: 199, 301,
+// 1037, 228, 109, 93.7. Eight slots for weights and four for rows: 196, 307, 1098,
+// 219, 106, 92.1 (gate/up in L2 1654 TFLOP/s instead of 1805).
 #pragma once
 
 namespace decomoe {
@@ -39,14 +44,15 @@ namespace decomoe {
 constexpr int PF_BM = 128;                  // rows per CTA (256 per tile)
 constexpr int PF_BN = 256;                  // weight rows per tile (128 per CTA)
 constexpr int PF_BK = 64;
-constexpr int PF_STAGES = 6;
-constexpr int PF_HALF = 128 * PF_BK * 2;    // A or B of one stage and CTA (16 KB)
+constexpr int PF_NB = 6, PF_NA = 6;         // ring slots for weights and for rows
+static_assert(PF_NA <= PF_NB, "the rows' slots are freed through the weights' barriers");
+constexpr int PF_HALF = 128 * PF_BK * 2;    // A or B of one k-block and CTA (16 KB)
 constexpr int PF_EW = 8;                    // epilogue warps
 constexpr int PF_GW = 4;                    // gather warps
 constexpr int PF_THREADS = 96 + 32 * (PF_EW + PF_GW);  // TMA, MMA, relay, epilogue and gather warps
 constexpr int PF_STG = 32 * 64;             // store staging per epilogue warp: 32 rows x 64 bytes
-constexpr int PF_NBARS = 4 * PF_STAGES + 5;
-constexpr size_t PF_SMEM = 1024 + static_cast<size_t>(PF_STAGES) * 2 * PF_HALF + PF_EW * PF_STG + PF_NBARS * 8 +
+constexpr int PF_NBARS = 3 * PF_NB + 2 * PF_NA + 5;
+constexpr size_t PF_SMEM = 1024 + static_cast<size_t>(PF_NA + PF_NB) * PF_HALF + PF_EW * PF_STG + PF_NBARS * 8 +
                            2 * (DECOMOE_MAX_E + 1) * 4 + 16;
 static_assert(PF_SMEM <= 232448, "shared memory budget");
 static_assert(PF_SMEM > 232448 / 2, "one CTA per SM: the dependency waits need every CTA resident");
@@ -88,23 +94,17 @@ __device__ __forceinline__ void mbar_arrive_rank(uint32_t bar, uint32_t rank) {
       "r"(rank)
       : "memory");
 }
-// mbar_wait for a warp with time to spare: one lane tests, and sleeps in
-// between. Tests read shared memory, whose bandwidth the products need.
+// mbar_wait of a whole warp with time to spare: it sleeps between tests (they
+// read shared memory, whose bandwidth the products need).
 __device__ __forceinline__ bool mbar_wait_idle(uint32_t bar, uint32_t parity, uint64_t limit_ns, volatile int* abort,
                                                uint32_t sleep_ns) {
-  bool ok = true;
-  if ((threadIdx.x & 31) == 0 && !mbar_try_wait(bar, parity)) {
-    const uint64_t t0 = globaltimer_ns();
-    while (true) {
-      __nanosleep(sleep_ns);
-      if (mbar_try_wait(bar, parity)) break;
-      if (*abort || globaltimer_ns() - t0 > limit_ns) {
-        ok = false;
-        break;
-      }
-    }
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const uint64_t t0 = globaltimer_ns();
+  while (true) {
+    __nanosleep(sleep_ns);
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if (__any_sync(0xffffffffu, *abort != 0 || globaltimer_ns() - t0 > limit_ns)) return false;
   }
-  return __shfl_sync(0xffffffffu, ok, 0);
 }
 __device__ __forceinline__ void tc2_mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                             uint32_t accumulate) {
@@ -143,8 +143,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
   const uint32_t pad = (1024u - (raw & 1023u)) & 1023u;  // the same in both CTAs: one kernel, one layout
   uint8_t* smem = smem_raw + pad;
   const uint32_t sA = raw + pad;
-  const uint32_t sB = sA + PF_STAGES * PF_HALF;
-  uint8_t* stg = smem + 2 * PF_STAGES * PF_HALF;
+  const uint32_t sB = sA + PF_NA * PF_HALF;
+  uint8_t* stg = smem + (PF_NA + PF_NB) * PF_HALF;
   uint64_t* bars = reinterpret_cast<uint64_t*>(stg + PF_EW * PF_STG);
   int* s_off = reinterpret_cast<int*>(bars + PF_NBARS);
   int* s_mt = s_off + (DECOMOE_MAX_E + 1);
@@ -154,22 +154,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
   const uint32_t bar0 = smem_u32(bars);
-  auto FULL = [&](int s) { return bar0 + 8u * s; };                      // TMA loads of this CTA
-  auto ROWS = [&](int s) { return bar0 + 8u * (PF_STAGES + s); };        // gathered rows of this CTA
-  auto LOADED = [&](int s) { return bar0 + 8u * (2 * PF_STAGES + s); };  // CTA 0: the stage is loaded in both CTAs
-  auto EMPTY = [&](int s) { return bar0 + 8u * (3 * PF_STAGES + s); };   // products have read the stage
-  auto TFULL = [&](int a) { return bar0 + 8u * (4 * PF_STAGES + a); };
-  auto TEMPTY = [&](int a) { return bar0 + 8u * (4 * PF_STAGES + 2 + a); };  // CTA 0: both epilogues are done
-  const uint32_t DRAIN = bar0 + 8u * (4 * PF_STAGES + 4);
+  // k-block c (counted over the CTA's items) has its weights in slot c % PF_NB
+  // and its rows in slot c % PF_NA
+  auto FULLB = [&](int s) { return bar0 + 8u * s; };                     // weights loaded (this CTA)
+  auto LOADED = [&](int s) { return bar0 + 8u * (PF_NB + s); };          // CTA 0: the k-block is loaded in both CTAs
+  auto EMPTY = [&](int s) { return bar0 + 8u * (2 * PF_NB + s); };       // products have read the k-block of weight slot s
+  auto FULLA = [&](int s) { return bar0 + 8u * (3 * PF_NB + s); };       // rows loaded by TMA (this CTA)
+  auto ROWS = [&](int s) { return bar0 + 8u * (3 * PF_NB + PF_NA + s); };  // rows gathered (this CTA)
+  auto TFULL = [&](int a) { return bar0 + 8u * (3 * PF_NB + 2 * PF_NA + a); };
+  auto TEMPTY = [&](int a) { return bar0 + 8u * (3 * PF_NB + 2 * PF_NA + 2 + a); };  // CTA 0: both epilogues are done
+  const uint32_t DRAIN = bar0 + 8u * (3 * PF_NB + 2 * PF_NA + 4);
 
   const int G = g.G;
   if (threadIdx.x == 0) {
     *s_abort = 0;
-    for (int s = 0; s < PF_STAGES; ++s) {
-      mbar_init(FULL(s), 1);
-      mbar_init(ROWS(s), 32 * PF_GW);
+    for (int s = 0; s < PF_NB; ++s) {
+      mbar_init(FULLB(s), 1);
       mbar_init(LOADED(s), 2);
       mbar_init(EMPTY(s), 1);
+    }
+    for (int s = 0; s < PF_NA; ++s) {
+      mbar_init(FULLA(s), 1);
+      mbar_init(ROWS(s), 32 * PF_GW);
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(TFULL(a), 1);
@@ -250,107 +256,49 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
   const bool dep = g.gu && g.dn;  // down tiles wait for the gate/up tiles of this launch
 
   if (warp == 0) {
-    // ------------------------------------------------ TMA producer (lane 0)
+    // ------------------------------------------------ weights by TMA (lane 0)
     if (lane == 0) {
-      tma_prefetch_desc(&tma_a1);
       tma_prefetch_desc(&tma_b1);
-      tma_prefetch_desc(&tma_a2);
       tma_prefetch_desc(&tma_b2);
       int stage = 0;
       uint32_t ph = 0;
       bool ok = true;
       uint32_t armed = 0, armed_ph = 0;
-      // readiness of this CTA's rows of a down item, acquire-loaded one item ahead
-      auto flag_of = [&](int t) -> int {
-        if (!dep || t < total1 || t >= total) return 0;
-        const Item it = item(t);
-        return ld_acquire_gpu(g.ready + 2 * it.mtg + rank);
-      };
-      int flag_next = flag_of(cid);
       const uint64_t pol_once = policy_evict_first();
       for (int t = cid; ok && t < total; t += ncl) {
         const Item it = item(t);
-        const int flag = flag_next;
-        flag_next = flag_of(t + ncl);
-        const CUtensorMap* ta = it.half ? (it.dn ? &tma_a2s : &tma_a1s) : (it.dn ? &tma_a2 : &tma_a1);
         const CUtensorMap* tb = it.dn ? &tma_b2 : &tma_b1;
         const int brow = it.grp * (it.dn ? g.d : 2 * g.m) + it.nb * PF_BN + static_cast<int>(rank) * 128;
         const int KB = (it.dn ? g.m : g.d) / PF_BK;
-        const bool load_a = it.nrow > 0 && (it.dn || !gather);
-        const uint32_t bytes = PF_HALF + (load_a ? (it.half ? PF_HALF / 2 : PF_HALF) : 0);
         // weights that one row tile reads go to L2 as evict-first
         const bool once = s_mt[it.grp + 1] - s_mt[it.grp] == 1;
-        auto arm_b = [&](int kb) -> bool {  // waits for the stage, arms it and requests its weights
-          if (!mbar_wait(EMPTY(stage), ph ^ 1u, g.limit_ns, s_abort)) return false;
-          mbar_arrive_expect_tx(FULL(stage), bytes);
-          if (once)
-            tma_load_2d_hint(sB + stage * PF_HALF, tb, FULL(stage), kb * PF_BK, brow, pol_once);
-          else
-            tma_load_2d(sB + stage * PF_HALF, tb, FULL(stage), kb * PF_BK, brow);
-          armed |= 1u << stage;
-          armed_ph = (armed_ph & ~(1u << stage)) | (ph << stage);
-          return true;
-        };
-        auto next = [&]() {
-          if (++stage == PF_STAGES) {
-            stage = 0;
-            ph ^= 1u;
-          }
-        };
-        int pre = 0;  // k-blocks whose weights go out before the dependency is met
-        if (it.dn && dep && load_a) {
-          if (flag >= NT1) {
-            fence_proxy_async_all();  // h written by generic stores, read through TMA
-          } else {
-            pre = KB < PF_STAGES ? KB : PF_STAGES;
-            const int st0 = stage;
-            int got = 0;
-            for (; got < pre; ++got) {
-              if (!arm_b(got)) {
-                ok = false;
-                break;
-              }
-              next();
-            }
-            if (ok) {
-              const volatile int32_t* rp = g.ready + 2 * it.mtg + rank;
-              const uint64_t t0 = globaltimer_ns();
-              while (*rp < NT1) {
-                if (*s_abort || globaltimer_ns() - t0 > g.limit_ns) {
-                  ok = false;
-                  break;
-                }
-              }
-              __threadfence();
-              fence_proxy_async_all();
-            }
-            // the rows of the armed stages; after a timeout too, so that every
-            // armed barrier completes and can be waited for
-            int st = st0;
-            for (int kb = 0; kb < got; ++kb) {
-              tma_load_2d(sA + st * PF_HALF, ta, FULL(st), kb * PF_BK, it.row0);
-              if (++st == PF_STAGES) st = 0;
-            }
-          }
-        }
-        for (int kb = pre; ok && kb < KB; ++kb) {
-          if (!arm_b(kb)) {
+        for (int kb = 0; kb < KB; ++kb) {
+          if (!mbar_wait(EMPTY(stage), ph ^ 1u, g.limit_ns, s_abort)) {
             ok = false;
             break;
           }
-          if (load_a) tma_load_2d(sA + stage * PF_HALF, ta, FULL(stage), kb * PF_BK, it.row0);
-          next();
+          mbar_arrive_expect_tx(FULLB(stage), PF_HALF);
+          if (once)
+            tma_load_2d_hint(sB + stage * PF_HALF, tb, FULLB(stage), kb * PF_BK, brow, pol_once);
+          else
+            tma_load_2d(sB + stage * PF_HALF, tb, FULLB(stage), kb * PF_BK, brow);
+          armed |= 1u << stage;
+          armed_ph = (armed_ph & ~(1u << stage)) | (ph << stage);
+          if (++stage == PF_NB) {
+            stage = 0;
+            ph ^= 1u;
+          }
         }
       }
       int no_abort = 0;
       if (!ok) {
         *s_abort = 1;
         report_status(g.status, DECOMOE_ERR_TIMEOUT);
-        for (int s = 0; s < PF_STAGES; ++s)
-          if ((armed >> s) & 1u) mbar_wait(FULL(s), (armed_ph >> s) & 1u, g.limit_ns, &no_abort);
+        for (int s = 0; s < PF_NB; ++s)
+          if ((armed >> s) & 1u) mbar_wait(FULLB(s), (armed_ph >> s) & 1u, g.limit_ns, &no_abort);
       } else {
         // the last products' arrivals land here before the CTA may leave
-        for (int s = 0; s < PF_STAGES; ++s)
+        for (int s = 0; s < PF_NB; ++s)
           if ((armed >> s) & 1u) mbar_wait(EMPTY(s), (armed_ph >> s) & 1u, g.limit_ns, s_abort);
       }
     }
@@ -362,7 +310,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
       // products each, what this loop spends between them is lost.
       const bool leader = elect_one();
       const uint64_t ad0 = smem_desc_kmajor<PF_BK>(sA), bd0 = smem_desc_kmajor<PF_BK>(sB);
-      int stage = 0;
+      int stage = 0, rows = 0;  // weight slot, row slot
       uint32_t ph = 0;
       bool ok = true, issued = false;
       int n = 0;
@@ -382,7 +330,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
             break;
           }
           tc_fence_after();
-          const uint64_t ad = ad0 + static_cast<uint32_t>(stage * (PF_HALF >> 4));
+          const uint64_t ad = ad0 + static_cast<uint32_t>(rows * (PF_HALF >> 4));
           const uint64_t bd = bd0 + static_cast<uint32_t>(stage * (PF_HALF >> 4));
           if (leader) {
             tc2_mma_f16(dt, ad, bd, idesc, kb != 0 ? 1u : 0u);
@@ -393,7 +341,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
           }
           if (kb == 0) half_next = t + ncl < total && item(t + ncl).half;  // while the products run
           issued = true;
-          if (++stage == PF_STAGES) {
+          if (++rows == PF_NA) rows = 0;
+          if (++stage == PF_NB) {
             stage = 0;
             ph ^= 1u;
           }
@@ -414,24 +363,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
     // ------------------------------------------------ relay: this CTA's part of
     // each k-block is in shared memory
     if (lane == 0) {
-      int stage = 0;
-      uint32_t ph = 0;
+      uint32_t b = 0, a = 0, pb = 0;  // weight slot, row slot, the weight ring's phase
+      uint32_t pt = 0, pg = 0;        // phase per row slot: rows by TMA, gathered
       bool ok = true;
       for (int t = cid; ok && t < total; t += ncl) {
         const bool rows = gather && t < total1;
         const int KB = (t >= total1 ? g.m : g.d) / PF_BK;
         for (int kb = 0; kb < KB; ++kb) {
-          if (!mbar_wait(FULL(stage), ph, g.limit_ns, s_abort) ||
-              (rows && !mbar_wait(ROWS(stage), ph, g.limit_ns, s_abort))) {
+          if (!mbar_wait(FULLB(b), pb, g.limit_ns, s_abort) ||
+              !(rows ? mbar_wait(ROWS(a), pg >> a & 1u, g.limit_ns, s_abort)
+                     : mbar_wait(FULLA(a), pt >> a & 1u, g.limit_ns, s_abort))) {
             ok = false;
             break;
           }
-          if (rows) fence_proxy_async_smem();  // cp.async rows, read by the tensor cores
-          mbar_arrive_rank(LOADED(stage), 0);
-          if (++stage == PF_STAGES) {
-            stage = 0;
-            ph ^= 1u;
+          if (rows) {
+            fence_proxy_async_smem();  // cp.async rows, read by the tensor cores
+            pg ^= 1u << a;
+          } else {
+            pt ^= 1u << a;
           }
+          mbar_arrive_rank(LOADED(b), 0);
+          if (++a == PF_NA) a = 0;
+          if (++b == PF_NB) b = 0, pb ^= 1u;
         }
       }
       if (!ok) {
@@ -529,35 +482,49 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
       *s_abort = 1;
       report_status(g.status, DECOMOE_ERR_TIMEOUT);
     }
-  } else if (gather && warp < 2 + PF_EW + PF_GW) {
-    // ------------------------------------------------ row gather (gate/up items)
-    // eight lanes take one row's 128 bytes of the k-block, four rows per copy
+  } else {
+    // ------------------------------------------------ rows: gate/up items by
+    // index (four warps; eight lanes take one row's 128 bytes of the k-block,
+    // four rows per copy), grouped rows and h by TMA (one thread)
     const int gw = warp - 2 - PF_EW;
-    const int sub = lane >> 3, c = lane & 7;
-    int stage = 0;
-    uint32_t ph = 0;
+    // k-block c takes row slot a once the products of k-block c - PF_NA are
+    // done, which the barrier of that one's weight slot eb says. It cannot be a
+    // phase ahead of this wait: that would need k-block c's products.
+    uint32_t a = 0, eb = 0, pe = 0;
+    int unused = PF_NA;  // slots not taken yet
+    auto slot_next = [&]() {
+      if (++a == PF_NA) a = 0;
+      if (unused > 0) {
+        --unused;
+      } else if (++eb == PF_NB) {
+        eb = 0;
+        pe ^= 1u;
+      }
+    };
     bool ok = true;
-    for (int t = cid; ok && t < total1; t += ncl) {
+    int t = cid;
+    for (; gather && ok && t < total1; t += ncl) {
       const Item it = item(t);
+      const int sub = lane >> 3, ch = lane & 7;
       const uint8_t* src[8];
       uint32_t dst[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int r = 32 * gw + 4 * i + sub;
         const int tok = r < it.nrow ? g.perm[it.row0 + r] : -1;
-        src[i] = tok >= 0 ? g.x + (static_cast<int64_t>(tok) * g.d + 8 * c) * 2 : nullptr;
-        dst[i] = sA + r * 128 + ((c ^ (r & 7)) << 4);
+        src[i] = tok >= 0 ? g.x + (static_cast<int64_t>(tok) * g.d + 8 * ch) * 2 : nullptr;
+        dst[i] = sA + r * 128 + ((ch ^ (r & 7)) << 4);
       }
       const int KB = g.d / PF_BK;
-      for (int kb = 0; kb < KB; ++kb) {
-        if (!mbar_wait_idle(EMPTY(stage), ph ^ 1u, g.limit_ns, s_abort, 20)) {
+      for (int kb = 0; kb < KB; ++kb, slot_next()) {
+        if (unused == 0 && !mbar_wait_idle(EMPTY(eb), pe, g.limit_ns, s_abort, 20)) {
           ok = false;
           break;
         }
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-          if (src[i] != nullptr) cp_async16(dst[i] + stage * PF_HALF, src[i] + kb * (PF_BK * 2));
-        cp_async_mbar_arrive_noinc(ROWS(stage));
+          if (src[i] != nullptr) cp_async16(dst[i] + a * PF_HALF, src[i] + kb * (PF_BK * 2));
+        cp_async_mbar_arrive_noinc(ROWS(a));
         if (g.x_copy != nullptr && it.nb == 0) {  // one of the row tile's items also leaves the rows behind
           uint4 v[8];
 #pragma unroll
@@ -567,15 +534,65 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
           for (int i = 0; i < 8; ++i)
             if (src[i] != nullptr)
               *reinterpret_cast<uint4*>(g.x_copy + static_cast<int64_t>(it.row0 + 32 * gw + 4 * i + sub) * g.d * 2 +
-                                        kb * (PF_BK * 2) + 16 * c) = v[i];
-        }
-        if (++stage == PF_STAGES) {
-          stage = 0;
-          ph ^= 1u;
+                                        kb * (PF_BK * 2) + 16 * ch) = v[i];
         }
       }
     }
     cp_async_wait_all();
+    if (ok && gw == 0 && lane == 0) {
+      tma_prefetch_desc(&tma_a1);
+      tma_prefetch_desc(&tma_a2);
+      uint32_t armed = 0, pt = 0;  // slots with a copy in flight; phase per slot
+      // readiness of this CTA's rows of a down item, acquire-loaded one item ahead
+      auto flag_of = [&](int i) -> int {
+        if (!dep || i < total1 || i >= total) return 0;
+        return ld_acquire_gpu(g.ready + 2 * item(i).mtg + rank);
+      };
+      int flag_next = flag_of(t);
+      for (; ok && t < total; t += ncl) {
+        const Item it = item(t);
+        const int flag = flag_next;
+        flag_next = flag_of(t + ncl);
+        const CUtensorMap* ta = it.half ? (it.dn ? &tma_a2s : &tma_a1s) : (it.dn ? &tma_a2 : &tma_a1);
+        const uint32_t bytes = it.half ? PF_HALF / 2 : PF_HALF;
+        const int KB = (it.dn ? g.m : g.d) / PF_BK;
+        if (it.dn && dep && it.nrow > 0) {
+          // h of these rows: every gate/up tile of theirs has stored it
+          if (flag < NT1) {
+            const volatile int32_t* rp = g.ready + 2 * it.mtg + rank;
+            const uint64_t t0 = globaltimer_ns();
+            while (*rp < NT1) {
+              if (*s_abort || globaltimer_ns() - t0 > g.limit_ns) {
+                ok = false;
+                break;
+              }
+            }
+            if (!ok) break;
+            __threadfence();
+          }
+          fence_proxy_async_all();  // written by generic stores, read through TMA
+        }
+        for (int kb = 0; kb < KB; ++kb, slot_next()) {
+          if (unused == 0 && !mbar_wait(EMPTY(eb), pe, g.limit_ns, s_abort)) {
+            ok = false;
+            break;
+          }
+          if (it.nrow > 0) {
+            mbar_arrive_expect_tx(FULLA(a), bytes);
+            tma_load_2d(sA + a * PF_HALF, ta, FULLA(a), kb * PF_BK, it.row0);
+            armed |= 1u << a;
+          } else {
+            mbar_arrive(FULLA(a));  // no rows of this CTA in the tile
+            armed &= ~(1u << a);
+          }
+          pt ^= 1u << a;
+        }
+      }
+      int no_abort = 0;
+      if (!ok)
+        for (int s = 0; s < PF_NA; ++s)
+          if ((armed >> s) & 1u) mbar_wait(FULLA(s), ~(pt >> s) & 1u, g.limit_ns, &no_abort);
+    }
     if (!ok) {
       *s_abort = 1;
       report_status(g.status, DECOMOE_ERR_TIMEOUT);
