@@ -599,7 +599,7 @@ __global__ void __launch_bounds__(DL_THREADS, 1)
       }
       float my_v;
       int my_i;
-      warp_topk(v, lim, k, lane, my_v, my_i);
+      warp_topk_n<8>(v, lim, k, lane, my_v, my_i);
       if (g.want_mass) {
         const float wf = pick_weight(my_v, lane, k);
         if (lane < k) {
@@ -607,7 +607,7 @@ __global__ void __launch_bounds__(DL_THREADS, 1)
           g_fpw[t * k + lane] = wf;
         }
         const bool inside = __all_sync(0xffffffffu, lane >= k || my_i < g.K_fixed);
-        if (!inside) warp_topk(v, g.K_fixed, k, lane, my_v, my_i);
+        if (!inside) warp_topk_n<8>(v, g.K_fixed, k, lane, my_v, my_i);
       }
       const float w = pick_weight(my_v, lane, k);
       if (lane < k) {

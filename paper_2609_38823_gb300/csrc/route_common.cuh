@@ -83,11 +83,6 @@ __device__ __forceinline__ void warp_topk_n(const uint32_t (&key_in)[NSL], int l
   }
 }
 
-__device__ __forceinline__ void warp_topk(const uint32_t (&key_in)[8], int lim, int k, int lane, float& my_v,
-                                          int& my_i) {
-  warp_topk_n<8>(key_in, lim, k, lane, my_v, my_i);
-}
-
 // Renormalised weight of this lane's pick (lanes >= k get 0).
 __device__ __forceinline__ float pick_weight(float my_v, int lane, int k) {
   const float v0 = __shfl_sync(0xffffffffu, my_v, 0);
