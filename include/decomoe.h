@@ -519,7 +519,8 @@ DECOMOE_API int decomoe_moe_layer_exit(const void* x, const void* w_r, const flo
  * for inspection: logits, topk_idx, topk_w, mass, counts, offsets, perm_token,
  * inv_slot, x_perm, h, y_perm, device K (12 entries written to offs_host).
  * The layer's scratch rows are dropped from L2 after their last read, and
- * above 8*K routed rows x_perm is not made (see decomoe_set_discard_scratch):
+ * x_perm is not made where the experts read x by index (above 8*K routed rows,
+ * and in fp32; see decomoe_set_discard_scratch):
  * turn that off before a call whose x_perm or y_perm is to be inspected. */
 DECOMOE_API int decomoe_moe_layer_workspace_layout(int64_t T, int d, int E, int k, int m, int dtype,
                                        size_t* offs_host);
@@ -585,8 +586,8 @@ DECOMOE_API int decomoe_selftest_wait(int32_t* status_dev, int64_t limit_ns, dec
  * decomoe_moe_layer_exit drop the L2 lines of their workspace's y_perm rows
  * once the combine has read them (discard.global.L2): the rows are not
  * written back to HBM, and the next layer's writes find clean lines to
- * evict; and where the experts read x by index (more than 8*K routed rows) the
- * grouped copy x_perm is not written. Those workspace rows are undefined after
+ * evict; and where the experts read x by index (more than 8*K routed rows, and
+ * fp32) the grouped copy x_perm is not written. Those workspace rows are undefined after
  * the call. on == 0 makes and keeps them (for inspection). Process-wide;
  * applies to later calls.
  * ------------------------------------------------------------------------ */
