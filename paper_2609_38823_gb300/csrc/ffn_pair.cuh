@@ -503,27 +503,42 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
     };
     bool ok = true;
     int t = cid;
-    for (; gather && ok && t < total1; t += ncl) {
-      const Item it = item(t);
-      const int sub = lane >> 3, ch = lane & 7;
-      const uint8_t* src[8];
-      uint32_t dst[8];
+    const int sub = lane >> 3, ch = lane & 7;
+    // an item's rows and tokens are looked up half an item ahead: the ring holds
+    // less time than that chain of loads takes (gate/up by index 1559 -> 1660
+    // TFLOP/s with weights in L2, T = 16384 1023 -> 1000 us a layer)
+    Item it = item(t), it_next = it;
+    int tok[8];
+    auto tokens = [&](const Item& i2, bool any) {
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int r = 32 * gw + 4 * i + sub;
-        const int tok = r < it.nrow ? g.perm[it.row0 + r] : -1;
-        src[i] = tok >= 0 ? g.x + (static_cast<int64_t>(tok) * g.d + 8 * ch) * 2 : nullptr;
-        dst[i] = sA + r * 128 + ((ch ^ (r & 7)) << 4);
+        tok[i] = any && r < i2.nrow ? g.perm[i2.row0 + r] : -1;
       }
+    };
+    if (gather && t < total1) tokens(it, true);
+    for (; gather && ok && t < total1; t += ncl) {
+      it = it_next;
+      const uint8_t* src[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        src[i] = tok[i] >= 0 ? g.x + (static_cast<int64_t>(tok[i]) * g.d + 8 * ch) * 2 : nullptr;
       const int KB = g.d / PF_BK;
       for (int kb = 0; kb < KB; ++kb, slot_next()) {
+        if (kb == KB / 2 && t + ncl < total) {
+          it_next = item(t + ncl);
+          tokens(it_next, t + ncl < total1);
+        }
         if (unused == 0 && !mbar_wait_idle(EMPTY(eb), pe, g.limit_ns, s_abort, 20)) {
           ok = false;
           break;
         }
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-          if (src[i] != nullptr) cp_async16(dst[i] + a * PF_HALF, src[i] + kb * (PF_BK * 2));
+          if (src[i] != nullptr) {
+            const int r = 32 * gw + 4 * i + sub;
+            cp_async16(sA + a * PF_HALF + r * 128 + ((ch ^ (r & 7)) << 4), src[i] + kb * (PF_BK * 2));
+          }
         cp_async_mbar_arrive_noinc(ROWS(a));
         if (g.x_copy != nullptr && it.nb == 0) {  // one of the row tile's items also leaves the rows behind
           uint4 v[8];
@@ -543,36 +558,39 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
       tma_prefetch_desc(&tma_a1);
       tma_prefetch_desc(&tma_a2);
       uint32_t armed = 0, pt = 0;  // slots with a copy in flight; phase per slot
-      // readiness of this CTA's rows of a down item, acquire-loaded one item ahead
-      auto flag_of = [&](int i) -> int {
-        if (!dep || i < total1 || i >= total) return 0;
-        return ld_acquire_gpu(g.ready + 2 * item(i).mtg + rank);
+      // readiness of this CTA's rows of a down item, acquire-loaded one item
+      // ahead (an acquire holds up the thread's later loads)
+      auto ready_of = [&](const Item& i2) -> bool {
+        if (!(dep && i2.dn && i2.nrow > 0)) return true;
+        if (ld_acquire_gpu(g.ready + 2 * i2.mtg + rank) < NT1) return false;
+        fence_proxy_async_all();  // h, written by generic stores, is read through TMA
+        return true;
       };
-      int flag_next = flag_of(t);
+      bool ready_next = t < total ? ready_of(it_next) : true;
       for (; ok && t < total; t += ncl) {
-        const Item it = item(t);
-        const int flag = flag_next;
-        flag_next = flag_of(t + ncl);
+        it = it_next;
+        const bool ready = ready_next;
         const CUtensorMap* ta = it.half ? (it.dn ? &tma_a2s : &tma_a1s) : (it.dn ? &tma_a2 : &tma_a1);
         const uint32_t bytes = it.half ? PF_HALF / 2 : PF_HALF;
         const int KB = (it.dn ? g.m : g.d) / PF_BK;
-        if (it.dn && dep && it.nrow > 0) {
-          // h of these rows: every gate/up tile of theirs has stored it
-          if (flag < NT1) {
-            const volatile int32_t* rp = g.ready + 2 * it.mtg + rank;
-            const uint64_t t0 = globaltimer_ns();
-            while (*rp < NT1) {
-              if (*s_abort || globaltimer_ns() - t0 > g.limit_ns) {
-                ok = false;
-                break;
-              }
+        if (!ready) {  // wait until every gate/up tile of these rows has stored its h
+          const volatile int32_t* rp = g.ready + 2 * it.mtg + rank;
+          const uint64_t t0 = globaltimer_ns();
+          while (*rp < NT1) {
+            if (*s_abort || globaltimer_ns() - t0 > g.limit_ns) {
+              ok = false;
+              break;
             }
-            if (!ok) break;
-            __threadfence();
           }
-          fence_proxy_async_all();  // written by generic stores, read through TMA
+          if (!ok) break;
+          __threadfence();
+          fence_proxy_async_all();
         }
         for (int kb = 0; kb < KB; ++kb, slot_next()) {
+          if (kb == 0 && t + ncl < total) {
+            it_next = item(t + ncl);
+            ready_next = ready_of(it_next);
+          }
           if (unused == 0 && !mbar_wait(EMPTY(eb), pe, g.limit_ns, s_abort)) {
             ok = false;
             break;
