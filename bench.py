@@ -855,7 +855,7 @@ def run_isolated(dm, ws, pk, only=None, steps=10, warmup=3, att_len=0):
                 ms = timed_ev(lambda: dm.decomoe_attention(q, kc, vc, o, aws))
                 fl = 2.0 * Hq * Dh * S * (S + 1)
                 tf = fl / (ms * 1e-3) / 1e12
-                out.append({"mode": f"isolated attention prefill, {name}, {kind}", "kernel": "k_attn_vt + k_attn_prefill",
+                out.append({"mode": f"isolated attention prefill, {name}, {kind}", "kernel": "k_attn_prefill",
                             "shape": f"q [{S}, 32, 128], K and V [{S}, 4, 128] bf16", "ms": round(ms, 4),
                             "algo_flops": fl, "tflops": round(tf, 1),
                             "tensor_frac": round(tf / pk["bf16_tflops"], 4)})

@@ -32,11 +32,11 @@
 // weight stream. The MMA warp's loop decides: issued by one thread of a divergent
 // branch with two barriers per k-block, the same kernel took 637 cycles per
 // k-block (gate/up 1576 TFLOP/s) instead of 512, and an arrival with cluster
-// release 1900. Layer against the one-SM kernels: T = 2048, K = 64 222 -> 192 us;
-// 4096 361 -> 295; 16384, K = 128 1237 -> 1027; 1552, K = 128 237 -> 219; 272, K =
-// 57 114 -> 105; 131, K = 64 97.6 -> 91.5. One ring for both operands: 199, 301,
-// 1037, 228, 109, 93.7. Eight slots for weights and four for rows: 196, 307, 1098,
-// 219, 106, 92.1 (gate/up in L2 1654 TFLOP/s instead of 1805).
+// release 1900. Layer against the one-SM kernels: T = 2048, K = 64 222 -> 187 us;
+// 4096 361 -> 282; 16384, K = 128 1237 -> 976; 1552, K = 128 237 -> 216; 272, K =
+// 57 114 -> 106; 131, K = 64 97.6 -> 91.3. With one ring for both operands it had
+// been 199, 301, 1037, 228, 109 and 93.7; with eight slots for weights and four
+// for rows gate/up from L2 ran at 1654 TFLOP/s instead of 1805.
 #pragma once
 
 namespace decomoe {
@@ -402,6 +402,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
     for (int t = cid; t < total; t += ncl, ++n) {
       const Item it = item(t);
       const int acc = n & 1;
+      if (g.x_copy != nullptr && !it.dn) {
+        // the grouped rows are wanted too: this item's share (rows dealt over
+        // the row tile's gate/up items), while its accumulator is computed
+        const int vec = g.d / 8, per = (it.nrow + NT1 - 1) / NT1;
+        const int a = min(it.nb * per, it.nrow), nv = (min(a + per, it.nrow) - a) * vec;
+        for (int i0 = threadIdx.x - 64; i0 < nv; i0 += 32 * PF_EW * 4) {
+          uint4 v[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int i = i0 + u * 32 * PF_EW;
+            if (i < nv)
+              v[u] = __ldg(reinterpret_cast<const uint4*>(g.x) +
+                           static_cast<int64_t>(g.perm[it.row0 + a + i / vec]) * vec + i % vec);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int i = i0 + u * 32 * PF_EW;
+            if (i < nv) reinterpret_cast<uint4*>(g.x_copy)[(static_cast<int64_t>(it.row0) + a) * vec + i] = v[u];
+          }
+        }
+        __syncwarp();
+      }
       if (!mbar_wait_idle(TFULL(acc), (n >> 1) & 1, g.limit_ns, s_abort, 100)) {
         ok = false;
         break;
@@ -540,17 +562,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
             cp_async16(sA + a * PF_HALF + r * 128 + ((ch ^ (r & 7)) << 4), src[i] + kb * (PF_BK * 2));
           }
         cp_async_mbar_arrive_noinc(ROWS(a));
-        if (g.x_copy != nullptr && it.nb == 0) {  // one of the row tile's items also leaves the rows behind
-          uint4 v[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            if (src[i] != nullptr) v[i] = __ldg(reinterpret_cast<const uint4*>(src[i] + kb * (PF_BK * 2)));
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            if (src[i] != nullptr)
-              *reinterpret_cast<uint4*>(g.x_copy + static_cast<int64_t>(it.row0 + 32 * gw + 4 * i + sub) * g.d * 2 +
-                                        kb * (PF_BK * 2) + 16 * ch) = v[i];
-        }
       }
     }
     cp_async_wait_all();
