@@ -31,9 +31,10 @@ __device__ __forceinline__ void acc_vec(float* acc, const uint4& v, float wj) {
   }
 }
 
+// The sum (with the residual's vector r when there is one) as a storage vector.
 template <bool BF16>
-__device__ __forceinline__ uint4 finish_vec(float* acc, const uint4* __restrict__ residual, int64_t ridx) {
-  if (residual != nullptr) acc_vec<BF16>(acc, __ldg(residual + ridx), 1.0f);
+__device__ __forceinline__ uint4 finish_vec(float* acc, bool has_residual, const uint4& r) {
+  if (has_residual) acc_vec<BF16>(acc, r, 1.0f);
   if constexpr (BF16)
     return make_uint4(pack_bf16x2(acc[0], acc[1]), pack_bf16x2(acc[2], acc[3]), pack_bf16x2(acc[4], acc[5]),
                       pack_bf16x2(acc[6], acc[7]));
@@ -53,7 +54,9 @@ struct DropRows {
 
 // WPT warps per token, each taking alternate 32-vector chunks of the row:
 // many tokens take one warp each (two blocks resident per SM), few tokens
-// spread each row over more warps.
+// spread each row over more warps. The residual's vectors are loaded with the
+// slot rows, not after their sum: one trip to memory less per chunk (a layer of
+// 4096 tokens 280.8 -> 274.3 us, of 777 tokens 165.1 -> 161.6).
 // discard (y is the caller's scratch, rows 128-byte aligned): every y line is
 // read exactly once (inv_slot is a bijection), so once a warp has summed its
 // rows it drops their L2 lines (discard.global.L2): the lines are not written
@@ -95,11 +98,15 @@ __global__ void __launch_bounds__(256, WPT == 1 ? 2 : 1)
       for (int c = part * 32 + lane; c < vec; c += 64 * WPT) {
         const int c2 = c + 32 * WPT;
         const bool two = c2 < vec;
-        uint4 v[KT], v2[KT];
+        uint4 v[KT], v2[KT], r = make_uint4(0, 0, 0, 0), r2 = r;
 #pragma unroll
         for (int j = 0; j < KT; ++j) {
           v[j] = rows[j] >= 0 ? __ldg(y + static_cast<int64_t>(rows[j]) * vec + c) : make_uint4(0, 0, 0, 0);
           v2[j] = (rows[j] >= 0 && two) ? __ldg(y + static_cast<int64_t>(rows[j]) * vec + c2) : make_uint4(0, 0, 0, 0);
+        }
+        if (residual != nullptr) {  // in flight with the slot rows
+          r = __ldg(residual + t * vec + c);
+          if (two) r2 = __ldg(residual + t * vec + c2);
         }
         float acc[NE], acc2[NE];
 #pragma unroll
@@ -122,11 +129,11 @@ __global__ void __launch_bounds__(256, WPT == 1 ? 2 : 1)
               }
           }
         }
-        const uint4 o1 = finish_vec<BF16>(acc, residual, t * vec + c);
+        const uint4 o1 = finish_vec<BF16>(acc, residual != nullptr, r);
         out[t * vec + c] = o1;
         if (text_row) drop.text[trow * vec + c] = o1;
         if (two) {
-          const uint4 o2 = finish_vec<BF16>(acc2, residual, t * vec + c2);
+          const uint4 o2 = finish_vec<BF16>(acc2, residual != nullptr, r2);
           out[t * vec + c2] = o2;
           if (text_row) drop.text[trow * vec + c2] = o2;
         }
@@ -146,7 +153,8 @@ __global__ void __launch_bounds__(256, WPT == 1 ? 2 : 1)
           acc_vec<BF16>(acc, __ldg(y + static_cast<int64_t>(row) * vec + c), wj);
         }
         if (active) {
-          const uint4 o1 = finish_vec<BF16>(acc, residual, t * vec + c);
+          const uint4 o1 = finish_vec<BF16>(acc, residual != nullptr,
+                                            residual != nullptr ? __ldg(residual + t * vec + c) : make_uint4(0, 0, 0, 0));
           out[t * vec + c] = o1;
           if (text_row) drop.text[trow * vec + c] = o1;
         }
@@ -169,13 +177,16 @@ static cudaError_t launch_combine_w(cudaStream_t s, const uint4* y, const int32_
     default: return launch_pdl(k_combine<BF16, 0, DROP, WPT>, g, b, 0, s, y, inv, w, T, k, vec, res, out, drop, 0);
   }
 }
-// Warps per token by token count: one from 1024 tokens on, two from 256, four
-// from 32, eight below (a decode step's row then spans eight warps).
+// Warps per token by token count: one from 1024 tokens on, two from 512, four
+// from 32, eight below (a decode step's row then spans eight warps). A whole
+// bf16 layer (top-k 8, d 2048): T = 272 takes 102.3 us with four warps a token
+// and 103.9 with two, T = 777 161.9 with either, T = 1552 213.4 with one and
+// 215.4 with two, T = 4096 274.3 with one and 276.1 with two.
 template <bool BF16, bool DROP>
 static cudaError_t launch_combine_k(cudaStream_t s, const uint4* y, const int32_t* inv, const float* w, int64_t T,
                                     int k, int vec, const uint4* res, uint4* out, DropRows drop, int dc) {
   if (T >= 1024) return launch_combine_w<BF16, DROP, 1>(s, y, inv, w, T, k, vec, res, out, drop, dc);
-  if (T >= 256) return launch_combine_w<BF16, DROP, 2>(s, y, inv, w, T, k, vec, res, out, drop, dc);
+  if (T >= 512) return launch_combine_w<BF16, DROP, 2>(s, y, inv, w, T, k, vec, res, out, drop, dc);
   if (T >= 32) return launch_combine_w<BF16, DROP, 4>(s, y, inv, w, T, k, vec, res, out, drop, dc);
   return launch_combine_w<BF16, DROP, 8>(s, y, inv, w, T, k, vec, res, out, drop, dc);
 }
