@@ -27,8 +27,8 @@ constexpr int ATT_PROW = ATT_D + 4;             // floats per partial row: acc[D
 // ------------------------------------------------------------------ decode sizes
 // Few queries per KV head (a decode step over the cache, or a short chunk):
 // block (split s, KV head g, query tile group z) streams keys
-// [s * kps, (s + 1) * kps) of head g through a three-chunk TMA ring of 128
-// keys (128-byte swizzled 64-feature halves; rows past C read as zero) and
+// [s * kps, (s + 1) * kps) of head g through a three-chunk TMA ring of up to
+// 128 keys each (128-byte swizzled 64-feature halves; rows past C read as zero) and
 // runs the online softmax of up to 32 of the group's
 // nq = n * Hq / Hkv queries on the tensor cores with warp-level
 // mma.m16n8k16 (bf16 in, fp32 accumulate): per 16 keys a warp computes
@@ -74,7 +74,8 @@ static_assert(ATD_WARPS * ATD_QT * 16 * (ATD_OROW + 2) * 4 <= ATD_NST * ATD_STAG
 struct AttDecArgs {
   const uint4* q;   // [n, Hq, D] (K and V [C, Hkv, D] come through the tensor maps)
   int64_t n, C;
-  int Hq, Hkv, kps; // keys per block; a cluster (grid.x) is a run of the head's splits
+  int Hq, Hkv, ck;  // keys per chunk (a multiple of 16, at most ATD_CH)
+  int kps;          // keys per block, whole chunks; a cluster (grid.x) is a run of the head's splits
   int S;            // clusters per (KV head, query tile group): grid.y = Hkv * S
   float sl2;        // scale * log2(e)
   __nv_bfloat16* out;
@@ -142,7 +143,8 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint3
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-template <int QT>
+// FULL: chunks of ATD_CH keys, else of a.ck.
+template <int QT, bool FULL>
 __global__ void __launch_bounds__(ATD_THREADS)
     k_attn_dec(const __grid_constant__ CUtensorMap tma_k, const __grid_constant__ CUtensorMap tma_v,
                const AttDecArgs a) {
@@ -165,7 +167,8 @@ __global__ void __launch_bounds__(ATD_THREADS)
   constexpr int VPR = ATT_D / 8;  // 16-byte vectors per head row
   const int64_t k0 = static_cast<int64_t>(cset * static_cast<int>(gridDim.x) + s) * a.kps;
   const int64_t k1 = k0 + a.kps < a.C ? k0 + a.kps : a.C;
-  const int nch = k1 > k0 ? static_cast<int>((k1 - k0 + ATD_CH - 1) / ATD_CH) : 0;  // a split past C: none
+  const int ck = FULL ? ATD_CH : a.ck;
+  const int nch = k1 > k0 ? (static_cast<int>(k1 - k0) + ck - 1) / ck : 0;  // a split past C: none
   if (tid == 0) {
     *s_abort = 0;
     for (int st = 0; st < ATD_NST; ++st) mbar_init(bar0 + 8u * st, 1);
@@ -185,8 +188,8 @@ __global__ void __launch_bounds__(ATD_THREADS)
   auto issue = [&](int c, int st) {
     const uint32_t bar = bar0 + 8u * st;
     const uint32_t base = sKVa + st * ATD_STAGE;
-    const int key0 = static_cast<int>(k0) + c * ATD_CH;
-    mbar_arrive_expect_tx(bar, ATD_STAGE);
+    const int key0 = static_cast<int>(k0) + c * ck;  // the maps' boxes are ck keys high
+    mbar_arrive_expect_tx(bar, static_cast<uint32_t>(ck) * (ATT_D * 4));
     tma_load_3d(base, &tma_k, bar, 0, g, key0);
     tma_load_3d(base + ATD_HALF, &tma_k, bar, 64, g, key0);
     tma_load_3d(base + 2 * ATD_HALF, &tma_v, bar, 0, g, key0);
@@ -208,6 +211,9 @@ __global__ void __launch_bounds__(ATD_THREADS)
   int issued = nch < ATD_NST ? nch : ATD_NST;  // chunks whose copies were requested (thread 0)
   if (tid == 0)
     for (int c = 0; c < issued; ++c) issue(c, c);
+  // the next launch may be scheduled now that the copies are under way (its
+  // griddepcontrol.wait still waits for this grid's completion)
+  if (a.S == 1) pdl_trigger();
   cp_async_wait_all();
   __syncthreads();  // the query rows are in place
 
@@ -237,8 +243,8 @@ __global__ void __launch_bounds__(ATD_THREADS)
     if (!ok && c_fail == nch) c_fail = c;
     const uint32_t sKa = sKVa + buf * ATD_STAGE;  // K halves; V halves follow
     const uint32_t sVa = sKa + 2 * ATD_HALF;
-    const int64_t kw = k0 + static_cast<int64_t>(c) * ATD_CH + 16 * warp;  // this warp's first key
-    if (ok && kw < k1) {
+    const int64_t kw = k0 + static_cast<int64_t>(c) * ck + 16 * warp;  // this warp's first key
+    if (ok && 16 * warp < ck && kw < k1) {
       // S = Q K^T for this warp's 16 keys (two 8-key n-tiles), per query tile
       float sc[QT][2][4];
 #pragma unroll
@@ -450,7 +456,6 @@ __global__ void __launch_bounds__(ATD_THREADS)
       }
     }
   }
-  if (a.S == 1) pdl_trigger();
 }
 
 // The S <= ATT_MAX_SETS clusters of a (KV head g = blockIdx.x, query tile
@@ -532,11 +537,32 @@ static AttPlan att_plan(int64_t C, int Hkv, int nz) {
   }
   return best;
 }
-// Keys per block, in whole chunks, for the plan's cs * S splits.
-static int64_t att_kps(int64_t C, const AttPlan& pl) {
-  const int64_t nsplit = std::max<int64_t>(1, std::min<int64_t>((C + ATD_CH - 1) / ATD_CH, pl.cs)) * pl.S;
-  int64_t kps = (C + nsplit - 1) / nsplit;
-  return (kps + ATD_CH - 1) / ATD_CH * ATD_CH;
+// Keys per chunk and per block for the plan's cs * S splits. A short cache is
+// spread over up to 12 blocks of at least 32 keys, one chunk each, before its
+// chunks grow to ATD_CH: less for each SM to copy, and rows of the merge for
+// more blocks. A block's two to four chunks are made equal in whole 16s where
+// that was measured to pay (several clusters per head, or more than 16 queries
+// per head); else, and always past four, chunks are whole, which the compiler
+// sees as a constant. 32 query heads on 4 KV heads, launches after one
+// another, 128-key chunks throughout and the next launch scheduled at the end
+// -> this: 1 query over 40 keys 5.5 -> 4.0 us, 257 keys 4.5 -> 3.6, 600 keys
+// 4.4 -> 3.6, 2049 keys 4.87 -> 4.62 (the earlier scheduling), 9000 keys 8.3 ->
+// 7.9; 8 queries over 300 keys 9.5 -> 7.4, 2049 keys 11.4 -> 10.5. Over 1000
+// keys 8, 12 and 16 blocks take 3.7, 3.8 and 3.9 us, over 600 3.7, 3.6 and 3.8;
+// equal chunks for 1 query over 3000 keys 5.0 us, whole ones 4.75.
+struct AttKeys {
+  int ck;       // keys per chunk
+  int64_t kps;  // keys per block: whole chunks
+};
+static AttKeys att_keys(int64_t C, const AttPlan& pl, int64_t nq) {
+  int64_t nsplit = (C + ATD_CH - 1) / ATD_CH;
+  nsplit = std::max<int64_t>(nsplit, std::min<int64_t>((C + 31) / 32, 12));
+  nsplit = std::max<int64_t>(1, std::min<int64_t>(nsplit, pl.cs)) * pl.S;
+  const int64_t kps = (C + nsplit - 1) / nsplit;
+  const int64_t nch = (kps + ATD_CH - 1) / ATD_CH;
+  if (nch > 1 && (nch > 4 || (nq <= 16 && pl.S == 1))) return {ATD_CH, nch * ATD_CH};
+  const int ck = static_cast<int>((kps + nch * 16 - 1) / (nch * 16)) * 16;
+  return {ck, ck * nch};
 }
 
 // Largest cluster of decode blocks this device schedules (16 where the
@@ -549,7 +575,7 @@ static int att_max_cluster() {
   if (v != 0) return v;
   v = 8;
   bool ok = true;
-  for (auto kern : {k_attn_dec<1>, k_attn_dec<2>}) {
+  for (auto kern : {k_attn_dec<1, true>, k_attn_dec<2, true>}) {
     ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(ATD_SMEM)) ==
                    cudaSuccess;
     ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
@@ -567,8 +593,8 @@ static int att_max_cluster() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n1 = 0, n2 = 0;
-    if (cudaOccupancyMaxActiveClusters(&n1, k_attn_dec<1>, &cfg) == cudaSuccess &&
-        cudaOccupancyMaxActiveClusters(&n2, k_attn_dec<2>, &cfg) == cudaSuccess && n1 >= 1 && n2 >= 1)
+    if (cudaOccupancyMaxActiveClusters(&n1, k_attn_dec<1, true>, &cfg) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&n2, k_attn_dec<2, true>, &cfg) == cudaSuccess && n1 >= 1 && n2 >= 1)
       v = 16;
   }
   cudaGetLastError();  // a refused query leaves no error behind
@@ -598,8 +624,8 @@ static int att_active_clusters(int cs) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n1 = 0, n2 = 0;
-  if (cudaOccupancyMaxActiveClusters(&n1, k_attn_dec<1>, &cfg) != cudaSuccess ||
-      cudaOccupancyMaxActiveClusters(&n2, k_attn_dec<2>, &cfg) != cudaSuccess)
+  if (cudaOccupancyMaxActiveClusters(&n1, k_attn_dec<1, true>, &cfg) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n2, k_attn_dec<2, true>, &cfg) != cudaSuccess)
     n1 = n2 = 0;
   cudaGetLastError();  // a refused query leaves no error behind
   v = std::min(n1, n2);
@@ -1372,8 +1398,10 @@ int decomoe_attention(const void* q, int64_t n, const void* k_cache, const void*
   const int nz = att_nz(nq);
   const AttPlan pl = att_plan(C, Hkv, nz);
   const int S = pl.S;
-  const int64_t kps = att_kps(C, pl);
+  const AttKeys ks = att_keys(C, pl, nq);
+  const int64_t kps = ks.kps;
   DM_ARG_CHECK(kps <= 0x7fffffffLL, "attention: C=%lld keys is too long", (long long)C);
+  a.ck = ks.ck;
   a.kps = static_cast<int>(kps);
   a.S = S;
   a.part = static_cast<float*>(ws);
@@ -1390,10 +1418,10 @@ int decomoe_attention(const void* q, int64_t n, const void* k_cache, const void*
   a.out = static_cast<__nv_bfloat16*>(out);
   a.status = status_dev;
   a.limit_ns = static_cast<uint64_t>(wait_limit_ns());
-  CUtensorMap tk, tv;  // [C][Hkv][D]: boxes of 128 keys x 64 features of one head
+  CUtensorMap tk, tv;  // [C][Hkv][D]: boxes of one chunk's keys x 64 features of one head
   const uint64_t dkv[3] = {static_cast<uint64_t>(D), static_cast<uint64_t>(Hkv), static_cast<uint64_t>(C)};
   const uint64_t skv[2] = {static_cast<uint64_t>(D) * 2, static_cast<uint64_t>(Hkv) * D * 2};
-  const uint32_t bkv[3] = {64, 1, ATD_CH};
+  const uint32_t bkv[3] = {64, 1, static_cast<uint32_t>(a.ck)};
   DM_RET(make_tmap_bf16_3d(&tk, k_cache, dkv, skv, bkv));
   DM_RET(make_tmap_bf16_3d(&tv, v_cache, dkv, skv, bkv));
   const dim3 grid(static_cast<unsigned>(nsplit), static_cast<unsigned>(Hkv * S), static_cast<unsigned>(nz));
@@ -1425,7 +1453,8 @@ int decomoe_attention(const void* q, int64_t n, const void* k_cache, const void*
                                Hq, Hkv, static_cast<__nv_bfloat16*>(out)));
     return DECOMOE_OK;
   };
-  return nq <= 16 ? go(k_attn_dec<1>) : go(k_attn_dec<2>);
+  if (a.ck == ATD_CH) return nq <= 16 ? go(k_attn_dec<1, true>) : go(k_attn_dec<2, true>);
+  return nq <= 16 ? go(k_attn_dec<1, false>) : go(k_attn_dec<2, false>);
 }
 
 }  // extern "C"

@@ -64,6 +64,20 @@ def test_attention_decode_parity(n, C):
     assert_close_out(f64(out), ref, BF16_REL_L2, BF16_MAX_ABS, f"attention n={n} C={C}")
 
 
+@pytest.mark.parametrize("n,C", [(1, 16), (1, 31), (1, 32), (1, 33), (1, 383), (1, 384), (1, 385), (2, 1535),
+                                 (1, 1536), (1, 1537), (5, 33), (5, 401), (5, 2049), (8, 3073), (1, 8200)])
+def test_attention_decode_chunk_sizes(n, C):
+    # one chunk of 16 to 128 keys in up to 12 blocks, at the steps of the rule
+    # (32 keys a block, 12 blocks, whole chunks); two and three equal chunks of
+    # fewer than 128 keys for more than 16 queries per head and, at 8200 keys,
+    # for several clusters per head
+    q, k, v = _qkv(n, C, seed=3 * C + n)
+    out = _run(q, k, v)
+    ref = O.attention(f64(q), f64(k), f64(v))
+    assert_close_out(f64(out), ref, BF16_REL_L2, BF16_MAX_ABS, f"attention n={n} C={C}")
+    assert torch.equal(_run(q, k, v), out)
+
+
 @pytest.mark.parametrize("n,C", [(9, 9), (9, 300), (128, 128), (129, 200), (300, 300), (640, 1000), (1024, 1024)])
 def test_attention_prefill_parity(n, C):
     q, k, v = _qkv(n, C, seed=7 * C + n)
