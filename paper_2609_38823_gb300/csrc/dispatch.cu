@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(DSP_THREADS)
 }
 
 // Pass 2: the tile kernel (dispatch_tile). SINGLE: one tile in one block
-// (decode sizes); blocks from 1 on finish a deferred mass.
+// that also copies the rows; blocks from 1 on finish a deferred mass.
 template <bool SINGLE>
 __global__ void __launch_bounds__(DSP_THREADS)
     k_dispatch_scatter(const int32_t* __restrict__ idx, int64_t N, int k, int K,
@@ -302,16 +302,19 @@ int dispatch_with_mass(const int32_t* topk_idx, int64_t T, int k, int K, const v
   }
   const int ntiles = static_cast<int>((N + DSP_TILE - 1) / DSP_TILE);
   int32_t* tile_hist = static_cast<int32_t*>(ws);
-  if (ntiles == 1) {
-    // one tile (decode sizes): count, scan and rank in one block, and copy
-    // the rows there too when they are few
-    const bool gather_here = x_perm != nullptr && static_cast<size_t>(N) * row_bytes <= 64 * 1024;
+  const bool gather_here = ntiles == 1 && x_perm != nullptr && static_cast<size_t>(N) * row_bytes <= 64 * 1024;
+  if (gather_here) {
+    // one tile with few rows to copy: count, scan, rank and copy in one block.
+    // Without the copy the cluster below is faster from 16 pairs on (8 pairs 2.3
+    // us here and 2.4 there, 128 pairs 3.5 and 2.3, 512 4.2 and 2.8, 1024 5.0 and
+    // 3.1)
     DM_CUDA_CHECK(launch_pdl(k_dispatch_scatter<true>, dim3(1 + mblocks), dim3(DSP_THREADS), 0, s, topk_idx, N,
                              k, K, static_cast<const int32_t*>(nullptr), 1, counts, offsets, perm_token, inv_slot,
                              status_dev, static_cast<const uint4*>(x), static_cast<int>(row_bytes / 16),
-                             gather_here ? static_cast<uint4*>(x_perm) : static_cast<uint4*>(nullptr), mf));
-    if (gather_here) return DECOMOE_OK;
-  } else if (N <= DSC_MAX_PAIRS) {
+                             static_cast<uint4*>(x_perm), mf));
+    return DECOMOE_OK;
+  }
+  if (N <= DSC_MAX_PAIRS) {
     const int P = static_cast<int>((N + DSC_CTAS * DSP_WARPS * 32 - 1) / (DSC_CTAS * DSP_WARPS * 32)) * 32;
     auto kern = P <= 64 ? k_dispatch_cluster<2> : P <= 128 ? k_dispatch_cluster<4> : k_dispatch_cluster<DSC_MAX_ROUNDS>;
     cudaLaunchConfig_t cfg = {};

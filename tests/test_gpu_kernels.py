@@ -187,7 +187,8 @@ def test_dispatch_parity(T, k, K, d, dt, pattern):
 
 
 @pytest.mark.parametrize("T,k,K", [(1025, 1, 3), (205, 5, 200), (4096, 1, 64), (4097, 1, 256), (513, 8, 128),
-                                   (16384, 1, 17), (16385, 1, 17)])
+                                   (16384, 1, 17), (16385, 1, 17), (5, 1, 4), (16, 2, 5), (33, 1, 256),
+                                   (125, 8, 64), (128, 8, 200)])
 def test_dispatch_cluster_sizes(T, k, K):
     """One launch of a cluster up to 16384 pairs (two, four and eight 32-pair
     rounds per warp, the last warps partly or wholly empty), the two-launch form
