@@ -402,7 +402,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
     for (int t = cid; t < total; t += ncl, ++n) {
       const Item it = item(t);
       const int acc = n & 1;
-      if (g.x_copy != nullptr && !it.dn) {
+      if (ok && g.x_copy != nullptr && !it.dn) {
         // the grouped rows are wanted too: this item's share (rows dealt over
         // the row tile's gate/up items), while its accumulator is computed
         const int vec = g.d / 8, per = (it.nrow + NT1 - 1) / NT1;
@@ -424,9 +424,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
         }
         __syncwarp();
       }
-      if (!mbar_wait_idle(TFULL(acc), (n >> 1) & 1, g.limit_ns, s_abort, 100)) {
+      // a warp whose wait ran out stores nothing more, but goes on to the barrier
+      // that the others may have reached
+      if (ok && !mbar_wait_idle(TFULL(acc), (n >> 1) & 1, g.limit_ns, s_abort, 100)) {
         ok = false;
-        break;
+        *s_abort = 1;
       }
       tc_fence_after();
       const uint32_t tb = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * PF_BN);
@@ -452,7 +454,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
         }
         __syncwarp();
       };
-      if (nmine > 0) {
+      if (ok && nmine > 0) {
         const int64_t row = it.row0 + r0;
         if (!it.dn) {
           constexpr int GU = DECOMOE_GU_BLOCK;
@@ -494,7 +496,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
         // this CTA's h columns of the tile are stored: publish them to the down tiles
         fence_proxy_async_all();
         named_bar_sync(1, 32 * PF_EW);
-        if (warp == 2 && lane == 0) {
+        if (ok && warp == 2 && lane == 0) {
           __threadfence();
           atomicAdd(g.ready + 2 * it.mtg + rank, 1);
         }
