@@ -1241,6 +1241,7 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
     } else {
       *s_abort = 1;
       report_status(a.status, DECOMOE_ERR_TIMEOUT);
+      named_bar_sync(1 + x, 128);  // the head's other warps may have passed their waits
     }
   }
   pdl_trigger();
