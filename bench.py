@@ -35,9 +35,10 @@ sys.path.insert(0, ROOT)
 import workloads as W  # noqa: E402
 
 # at T=2048: router k slices, routing (reads the slices) with mass partials,
-# dispatch 2 (histogram + mass sum, ranks), the expert FFN (row gather, gate/up,
-# SwiGLU and down in one launch), combine with the visual-block removal
-LAUNCHES_PER_STEP = 6
+# dispatch (one cluster launch, mass sum in extra blocks), the expert FFN (rows by
+# index, gate/up, SwiGLU and down in one launch), combine with the visual-block
+# removal
+LAUNCHES_PER_STEP = 5
 
 
 def parse():
@@ -226,10 +227,10 @@ class Buffers:
 
 
 def layer_gathers(R):
-    """Whether the layer's one-launch expert FFN also does the dispatch's row
-    gather at R routed rows (from 8192 rows up to the one-launch limit of
-    32768; above it the layer gathers in the dispatch and runs the two expert
-    GEMMs as separate launches)."""
+    """Whether the timed expert call at R routed rows reads x by index, as the
+    layer does, and writes the grouped copy beside it (the range of
+    decomoe_expert_swiglu_fused_gather's one launch timed here), or takes
+    grouped rows from the dispatch."""
     return 8192 <= R <= 32768
 
 
@@ -246,8 +247,8 @@ def run_step(dm, wl, L, B, K, v0, nv, text, ev=None):
                              status=B.status, text_out=text, v0=v0, nv=nv)
         return
     # a1 + a2 (Eq. 11) + a4 + a5: router logits, routing with the activated
-    # mass, dispatch (from 8192 routed rows the layer leaves the row gather to
-    # the expert launch, and so does this)
+    # mass, dispatch (without the grouped rows where the expert launch reads by
+    # index)
     gather = layer_gathers(L.x.shape[0] * k)
     dm.decomoe_router_route_dispatch(L.x, L.w_r, L.bias, B.logits, K, k, B.idx, B.w, B.counts[:K], B.offsets[:K + 1],
                                      B.perm, B.inv, None if gather else B.x_perm, B.rrd_ws, mass_out=B.mass,

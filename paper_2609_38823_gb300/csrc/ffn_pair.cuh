@@ -4,9 +4,11 @@
 // A cluster of two CTAs computes one tile of 256 rows x 256 weight rows. CTA r
 // holds rows [128 r, 128 r + 128) of the row tile (A) and weight rows [128 r,
 // 128 r + 128) (B). A row tile of at most 128 rows is an M = 128 product with 64
-// rows per CTA, half the time. One thread of CTA 0 issues M = 256, N = 256 products that
-// read both CTAs' operands, and each CTA's tensor memory receives its 128 rows
-// x 256 columns. Why pairs: at 128 x 256 on one SM a 64-deep k-block moves 48 KB
+// rows per CTA: its k-blocks take as long in the tensor pipe (a gate/up item
+// 20200 cycles against 19900), but half the row traffic (T = 2048, K = 64 184 us
+// a layer, with full tiles throughout 194). One thread of CTA 0 issues M = 256,
+// N = 256 products that read both CTAs' operands, and each CTA's tensor memory
+// receives its 128 rows x 256 columns. Why pairs: at 128 x 256 on one SM a 64-deep k-block moves 48 KB
 // into shared memory and the products read 48 KB back, 768 cycles of its 128
 // bytes a cycle against 512 of tensor work; half the weights per SM make that
 // 512 against 512, and six k-blocks are on their way instead of four. Weights and
