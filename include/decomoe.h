@@ -423,8 +423,9 @@ DECOMOE_API int decomoe_drop_visual_block_if(const int32_t* exit_flag, const voi
  * h: dtype (DECOMOE_BF16 or DECOMOE_F32), d a multiple of 64, 16-byte
  * aligned. w1 [H, 2d], b1 [H], w2 [2, H], b2 [2]: fp32 device arrays (w1
  * 16-byte aligned). p_exit, exit_flag: one fp32 / int32 on the device.
- * ws: decomoe_savb_gate_workspace_bytes(d, H) bytes, 16-byte aligned; it
- * need not start at zero. Two launches; no host synchronisation (the caller
+ * ws: decomoe_savb_gate_workspace_bytes(d, H) bytes, 16-byte aligned (down to
+ * 8d + 4H bytes, each rounded up to 256, and 256 more, pooling runs in fewer row
+ * classes; less is DECOMOE_ERR_WORKSPACE); it need not start at zero. Two launches; no host synchronisation (the caller
  * reads exit_flag to decide whether to remove the visual block before the
  * next layer, which changes the shapes of every later launch).
  * ------------------------------------------------------------------------ */

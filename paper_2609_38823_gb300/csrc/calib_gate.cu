@@ -288,14 +288,20 @@ static int gate_splits(int d) { return std::min(GATE_MAX_SPLITS, std::max(1, 128
 struct GateLayout {
   size_t part, last, zpart, counter, total;
 };
-static GateLayout gate_layout(int d, int H) {
+static GateLayout gate_layout(int d, int H, int splits) {
   GateLayout L;
   L.part = 0;
-  L.last = align_up(static_cast<size_t>(GATE_MAX_SPLITS) * d * sizeof(float), 256);
+  L.last = align_up(static_cast<size_t>(splits) * d * sizeof(float), 256);
   L.zpart = align_up(L.last + static_cast<size_t>(d) * sizeof(float), 256);
   L.counter = align_up(L.zpart + static_cast<size_t>(2) * ((H + GATE_UNITS - 1) / GATE_UNITS) * sizeof(float), 256);
   L.total = L.counter + 256;
   return L;
+}
+// The least workspace a call takes (x [2d], hidden [H] and the counter fit):
+// pooling then runs in as many row classes as there is room for, one at least.
+static size_t gate_base_bytes(int d, int H) {
+  return align_up(align_up(static_cast<size_t>(2) * d * sizeof(float), 256) + static_cast<size_t>(H) * sizeof(float), 256) +
+         256;
 }
 
 }  // namespace decomoe
@@ -378,7 +384,7 @@ int decomoe_permute_experts(const void* src, void* dst, const int32_t* pi, int E
 
 size_t decomoe_savb_gate_workspace_bytes(int d, int H) {
   if (d <= 0 || H <= 0) return 0;
-  return gate_layout(d, H).total;
+  return std::max(gate_layout(d, H, gate_splits(d)).total, gate_base_bytes(d, H));
 }
 
 int decomoe_savb_gate(const void* h, int64_t T, int d, int dtype, int64_t v0, int64_t nv, const float* w1,
@@ -393,11 +399,13 @@ int decomoe_savb_gate(const void* h, int64_t T, int d, int dtype, int64_t v0, in
   DM_ARG_CHECK(T - nv >= 1, "savb_gate: no text rows");
   DM_ARG_CHECK(h && w1 && b1 && w2 && b2 && p_exit && exit_flag, "savb_gate: null pointer");
   DM_ARG_CHECK(aligned16(h) && aligned16(w1), "savb_gate: h and w1 must be 16-byte aligned");
-  const GateLayout L = gate_layout(d, H);
-  if (ws == nullptr || ws_bytes < L.total) {
-    set_error("savb_gate: workspace needs %zu bytes", L.total);
+  if (ws == nullptr || ws_bytes < gate_base_bytes(d, H)) {
+    set_error("savb_gate: workspace needs %zu bytes", decomoe_savb_gate_workspace_bytes(d, H));
     return DECOMOE_ERR_WORKSPACE;
   }
+  int splits = gate_splits(d);
+  while (splits > 1 && ws_bytes < gate_layout(d, H, splits).total) --splits;
+  const GateLayout L = gate_layout(d, H, splits);
   DM_ARG_CHECK(aligned16(ws), "savb_gate: workspace must be 16-byte aligned");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   uint8_t* base = static_cast<uint8_t*>(ws);
@@ -406,7 +414,6 @@ int decomoe_savb_gate(const void* h, int64_t T, int d, int dtype, int64_t v0, in
   float* zpart = reinterpret_cast<float*>(base + L.zpart);
   unsigned* counter = reinterpret_cast<unsigned*>(base + L.counter);
   const int64_t n = T - nv;
-  const int splits = gate_splits(d);
   const dim3 grid(d / GATE_COLS, splits);
   if (dtype == DECOMOE_BF16)
     DM_CUDA_CHECK(launch_pdl(k_gate_pool<__nv_bfloat16>, grid, dim3(256), 0, s, static_cast<const __nv_bfloat16*>(h), d,

@@ -241,6 +241,31 @@ def test_savb_gate_parity(T, v0, nv, d, H, dt):
             assert int(ex.item()) == int(O.gate_decision(p_ref, theta))
 
 
+@pytest.mark.parametrize("d,H", [(2048, 512), (64, 1), (192, 100)])
+def test_savb_gate_smaller_workspaces(d, H):
+    """Every workspace down to x [2d], hidden [H] and the counter is taken (fewer
+    row classes: fp32 sums in another order, the tolerance of the full one);
+    less is refused."""
+    T, v0, nv = 700, 5, 400
+    h = torch.randn(T, d, generator=torch.Generator().manual_seed(d)).to(torch.bfloat16)
+    w1, b1, w2, b2 = _gate_params(d, H, seed=H)
+    dev = [torch.from_numpy(v).to(DEV) for v in (w1, b1, w2, b2)]
+    p = torch.empty(1, dtype=torch.float32, device=DEV)
+    ex = torch.empty(1, dtype=torch.int32, device=DEV)
+    p_ref = O.gate_exit_prob(O.gate_logits(O.gate_feature(f64(h), v0, nv), w1, b1, w2, b2))
+    full = dm.decomoe_savb_gate_workspace_bytes(d, H)
+    base = 8 * d + -(-4 * H // 256) * 256 + 256
+    assert base <= full
+    for nbytes in {base, (base + full) // 2 // 256 * 256, full}:
+        buf = torch.full((nbytes + 64,), 0x77, dtype=torch.uint8, device=DEV)
+        dm.decomoe_savb_gate(h.to(DEV), v0, nv, *dev, 0.5, p, ex, buf[:nbytes])
+        torch.cuda.synchronize()
+        assert abs(float(p.item()) - p_ref) <= 2e-5
+        assert (buf[nbytes:] == 0x77).all()
+    with pytest.raises(dm.DecomoeError):
+        dm.decomoe_savb_gate(h.to(DEV), v0, nv, *dev, 0.5, p, ex, buf[:base - 1])
+
+
 def test_savb_gate_fires_on_a_biased_head_and_graph_replays():
     T, v0, nv, d, H = 1552, 16, 1280, 2048, 512
     h = torch.randn(T, d, generator=torch.Generator().manual_seed(4)).to(torch.bfloat16).to(DEV)
