@@ -620,6 +620,26 @@ def test_rmsnorm():
         assert np.abs(f64(y) - ref).max() <= tol * np.abs(ref).max() * 2
 
 
+@pytest.mark.parametrize("T,d,dt", [(1, 8, "bf16"), (3, 2040, "bf16"), (305, 2048, "bf16"), (2433, 2048, "bf16"),
+                                    (5, 2056, "bf16"), (2, 4, "f32"), (153, 1024, "f32"), (2432, 1020, "f32"),
+                                    (7, 1028, "f32")])
+def test_rmsnorm_row_forms(T, d, dt):
+    """Rows in registers (up to 256 vectors, whole and ragged) and rows read
+    twice, one block per SM and more: fp32 sum of squares over d terms
+    (relative error at most d 2^-24 of it, halved by the root), one rounding to
+    the storage type."""
+    dtype = torch.bfloat16 if dt == "bf16" else torch.float32
+    x = torch.randn(T, d, generator=torch.Generator().manual_seed(T + d)).to(dtype)
+    y = torch.empty(T + 1, d, dtype=dtype, device=DEV).fill_(3.0)
+    dm.decomoe_rmsnorm(x.to(DEV), y[:T])
+    torch.cuda.synchronize()
+    xf = f64(x)
+    ref = xf / np.sqrt((xf * xf).mean(axis=1, keepdims=True) + 1e-6)
+    rel = (2.0 ** -8 if dt == "bf16" else 2.0 ** -22) + d * 2.0 ** -25
+    assert (np.abs(f64(y[:T]) - ref) <= np.abs(ref) * rel).all()
+    assert (y[T] == 3.0).all()
+
+
 # ----------------------------------------------------------------- routing + dispatch in one call
 
 @pytest.mark.parametrize("T,E,K,k,p", [(1, 128, 64, 8, 0.0), (7, 16, 10, 2, 0.0), (100, 128, 40, 8, 0.0),
