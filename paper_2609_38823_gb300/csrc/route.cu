@@ -135,9 +135,10 @@ __global__ void __launch_bounds__(ROUTE_THREADS)
   if (zero_ints != nullptr && blockIdx.x == 0)
     for (int i = threadIdx.x; i < n_zero; i += ROUTE_THREADS) zero_ints[i] = 0;
   if (K_dev != nullptr) K = *K_dev;  // prefix chosen on the device (k <= K <= E by construction)
-  __shared__ int s_idx[ROUTE_TPB][DECOMOE_MAX_TOPK];
-  __shared__ float s_w[ROUTE_TPB][DECOMOE_MAX_TOPK];
-  __shared__ float s_row[NP > 1 ? ROUTE_TPB : 1][NP > 1 ? DECOMOE_MAX_E : 1];
+  // a token's logits (NP > 1), then its full-pool weights by expert (mass): one
+  // read per token and expert, where each thread looked for its expert among the
+  // block's 64 picks (with the mass 131 tokens 6.8 -> 5.9 us, 16384 23.3 -> 20.4)
+  __shared__ __align__(16) float s_row[ROUTE_TPB][32 * NSL];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t t = static_cast<int64_t>(blockIdx.x) * ROUTE_TPB + warp;
   const bool mass = part != nullptr;
@@ -187,15 +188,17 @@ __global__ void __launch_bounds__(ROUTE_THREADS)
         v[i] = (e < lim) ? fkey(s_row[warp][e]) : 0u;
       }
     }
+    if (mass) {
+      __syncwarp();
+      for (int e = lane; e < E; e += 32) s_row[warp][e] = 0.f;
+    }
     float my_v;
     int my_i;
     warp_topk_n<NSL>(v, lim, k, lane, my_v, my_i);
     if (mass) {
       const float wf = pick_weight(my_v, lane, k);
-      if (lane < k) {
-        s_idx[warp][lane] = my_i;
-        s_w[warp][lane] = wf;
-      }
+      __syncwarp();
+      if (lane < k && my_i >= 0 && my_i < E) s_row[warp][my_i] = wf;
       // full-pool picks all inside the prefix: they are the prefix picks too
       const bool inside = __all_sync(0xffffffffu, lane >= k || my_i < K);
       if (!inside) warp_topk_n<NSL>(v, K, k, lane, my_v, my_i);
@@ -215,9 +218,9 @@ __global__ void __launch_bounds__(ROUTE_THREADS)
                                           : ROUTE_TPB);
     for (int e = threadIdx.x; e < E; e += ROUTE_THREADS) {
       float acc = 0.f;
-      for (int tt = 0; tt < ntok; ++tt)
-        for (int j = 0; j < k; ++j)
-          if (s_idx[tt][j] == e) acc += s_w[tt][j];  // token order, then slot order
+#pragma unroll
+      for (int tt = 0; tt < ROUTE_TPB; ++tt)
+        if (tt < ntok) acc += s_row[tt][e];  // token order; a token that did not pick e adds zero
       part[static_cast<int64_t>(blockIdx.x) * E + e] = static_cast<double>(acc);
     }
   }
