@@ -178,7 +178,10 @@ static cudaError_t launch_combine_w(cudaStream_t s, const uint4* y, const int32_
   }
 }
 // Warps per token by token count: one from 1024 tokens on, two from 512, four
-// from 32, eight below (a decode step's row then spans eight warps). A whole
+// from 153 (from 32 where a row has no 256 vectors for eight warps), eight below
+// (a row then spans the eight warps of a block, at most one block per SM: T = 64
+// 82.7 us a layer against 83.0 with four, T = 131 90.8 and 91.0, T = 150 95.7 and
+// 96.1). A whole
 // bf16 layer (top-k 8, d 2048): T = 272 takes 102.3 us with four warps a token
 // and 103.9 with two, T = 777 161.9 with either, T = 1552 213.4 with one and
 // 215.4 with two, T = 4096 274.3 with one and 276.1 with two.
@@ -187,7 +190,7 @@ static cudaError_t launch_combine_k(cudaStream_t s, const uint4* y, const int32_
                                     int k, int vec, const uint4* res, uint4* out, DropRows drop, int dc) {
   if (T >= 1024) return launch_combine_w<BF16, DROP, 1>(s, y, inv, w, T, k, vec, res, out, drop, dc);
   if (T >= 512) return launch_combine_w<BF16, DROP, 2>(s, y, inv, w, T, k, vec, res, out, drop, dc);
-  if (T >= 32) return launch_combine_w<BF16, DROP, 4>(s, y, inv, w, T, k, vec, res, out, drop, dc);
+  if (T > 152 || (T >= 32 && vec < 256)) return launch_combine_w<BF16, DROP, 4>(s, y, inv, w, T, k, vec, res, out, drop, dc);
   return launch_combine_w<BF16, DROP, 8>(s, y, inv, w, T, k, vec, res, out, drop, dc);
 }
 template <bool BF16>
