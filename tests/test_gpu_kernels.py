@@ -481,6 +481,24 @@ def test_combine_parity(T, k, d, dt, resid):
         assert_close_out(got, ref, BF16_REL_L2, BF16_MAX_ABS, "combine bf16")
 
 
+@pytest.mark.parametrize("T,k,d", [(31, 8, 2048), (32, 8, 2048), (152, 8, 2048), (153, 8, 2048), (152, 3, 2040),
+                                   (511, 8, 512), (512, 8, 512), (1023, 2, 512), (1024, 2, 512)])
+def test_combine_warps_per_token(T, k, d):
+    """The steps of the warps-per-token rule, whole and ragged rows; fp32 sums of
+    k + 1 terms and one rounding to bf16, as in test_combine_parity."""
+    g = torch.Generator().manual_seed(T + d)
+    y = torch.randn(T * k, d, generator=g).to(torch.bfloat16)
+    inv = torch.randperm(T * k, generator=g).to(torch.int32)
+    w = torch.softmax(torch.randn(T, k, generator=g), -1).float()
+    res = torch.randn(T, d, generator=g).to(torch.bfloat16)
+    out = torch.empty(T, d, dtype=torch.bfloat16, device=DEV)
+    dm.decomoe_combine(y.to(DEV), inv.to(DEV), w.to(DEV), out, res.to(DEV))
+    torch.cuda.synchronize()
+    got, ref = f64(out), O.combine(f64(y), inv.numpy(), f64(w), f64(res))
+    mag = O.combine(np.abs(f64(y)), inv.numpy(), np.abs(f64(w)), np.abs(f64(res)))
+    assert (np.abs(got - ref) <= np.abs(ref) * 2.0 ** -8 + 2e-6 * mag).all()
+
+
 @pytest.mark.parametrize("T,k,d,dt,resid,v0,nv", [(2048, 8, 2048, "bf16", True, 0, 1792),
                                                    (333, 3, 128, "bf16", False, 100, 200),
                                                    (64, 2, 256, "f32", True, 10, 0),
