@@ -118,8 +118,11 @@ __global__ void __launch_bounds__(256, WPT == 1 ? 2 : 1)
             acc_vec<BF16>(acc2, v2[j], wts[j]);
           }
         if (discard) {
-          // every lane's loads of these lines have been consumed above
-          __syncwarp();
+          // every lane's loads of these lines have been consumed above; the lanes
+          // past the end of a row that is no multiple of 32 vectors (fp32, d =
+          // 96) are not in this iteration and must not be waited for
+          const int here = vec - (c - lane);
+          __syncwarp(here >= 32 ? 0xffffffffu : (1u << here) - 1u);
           if ((lane & 7) == 0) {
 #pragma unroll
             for (int j = 0; j < KT; ++j)

@@ -115,6 +115,27 @@ def test_layer_tiny_fp32_residual():
     _compare(g_cpu, out, logits, idx, w, 10, wl.k, np.arange(wl.T), (F32_REL_L2, F32_MAX_ABS), residual=res)
 
 
+@pytest.mark.parametrize("T,d", [(5, 96), (70, 288), (600, 96), (1100, 288), (12000, 96), (12000, 288)])
+def test_layer_fp32_ragged_rows_with_scratch_discarded(T, d):
+    """Rows of 24 and 72 vectors (whole 128-byte lines, no multiple of 32
+    vectors), every number of warps per token, and several tokens a warp: the
+    combine drops the lines of its scratch after reading them, and its lanes
+    past a row's end take no part in that. The bits of the layer that keeps its
+    scratch, and the oracle's values."""
+    wl = W.with_(W.TINY, T=T, d=d)
+    g_cpu = W.make_layer(wl, device="cpu")
+    g = {n: t.to(DEV) for n, t in g_cpu.items()}
+    out, _, _, logits, idx, w, _ = _run_layer(g, wl.k, T, K_fixed=10)
+    dm.decomoe_set_discard_scratch(False)
+    try:
+        kept = _run_layer(g, wl.k, T, K_fixed=10)[0]
+    finally:
+        dm.decomoe_set_discard_scratch(True)
+    assert torch.equal(out, kept)
+    sample = np.unique(np.linspace(0, T - 1, 40).astype(int))
+    _compare(g_cpu, out, logits, idx, w, 10, wl.k, sample, (F32_REL_L2, F32_MAX_ABS))
+
+
 # ----------------------------------------------------------------- prefill T=2048 at full size
 
 @pytest.fixture(scope="module")
