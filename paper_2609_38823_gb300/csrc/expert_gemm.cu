@@ -678,9 +678,12 @@ __global__ void __launch_bounds__(192, 1)
       const WsTile T = ws_tile<WS_BN>(t, total, s_tt, s_off, G, nwb);
       const int acc = it & 1;
       const uint32_t aph = (it >> 1) & 1;
-      if (!mbar_wait(TFULL_BAR(acc), aph, g.limit_ns, s_abort)) {
+      // a warp whose wait ran out (or that saw another role give up) loads and
+      // stores nothing more, but goes on to the barriers, which have no limit
+      // and which the other warps may have reached
+      if (ok && !__all_sync(0xffffffffu, mbar_wait(TFULL_BAR(acc), aph, g.limit_ns, s_abort))) {
         ok = false;
-        break;
+        *s_abort = 1;
       }
       tc_fence_after();
       const uint32_t tb =
@@ -695,24 +698,26 @@ __global__ void __launch_bounds__(192, 1)
 #pragma unroll 1
       for (int c0 = 0; c0 < T.ntok; c0 += 32) {
         uint32_t r[32];
-        tmem_ld32(tb + c0, r);
-        tc_wait_ld();
+        if (ok) {
+          tmem_ld32(tb + c0, r);
+          tc_wait_ld();
+        }
         __nv_bfloat16* st = stile + xpar * (32 * OC);
         if constexpr (SWIGLU) {
           const bool is_gate = q < 2;
           const int pr = q & 1;
           float* xb = xch + (xpar * 2 + pr) * 1024;  // [32 columns][32 lanes]
-          if (!is_gate) {
+          if (ok && !is_gate) {
 #pragma unroll
             for (int c = 0; c < 32; ++c) xb[c * 32 + lane] = __uint_as_float(r[c]);
           }
           named_bar_sync(1, 128);
-          if (is_gate) {
+          if (ok && is_gate) {
 #pragma unroll
             for (int c = 0; c < 32; ++c)
               st[c * OC + pr * 32 + lane] = __float2bfloat16_rn(silu_f(__uint_as_float(r[c])) * xb[c * 32 + lane]);
           }
-        } else {
+        } else if (ok) {
 #pragma unroll
           for (int c = 0; c < 32; ++c) st[c * OC + q * 32 + lane] = __float2bfloat16_rn(__uint_as_float(r[c]));
         }
@@ -722,7 +727,7 @@ __global__ void __launch_bounds__(192, 1)
 #pragma unroll
         for (int v = et; v < 32 * VPR; v += 128) {
           const int row = v / VPR, cv = v - row * VPR;
-          if (row < nc) {
+          if (ok && row < nc) {
             const uint4 val = *reinterpret_cast<const uint4*>(st + row * OC + cv * 8);
             *reinterpret_cast<uint4*>(out + static_cast<int64_t>(T.row0 + c0 + row) * g.out_ld + fbase + cv * 8) = val;
           }
@@ -1087,9 +1092,10 @@ __global__ void __launch_bounds__(192, 1)
       const WsTile T = item(t, dn);
       const int acc = it & 1;
       const uint32_t aph = (it >> 1) & 1;
-      if (!mbar_wait(TFULL_BAR(acc), aph, g.limit_ns, s_abort)) {
+      // as in k_moe_ws: after a wait that ran out, barriers only
+      if (ok && !__all_sync(0xffffffffu, mbar_wait(TFULL_BAR(acc), aph, g.limit_ns, s_abort))) {
         ok = false;
-        break;
+        *s_abort = 1;
       }
       tc_fence_after();
       const uint32_t tb = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * BN);
@@ -1103,24 +1109,26 @@ __global__ void __launch_bounds__(192, 1)
 #pragma unroll 1
       for (int c0 = 0; c0 < T.ntok; c0 += 32) {
         uint32_t r[32];
-        tmem_ld32(tb + c0, r);
-        tc_wait_ld();
+        if (ok) {
+          tmem_ld32(tb + c0, r);
+          tc_wait_ld();
+        }
         __nv_bfloat16* st = stile + xpar * (32 * WS_BM);
         if (!dn) {
           const bool is_gate = q < 2;
           const int pr = q & 1;
           float* xb = xch + (xpar * 2 + pr) * 1024;  // [32 columns][32 lanes]
-          if (!is_gate) {
+          if (ok && !is_gate) {
 #pragma unroll
             for (int c = 0; c < 32; ++c) xb[c * 32 + lane] = __uint_as_float(r[c]);
           }
           named_bar_sync(1, 128);
-          if (is_gate) {
+          if (ok && is_gate) {
 #pragma unroll
             for (int c = 0; c < 32; ++c)
               st[c * OC + pr * 32 + lane] = __float2bfloat16_rn(silu_f(__uint_as_float(r[c])) * xb[c * 32 + lane]);
           }
-        } else {
+        } else if (ok) {
 #pragma unroll
           for (int c = 0; c < 32; ++c) st[c * OC + q * 32 + lane] = __float2bfloat16_rn(__uint_as_float(r[c]));
         }
@@ -1129,7 +1137,7 @@ __global__ void __launch_bounds__(192, 1)
         const int VPR = OC / 8;  // 16-byte vectors per token row
         for (int v = et; v < 32 * VPR; v += 128) {
           const int row = v / VPR, cv = v - row * VPR;
-          if (row < nc) {
+          if (ok && row < nc) {
             const uint4 val = *reinterpret_cast<const uint4*>(st + row * OC + cv * 8);
             *reinterpret_cast<uint4*>(out + static_cast<int64_t>(T.row0 + c0 + row) * ld + fbase + cv * 8) = val;
           }
@@ -1139,10 +1147,11 @@ __global__ void __launch_bounds__(192, 1)
       tc_fence_before();
       mbar_arrive(TEMPTY_BAR(acc));
       if (!dn) {
-        // this item's h slice is stored: publish it to the down items of T.g
+        // this item's h slice is stored (by every warp: a warp that gave up
+        // raised the flag ahead of the barrier): publish it to the down items of T.g
         fence_proxy_async_all();
         named_bar_sync(1, 128);
-        if (et == 0) {
+        if (et == 0 && !*s_abort) {
           __threadfence();
           atomicAdd(g.ready + T.g, 1);
         }

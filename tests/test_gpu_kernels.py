@@ -334,6 +334,33 @@ def test_expert_swiglu_bf16_parity(T, k, K, d, m, pattern):
         assert e.value.code == dm.DECOMOE_ERR_INVALID_ARG
 
 
+@pytest.mark.parametrize("T,k,K", [(5, 8, 64), (40, 8, 64), (64, 8, 64), (9, 8, 9), (300, 2, 16)])
+def test_fused_experts_wait_for_rows_that_never_come(T, k, K):
+    """Readiness counters that no number of stored tiles brings to their goal:
+    the down tiles' waits run out (after 20 ms here; every copy in flight has
+    landed by then), the launch ends with the status set, and the next call, on
+    zeroed counters, gives the two launches' bits. The weights-stationary form
+    with each token chunk it has, and the pair form."""
+    d, m = 512, 256
+    L, x_perm, offsets = _expert_case(T, k, K, d, m, "route", seed=2)
+    w_gu, w_dn = dm.fuse_gate_up(L["w_gate"].to(DEV), L["w_up"].to(DEV)), L["w_down"].to(DEV)
+    xp, off = x_perm.to(DEV), torch.from_numpy(offsets.astype(np.int32)).to(DEV)
+    h, y, h2, y2 = (torch.empty(T * k, n, dtype=torch.bfloat16, device=DEV) for n in (m, d, m, d))
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    ready = torch.full((dm.decomoe_expert_swiglu_ready_ints(T * k, K),), -100000, dtype=torch.int32, device=DEV)
+    dm.decomoe_set_wait_limit_ns(20_000_000)
+    try:
+        dm.decomoe_expert_swiglu_fused(xp, off, K, w_gu, w_dn, h, y, ready, status)
+        assert dm.decomoe_read_status(status) == dm.DECOMOE_ERR_TIMEOUT
+    finally:
+        dm.decomoe_set_wait_limit_ns(2_000_000_000)
+    ready.zero_()
+    dm.decomoe_expert_swiglu_fused(xp, off, K, w_gu, w_dn, h, y, ready, status)
+    dm.decomoe_expert_swiglu(xp, off, K, w_gu, w_dn, h2, y2, status)
+    assert dm.decomoe_read_status(status) == 0
+    assert torch.equal(y, y2) and torch.equal(h, h2)
+
+
 def test_expert_swiglu_f32_parity():
     T, k, K, d, m = 64, 2, 10, 256, 128
     L, x_perm, offsets = _expert_case(T, k, K, d, m, "route", seed=1, dtype=torch.float32)
