@@ -1033,9 +1033,13 @@ __global__ void __launch_bounds__(DL_THREADS, 1)
       item(t, dn, eg, wb);
       const int acc = it & 1;
       const uint32_t aph = (it >> 1) & 1;
-      if (!mbar_wait(TFULL_BAR(acc), aph, g.limit_ns, s_abort)) {
+      // A warp whose wait ran out (or that saw another role give up) loads and
+      // stores nothing more, but goes on to the barriers, which have no limit
+      // and which the other warps may have reached; the queue's wait above ends
+      // the loop for all four.
+      if (ok && !__all_sync(0xffffffffu, mbar_wait(TFULL_BAR(acc), aph, g.limit_ns, s_abort))) {
         ok = false;
-        break;
+        *s_abort = 1;
       }
       tc_fence_after();
       const uint32_t tb = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * DL_BN);
@@ -1043,24 +1047,26 @@ __global__ void __launch_bounds__(DL_THREADS, 1)
       // accumulator column c: token c of x (gate/up) or row r0 + c of h (down)
       const int OC = dn ? DL_BM : DL_BM / 2;
       uint32_t rr[32];
-      tmem_ld32(tb, rr);
-      tc_wait_ld();
+      if (ok) {
+        tmem_ld32(tb, rr);
+        tc_wait_ld();
+      }
       __nv_bfloat16* st = stile + xpar * (32 * DL_BM);
       if (!dn) {
         const bool is_gate = q < 2;
         const int pr = q & 1;
         float* xb = xch + (xpar * 2 + pr) * 1024;  // [32 columns][32 lanes]
-        if (!is_gate) {
+        if (ok && !is_gate) {
 #pragma unroll
           for (int c = 0; c < 32; ++c) xb[c * 32 + lane] = __uint_as_float(rr[c]);
         }
         named_bar_sync(1, 128);
-        if (is_gate) {
+        if (ok && is_gate) {
 #pragma unroll
           for (int c = 0; c < 32; ++c)
             st[c * OC + pr * 32 + lane] = __float2bfloat16_rn(silu_f(__uint_as_float(rr[c])) * xb[c * 32 + lane]);
         }
-      } else {
+      } else if (ok) {
 #pragma unroll
         for (int c = 0; c < 32; ++c) st[c * OC + q * 32 + lane] = __float2bfloat16_rn(__uint_as_float(rr[c]));
       }
@@ -1072,7 +1078,7 @@ __global__ void __launch_bounds__(DL_THREADS, 1)
       const int VPR = OC / 8;
       __nv_bfloat16* outp = dn ? g.y : g.h;
       const int64_t ld = dn ? d : g.m;
-      for (int v = et; v < nr * VPR; v += 128) {
+      for (int v = et; ok && v < nr * VPR; v += 128) {
         const int i = v / VPR, cv = v - i * VPR;
         const int col = dn ? i : s_perm[r0 + i];
         const uint4 val = *reinterpret_cast<const uint4*>(st + col * OC + cv * 8);
@@ -1080,16 +1086,17 @@ __global__ void __launch_bounds__(DL_THREADS, 1)
       }
       xpar ^= 1;
       if (!dn) {
-        // this item's h slice is stored: publish it to the down items of eg
+        // this item's h slice is stored (by every warp: one that gave up raised
+        // the flag ahead of the barrier): publish it to the down items of eg
         fence_proxy_async_all();
         named_bar_sync(1, 128);
-        if (et == 0) red_add_release_s32(ready + eg, 1);
+        if (et == 0 && !*s_abort) red_add_release_s32(ready + eg, 1);
       } else {
-        // y rows of block wb stored: count them per token; the tile that
+        // y rows of block wb stored (by every warp): count them per token; the tile that
         // completes a token's k slots of this block combines them
         if (et == 0) s_flag[2] = 0;
         named_bar_sync(1, 128);
-        if (et < nr) {
+        if (et < nr && !*s_abort) {
           const int tok = s_perm[r0 + et];
           // release this tile's y rows; the k-th arrival acquires the others'
           const int old = atom_add_acq_rel_s32(comb + tok * nfb + wb, 1);

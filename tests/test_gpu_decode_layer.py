@@ -250,3 +250,36 @@ def test_other_pool_shapes_against_oracle(E, k, T, K, p):
     wg, wu, wd = (_Experts(g[n]) for n in ("w_gate", "w_up", "w_down"))
     ref = np.stack([O.moe_token(f64(x[t]), logits[t].astype(np.float32), wg, wu, wd, Ku, k)[0] for t in range(T)])
     assert_close_out(f64(out)[keep], ref[keep], BF16_REL_L2, BF16_MAX_ABS, f"decode layer E={E} k={k} T={T}")
+
+
+@pytest.mark.parametrize("T,K", [(1, 64), (9, -1), (23, 96)])
+def test_rows_that_never_come_end_in_a_timeout(layer, T, K):
+    """Readiness counters set so low, in the counter block behind its signature,
+    that the down tiles' waits run out (after 20 ms; every copy in flight has
+    landed by then): the launch ends with the status set and without the
+    signature, so the next call starts from fresh counters and gives the bits
+    of the first."""
+    wl, g = layer
+    x = W.make_x(W.with_(wl, T=T), seed=T, device="cuda")
+    out, again = torch.empty_like(x), torch.empty_like(x)
+    ws = _ws(wl, T)
+    ws.zero_()
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    _call(wl, g, x, out, ws, K, status=status)
+    assert dm.decomoe_read_status(status) == 0
+    words = ws[:ws.numel() // 8 * 8].view(torch.int64)
+    at = ((words >> 40) & 0xFFFFFF == 0xD3C0AE).nonzero().flatten().tolist()  # the launch counter, 16 bytes in
+    assert len(at) == 1
+    ready = ws[8 * at[0] + 16:][:4 * wl.E].view(torch.int32)
+    assert int(ready.abs().sum()) == 0
+    ready.fill_(-100000)
+    dm.decomoe_set_wait_limit_ns(20_000_000)
+    try:
+        _call(wl, g, x, again, ws, K, status=status)
+        assert dm.decomoe_read_status(status) == dm.DECOMOE_ERR_TIMEOUT
+    finally:
+        dm.decomoe_set_wait_limit_ns(2_000_000_000)
+    assert int((words[at[0]] >> 40) & 0xFFFFFF) != 0xD3C0AE
+    _call(wl, g, x, again, ws, K, status=status)
+    assert dm.decomoe_read_status(status) == 0
+    assert torch.equal(_bits(again), _bits(out))
