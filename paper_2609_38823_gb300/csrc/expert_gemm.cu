@@ -294,7 +294,8 @@ __global__ void __launch_bounds__(64 + 32 * RT_EW, 1)
     for (int t = blockIdx.x; t < total; t += gridDim.x, ++n) {
       const int e = t / KS % MT * RT_BM + q * 32 + lane, n0 = t / KS / MT * BN;
       const int acc = n & 1;
-      if (!mbar_wait(TFULL(acc), (n >> 1) & 1, g.limit_ns, s_abort)) {
+      // decided by the whole warp: the tensor-memory loads below are a warp's
+      if (!__all_sync(0xffffffffu, mbar_wait(TFULL(acc), (n >> 1) & 1, g.limit_ns, s_abort))) {
         ok = false;
         break;
       }
