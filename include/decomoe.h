@@ -294,14 +294,16 @@ DECOMOE_API int decomoe_expert_swiglu(const void* x_perm, const int32_t* offsets
 
 /* decomoe_expert_swiglu with both GEMMs in one persistent launch where that
  * is faster (bf16, 16 to 32768 rows): the down tiles of an expert (decode
- * sizes) or of a 128-row tile (larger) start as soon as the gate/up tiles
- * they read have stored h, published through per-expert or per-row-tile counters
- * with release/acquire ordering. ready: decomoe_expert_swiglu_ready_ints(rows,
+ * sizes) or of a row tile (of 256 rows or, where at most 128 are left, 128) start
+ * as soon as the gate/up tiles they read have stored h, published through
+ * per-expert or per-row-tile counters with release/acquire ordering. ready: decomoe_expert_swiglu_ready_ints(rows,
  * K) int32, all zero at the call (decomoe_moe_layer clears its own); the call
  * leaves them non-zero. Outside that range the call runs the two launches of
  * decomoe_expert_swiglu and leaves ready untouched. Outputs are bit-identical
  * to decomoe_expert_swiglu. Needs every CTA of the launch resident at once
- * (it sizes the grid to the SMs of the current device). */
+ * (it sizes the grid to the SMs of the current device): work on other streams
+ * that holds SMs holds the call up, and two such launches on two streams, each
+ * with part of the SMs, would end in DECOMOE_ERR_TIMEOUT. */
 DECOMOE_API size_t decomoe_expert_swiglu_ready_ints(int64_t rows, int K);
 DECOMOE_API int decomoe_expert_swiglu_fused(const void* x_perm, const int32_t* offsets, int64_t rows, int K, int d,
                                             int m, int dtype, const void* w_gate_up, const void* w_down, void* h_ws,
@@ -494,7 +496,13 @@ DECOMOE_API int decomoe_rmsnorm(const void* x, void* y, int64_t T, int d, float 
  * K_used_host / K_sel_host may be NULL.
  * x, residual, out: [T, d] dtype (out may alias residual, not x).
  * ws: decomoe_moe_layer_workspace_bytes(...) bytes; every intermediate
- * (logits, routes, dispatch arrays, x_perm, h, y_perm) lives there.
+ * (logits, routes, dispatch arrays, h, y_perm, and x_perm where it is made: see
+ * decomoe_moe_layer_workspace_layout) lives there.
+ * In bf16, up to 32 tokens (the one-launch layer) and from 16 to 32768 routed
+ * rows (T*k, the one-launch experts) a kernel of the call waits for other blocks
+ * of its own launch, as decomoe_expert_swiglu_fused does, and needs them all on
+ * the device together: order such calls on different streams by events. Above
+ * 32768 rows, and in fp32, no kernel does.
  * ------------------------------------------------------------------------ */
 DECOMOE_API size_t decomoe_moe_layer_workspace_bytes(int64_t T, int d, int E, int k, int m, int dtype);
 DECOMOE_API int decomoe_moe_layer(const void* x, const void* w_r, const float* bias, const void* w_gate_up,

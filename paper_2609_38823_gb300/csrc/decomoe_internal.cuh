@@ -184,6 +184,7 @@ int moe_layer_impl(const void* x, const void* w_r, const float* bias, const void
 // perm (pair form only) the gate/up rows are gather_x[perm[r]] and x_perm is
 // not read; copy_rows: it receives those rows.
 enum { FFN_FUSED_NONE = 0, FFN_FUSED_WS = 1, FFN_FUSED_PAIR = 2 };
+constexpr int64_t FFN_FUSED_MAX_ROWS = 32768;  // above it no kernel of a layer waits for another block of its launch
 int expert_ffn_fused_kind(int64_t rows, int K, int dtype);
 size_t expert_ffn_sync_ints(int64_t rows, int E);
 int launch_expert_ffn_fused(const void* x_perm, const int32_t* offsets, int64_t rows, int K, int d, int m, int dtype,

@@ -1773,12 +1773,20 @@ namespace decomoe {
 #ifndef DECOMOE_FFN_FUSED_MIN_ROWS
 #define DECOMOE_FFN_FUSED_MIN_ROWS 16
 #endif
+// Rows up to which it is taken: FFN_FUSED_MAX_ROWS. Its down tiles wait for gate/up tiles of other
+// blocks, so the launch needs all its blocks on the device together: other
+// long-running work on the device holds it up, and a second launch of the kind
+// on another stream, each with part of the SMs, would end both in a timeout.
+// Two launches need nothing of other blocks. A layer (d = 2048, m = 768, top 8) in
+// one launch and in two: 4097 tokens, 128 experts 342 and 349 us, 8000 tokens 566
+// and 557, 16384 tokens 1050 and 1005.
 // Which one-launch form the expert FFN takes: FFN_FUSED_NONE (two launches:
-// fp32 and fewer than DECOMOE_FFN_FUSED_MIN_ROWS rows), FFN_FUSED_WS (at most 8
-// rows per expert on average) or FFN_FUSED_PAIR (above, any size).
+// fp32, fewer than DECOMOE_FFN_FUSED_MIN_ROWS rows or more than
+// FFN_FUSED_MAX_ROWS), FFN_FUSED_WS (at most 8 rows per expert on average) or
+// FFN_FUSED_PAIR (above).
 int expert_ffn_fused_kind(int64_t rows, int K, int dtype) {
   constexpr int64_t min_rows = DECOMOE_FFN_FUSED_MIN_ROWS;
-  if (dtype != DECOMOE_BF16 || rows < min_rows || rows <= 0 || K <= 0) return FFN_FUSED_NONE;
+  if (dtype != DECOMOE_BF16 || rows < min_rows || rows > FFN_FUSED_MAX_ROWS || K <= 0) return FFN_FUSED_NONE;
   return rows <= static_cast<int64_t>(DECOMOE_WS_MAX_AVG_ROWS) * K ? FFN_FUSED_WS : FFN_FUSED_PAIR;
 }
 
@@ -1807,8 +1815,6 @@ int launch_expert_ffn_fused(const void* x_perm, const int32_t* offsets, int64_t 
 
 // int32 counters the fused expert launch needs (zero at launch): one per
 // expert (decode kernel) or two per 256-row tile (pair kernel).
-// Rows that decomoe_expert_swiglu_fused runs as one launch (its contract).
-constexpr int64_t PUBLIC_FUSED_MAX_ROWS = 32768;
 size_t expert_ffn_sync_ints(int64_t rows, int E) { return 2 * static_cast<size_t>(rows / 128 + E + 1); }
 
 }  // namespace decomoe
@@ -1825,9 +1831,8 @@ int decomoe_expert_swiglu_fused(const void* x_perm, const int32_t* offsets, int6
   using namespace decomoe;
   clear_error();
   bool fused = false;
-  if (rows <= PUBLIC_FUSED_MAX_ROWS)
-    DM_RET(launch_expert_ffn_fused(x_perm, offsets, rows, K, d, m, dtype, w_gate_up, w_down, h_ws, y_perm, ready,
-                                   status_dev, reinterpret_cast<cudaStream_t>(stream), &fused));
+  DM_RET(launch_expert_ffn_fused(x_perm, offsets, rows, K, d, m, dtype, w_gate_up, w_down, h_ws, y_perm, ready,
+                                 status_dev, reinterpret_cast<cudaStream_t>(stream), &fused));
   if (fused) return DECOMOE_OK;
   return decomoe_expert_swiglu(x_perm, offsets, rows, K, d, m, dtype, w_gate_up, w_down, h_ws, y_perm, status_dev,
                                nullptr, stream);
@@ -1840,7 +1845,7 @@ int decomoe_expert_swiglu_fused_gather(const void* x, int64_t T, const int32_t* 
   using namespace decomoe;
   clear_error();
   DM_ARG_CHECK(x != nullptr && perm_token != nullptr && T >= 0, "expert_swiglu_fused_gather: null pointer");
-  DM_ARG_CHECK(rows <= PUBLIC_FUSED_MAX_ROWS && expert_ffn_fused_kind(rows, K, dtype) == FFN_FUSED_PAIR,
+  DM_ARG_CHECK(expert_ffn_fused_kind(rows, K, dtype) == FFN_FUSED_PAIR,
                "expert_swiglu_fused_gather: %lld rows at K=%d take no one-launch tokens-as-M form",
                (long long)rows, K);
   bool fused = false;

@@ -348,11 +348,15 @@ int moe_layer_impl(const void* x, const void* w_r, const float* bias, const void
   // dispatch has no rows to gather (T = 131, K = 64 99.8 -> 95.9 us, T = 777 181.8
   // -> 173.9, T = 16384 1144 -> 1057 against a gather launch). Their grouped copy
   // in the workspace is then left only for inspection (scratch not discarded).
-  // So do the fp32 experts (64 tokens 23.6 -> 22.3 us), which make no copy
+  // So do the pair kernel's two launches, at more rows than the one launch takes,
+  // and the fp32 experts (64 tokens 23.6 -> 22.3 us), which make no copy
   // themselves: with the scratch kept, the dispatch does.
   auto ffn_gathers = [&](int K_groups) {
-    return dtype == DECOMOE_F32 ? discard_scratch()
-                                : expert_ffn_fused_kind(T * k, K_groups, dtype) == FFN_FUSED_PAIR;
+    if (dtype == DECOMOE_BF16) {
+      const int kind = expert_ffn_fused_kind(T * k, K_groups, dtype);
+      if (kind != FFN_FUSED_NONE || T * k <= FFN_FUSED_MAX_ROWS) return kind == FFN_FUSED_PAIR;
+    }
+    return discard_scratch();
   };
   DM_ARG_CHECK(dtype != DECOMOE_F32 || (d % 4 == 0 && aligned16(x)),
                "moe_layer: rows must be 16-byte multiples and 16-byte aligned");
@@ -393,12 +397,10 @@ int moe_layer_impl(const void* x, const void* w_r, const float* bias, const void
                                   L.off[WS_KDEV] - L.off[WS_ROUTE], status_dev, stream));
   }
   if (K_used_host && K_fixed != -1) *K_used_host = K;
-  // a6: grouped SwiGLU experts over [0, K): at decode sizes gate/up and down
-  // in one launch, else the two GEMMs (static tile order: as fast as the
-  // dynamic queue here, and no counter reset between the launches, which
-  // keeps them chained programmatically)
+  // a6: grouped SwiGLU experts over [0, K): gate/up and down in one launch up
+  // to FFN_FUSED_MAX_ROWS routed rows, else in two
   bool fused = false;
-  const bool by_index = gathers && dtype == DECOMOE_BF16;
+  const bool by_index = gathers && expert_ffn_fused_kind(T * k, K, dtype) == FFN_FUSED_PAIR;
   DM_RET(launch_expert_ffn_fused(x_perm, offsets, T * k, K, d, m, dtype, w_gate_up, w_down, h, y_perm, sync,
                                  status_dev, s, &fused, by_index ? x : nullptr, by_index ? perm : nullptr,
                                  !discard_scratch()));

@@ -9,6 +9,8 @@ one that logits within the bounds rank first, and its weights and output are
 compared with the oracle evaluated on that set. Every sampled token is thus
 compared; the near-tie count is printed and bounded.
 """
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -343,3 +345,57 @@ def test_layer_exit_equals_layer_then_removal(prefill_layer, T, K_fixed, v0, nv)
     assert dm.decomoe_read_status(st) == 0
     assert torch.equal(out1.view(torch.int16), out2.view(torch.int16))
     assert torch.equal(text1.view(torch.int16), text2.view(torch.int16))
+
+
+def _kernels_of(call):
+    """Kernel launches of a call, counted in a capture of it (nothing runs)."""
+    rt = ctypes.CDLL("libcudart.so.13")
+    s = torch.cuda.Stream()
+    handle, graph = ctypes.c_void_p(s.cuda_stream), ctypes.c_void_p()
+    n = ctypes.c_size_t(0)
+    with torch.cuda.stream(s):
+        assert rt.cudaStreamBeginCapture(handle, 2) == 0  # relaxed mode
+        try:
+            call()
+        finally:
+            rc = rt.cudaStreamEndCapture(handle, ctypes.byref(graph))
+    assert rc == 0 and rt.cudaGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    nodes, kind = (ctypes.c_void_p * n.value)(), ctypes.c_int()
+    assert rt.cudaGraphGetNodes(graph, nodes, ctypes.byref(n)) == 0
+    kinds = []
+    for node in nodes:
+        assert rt.cudaGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        kinds.append(kind.value)
+    rt.cudaGraphDestroy(graph)
+    return kinds.count(0)  # cudaGraphNodeTypeKernel
+
+
+@pytest.mark.parametrize("K_fixed", [40, -1])
+def test_no_kernel_waits_for_other_blocks_above_the_fused_rows(K_fixed):
+    """Up to 32768 routed rows the experts are one launch, whose down tiles
+    wait for gate/up tiles of other blocks and so need them all on the device;
+    above, two launches, which a busy device only slows down. One more kernel,
+    the same bits as the layer that keeps its grouped rows, and the oracle's
+    values."""
+    wl = W.with_(W.PREFILL, T=4097, d=256, m=128)
+    g_cpu = W.make_layer(wl, device="cpu")
+    g = {n: t.to(DEV) for n, t in g_cpu.items()}
+    out, Ku, _, logits, idx, w, _ = _run_layer(g, wl.k, wl.T, K_fixed=K_fixed, p=0.7)
+    ws = dm.workspace(dm.decomoe_moe_layer_workspace_bytes(wl.T, wl.d, wl.E, wl.k, wl.m, 0), DEV)
+
+    def call(T):
+        return lambda: dm.decomoe_moe_layer(g["x"][:T], g["w_r"], g["bias"], g["w_gu"], g["w_down"], wl.k, out[:T], ws,
+                                            K_fixed=K_fixed, p=0.7)
+
+    assert _kernels_of(call(4097)) == _kernels_of(call(4096)) + 1
+    dm.decomoe_set_discard_scratch(False)
+    try:
+        kept = _run_layer(g, wl.k, wl.T, K_fixed=K_fixed, p=0.7)[0]
+    finally:
+        dm.decomoe_set_discard_scratch(True)
+    torch.cuda.synchronize()
+    assert torch.equal(out.view(torch.int16), kept.view(torch.int16))
+    sample = np.unique(np.linspace(0, wl.T - 1, 24).astype(int))
+    K = K_fixed if K_fixed > 0 else O.select_prefix(
+        O.activated_mass(O.router_logits(f64(g_cpu["x"]), f64(g_cpu["w_r"]), g_cpu["bias"].numpy()), wl.k), 0.7, wl.k)
+    _compare(g_cpu, out, logits, idx, w, K, wl.k, sample, (BF16_REL_L2, BF16_MAX_ABS))
