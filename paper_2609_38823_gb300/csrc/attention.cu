@@ -680,7 +680,7 @@ constexpr int ATP_REGS_SOFTMAX = 208, ATP_REGS_ISSUE = 88;
 static_assert(2 * ATP_REGS_SOFTMAX + ATP_REGS_ISSUE <= 3 * 168, "register split within the launch's total");
 constexpr int ATP_TMEM_COLS = 512;           // per head: S [0,128) (P over [0,64)), O [128,256)
 constexpr float ATP_RESCALE = 8.0f;          // log2 of the largest unnormalised p
-constexpr float ATP_NONE = -1.0e30f;         // reference maximum of a row that has seen no key
+constexpr float ATP_NONE = -FLT_MAX;         // reference maximum of a row that has seen no key: no score lies below it
 constexpr size_t ATP_SMEM = 1024 + (ATP_HEADS + ATP_NST) * ATP_SLOT + 32 * 8 + 16;
 static_assert(ATP_SMEM <= 232448, "prefill attention shared memory");
 

@@ -138,6 +138,18 @@ def test_attention_prefill_full_sizes_sampled(n, C):
     _sampled_rows(out, q, k, v, rows, f"prefill attention n={n} C={C} (sampled rows)")
 
 
+@pytest.mark.parametrize("n,C", [(40, 40), (300, 300), (300, 2500)])
+def test_attention_prefill_scores_near_the_lowest_float(n, C):
+    """Equal scores of -2^110 (powers of two, so the scaled scores are exact):
+    every row is the mean of the values it sees, whole tiles and split ones."""
+    _, _, v = _qkv(1, C, seed=C)
+    q = torch.full((n, HQ, D), 2.0 ** 60, dtype=torch.bfloat16)
+    k = torch.full((C, HKV, D), -(2.0 ** 43), dtype=torch.bfloat16)
+    out = _run(q, k, v, scale=1.0)
+    ref = O.attention(f64(q), f64(k), f64(v), scale=1.0)
+    assert_close_out(f64(out), ref, BF16_REL_L2, BF16_MAX_ABS, f"attention of very low scores n={n} C={C}")
+
+
 def test_attention_prefill_grouping_and_scale():
     # 8 query heads on 2 KV heads: 40 queries make 160 per KV head
     q, k, v = _qkv(40, 333, seed=6, Hq=8, Hkv=2)
