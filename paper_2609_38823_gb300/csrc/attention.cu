@@ -696,6 +696,7 @@ struct AttPreArgs {
   int64_t n, C;        // queries (the last n positions), keys
   int Hq, group;       // query heads, query heads per KV head
   int L;               // key blocks per item at most (0: every tile is one item)
+  int cut;             // tile t sees none of the second 64 keys of block t + cut
   float scale_log2;    // scale * log2(e)
   float* part;         // partial O of the split items, [item][head][128][128]
   float2* ml;          // their row maxima and sums, [item][head][128]
@@ -1026,7 +1027,10 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
           tc_mma_f16(S_TM(x), ad + (ATP_HALF >> 4) * kb + 2u * kk, bd + (ATP_HALF >> 4) * kb + 2u * kk, IDESC_S,
                      (kb | kk) != 0 ? 1u : 0u);
     };
-    // O_x += P_x V_j over 64 of the block's keys
+    // O_x += P_x V_j over 64 of the block's keys. Keys that no row of the tile sees
+    // are left out (a.cut): their weights are zero, but a value that is not finite
+    // would still reach the rows. The test keeps no register of its own: one more
+    // live in this loop costs 4 % of the kernel.
     auto issue_pv = [&](int x, int st, int half, bool acc) {
       const uint64_t bd = vd + static_cast<uint32_t>(st * (ATP_SLOT >> 4));
 #pragma unroll
@@ -1064,7 +1068,7 @@ __global__ void __launch_bounds__(ATP_THREADS, 1)
         for (int half = 0; half < 2; ++half) {
           ok = ok && wait(P_FULL(x, half), j & 1);
           tc_fence_after();
-          if (ok && leader) issue_pv(x, st, half, j > 0);
+          if (ok && leader && (half == 0 || it.first + j - qt != a.cut)) issue_pv(x, st, half, j > 0);
         }
         if (x == 0 && j + 1 < nblk) ok = ok && wait(FULL(stk), phk);
         tc_fence_after();
@@ -1377,6 +1381,10 @@ int decomoe_attention(const void* q, int64_t n, const void* k_cache, const void*
     AttPreSplit sp = att_pre_split(n, C, Hq);
     if (sp.split_items * ATP_ITEM_BYTES > ws_bytes) sp = {0, (n + ATP_BM - 1) / ATP_BM * (Hq / ATP_HEADS), 0, 0};
     pa.L = sp.L;
+    // every tile starts (C - n) % 128 keys into a block; after 1 to 64, the last
+    // block that it reaches into has a second half that it does not see
+    const int64_t off = C - n, r = off % ATP_BN;
+    pa.cut = r >= 1 && r <= ATP_BN / 2 ? static_cast<int>(off / ATP_BN) + 1 : -(1 << 30);
     pa.part = static_cast<float*>(ws);
     pa.ml = reinterpret_cast<float2*>(pa.part + sp.split_items * ATP_HEADS * ATP_PART);
     DM_CUDA_CHECK(cudaFuncSetAttribute(k_attn_prefill, cudaFuncAttributeMaxDynamicSharedMemorySize,

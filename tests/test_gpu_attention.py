@@ -150,6 +150,21 @@ def test_attention_prefill_scores_near_the_lowest_float(n, C):
     assert_close_out(f64(out), ref, BF16_REL_L2, BF16_MAX_ABS, f"attention of very low scores n={n} C={C}")
 
 
+@pytest.mark.parametrize("n,C,bad", [(256, 320, 200), (256, 320, 255), (200, 2564, 2500), (130, 194, 193)])
+def test_attention_prefill_later_values_do_not_reach_earlier_tiles(n, C, bad):
+    """A key block whose second 64 keys no row of the tile sees: a value there
+    that is not finite belongs to later rows and leaves the tile's bits as they
+    are, whole tiles and split ones."""
+    assert C - n + 127 < bad // 64 * 64 and bad % 128 >= 64
+    q, k, v = _qkv(n, C, seed=C + bad)
+    out = _run(q, k, v)
+    v[bad, :, ::3] = float("inf")
+    v[bad, :, 1::3] = float("nan")
+    got = _run(q, k, v)
+    assert torch.equal(got[:128], out[:128])
+    assert not torch.isfinite(got[bad - (C - n):, :, 0]).any()
+
+
 def test_attention_prefill_grouping_and_scale():
     # 8 query heads on 2 KV heads: 40 queries make 160 per KV head
     q, k, v = _qkv(40, 333, seed=6, Hq=8, Hkv=2)
