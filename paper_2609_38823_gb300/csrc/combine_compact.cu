@@ -180,20 +180,22 @@ static cudaError_t launch_combine_w(cudaStream_t s, const uint4* y, const int32_
     default: return launch_pdl(k_combine<BF16, 0, DROP, WPT>, g, b, 0, s, y, inv, w, T, k, vec, res, out, drop, 0);
   }
 }
-// Warps per token by token count: one from 1024 tokens on, two from 512, four
-// from 153 (from 32 where a row has no 256 vectors for eight warps), eight below
-// (a row then spans the eight warps of a block, at most one block per SM: T = 64
-// 82.7 us a layer against 83.0 with four, T = 131 90.8 and 91.0, T = 150 95.7 and
-// 96.1). A whole
-// bf16 layer (top-k 8, d 2048): T = 272 takes 102.3 us with four warps a token
-// and 103.9 with two, T = 777 161.9 with either, T = 1552 213.4 with one and
-// 215.4 with two, T = 4096 274.3 with one and 276.1 with two.
+// Warps per token: as many of eight, four and two as give every SM at most one
+// block of eight warps (which may then be scheduled while the kernel before
+// drains), two up to 1023 tokens, one above. Eight only where a row has a chunk
+// for each (from 32 tokens on; below, few tokens leave SMs idle either way). bf16
+// rows of 2048, top 8, calls after one another, on 152 SMs: 272 tokens 2.6 us with
+// four warps and 4.1 with two, 511 tokens 4.8 and 4.4 (rows of 256: 3.9 and 2.3),
+// 513 tokens 3.9 with two. In a layer 131 tokens take 90.8 us with eight and 91.0
+// with four, 1552 tokens 213.4 with one and 215.4 with two, 4096 tokens 274.3 and
+// 276.1.
 template <bool BF16, bool DROP>
 static cudaError_t launch_combine_k(cudaStream_t s, const uint4* y, const int32_t* inv, const float* w, int64_t T,
                                     int k, int vec, const uint4* res, uint4* out, DropRows drop, int dc) {
+  const int64_t sms = sm_count();
   if (T >= 1024) return launch_combine_w<BF16, DROP, 1>(s, y, inv, w, T, k, vec, res, out, drop, dc);
-  if (T >= 512) return launch_combine_w<BF16, DROP, 2>(s, y, inv, w, T, k, vec, res, out, drop, dc);
-  if (T > 152 || (T >= 32 && vec < 256)) return launch_combine_w<BF16, DROP, 4>(s, y, inv, w, T, k, vec, res, out, drop, dc);
+  if (T > 2 * sms) return launch_combine_w<BF16, DROP, 2>(s, y, inv, w, T, k, vec, res, out, drop, dc);
+  if (T > sms || (T >= 32 && vec < 256)) return launch_combine_w<BF16, DROP, 4>(s, y, inv, w, T, k, vec, res, out, drop, dc);
   return launch_combine_w<BF16, DROP, 8>(s, y, inv, w, T, k, vec, res, out, drop, dc);
 }
 template <bool BF16>

@@ -526,6 +526,13 @@ def test_combine_warps_per_token(T, k, d):
     assert (np.abs(got - ref) <= np.abs(ref) * 2.0 ** -8 + 2e-6 * mag).all()
 
 
+@pytest.mark.parametrize("per_sm,more", [(1, 0), (1, 1), (2, 0), (2, 1)])
+@pytest.mark.parametrize("k,d", [(8, 2048), (3, 2040), (8, 256)])
+def test_combine_warps_per_token_at_the_sm_count(per_sm, more, k, d):
+    """The rule's steps that follow the number of SMs, on this device."""
+    test_combine_warps_per_token(per_sm * torch.cuda.get_device_properties(0).multi_processor_count + more, k, d)
+
+
 @pytest.mark.parametrize("T,k,d,dt,resid,v0,nv", [(2048, 8, 2048, "bf16", True, 0, 1792),
                                                    (333, 3, 128, "bf16", False, 100, 200),
                                                    (64, 2, 256, "f32", True, 10, 0),
