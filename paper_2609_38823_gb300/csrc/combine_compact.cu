@@ -65,8 +65,16 @@ __device__ __forceinline__ void l2_discard_line(const void* p) {
   asm volatile("discard.global.L2 [%0], 128;" ::"l"(p) : "memory");
 }
 
+// Many tokens of one or two slots: a chunk has few loads, so four blocks per SM (64
+// registers, no spills; three with the second store of bf16) keep enough in flight:
+// 16384 tokens of 1024, top 2, no residual 12.0 us against 14.2 with three blocks.
+template <bool BF16, int KT, bool DROP>
+constexpr int combine_blocks_per_sm() {
+  return KT != 1 && KT != 2 ? 2 : BF16 && DROP ? 3 : 4;
+}
+
 template <bool BF16, int KT, bool DROP, int WPT>
-__global__ void __launch_bounds__(256, WPT == 1 ? 2 : 1)
+__global__ void __launch_bounds__(256, WPT == 1 ? combine_blocks_per_sm<BF16, KT, DROP>() : 1)
     k_combine(const uint4* __restrict__ y, const int32_t* __restrict__ inv_slot,
               const float* __restrict__ w, int64_t Tn, int k, int vec,
               const uint4* __restrict__ residual, uint4* __restrict__ out, DropRows drop, int discard) {
@@ -185,7 +193,7 @@ static cudaError_t launch_combine_w(cudaStream_t s, const uint4* y, const int32_
 // drains), two up to 1023 tokens, one above. Eight only where a row has a chunk
 // for each (from 32 tokens on; below, few tokens leave SMs idle either way). bf16
 // rows of 2048, top 8, calls after one another, on 152 SMs: 272 tokens 2.6 us with
-// four warps and 4.1 with two, 511 tokens 4.8 and 4.4 (rows of 256: 3.9 and 2.3),
+// four warps and 4.1 with two, 511 tokens 4.8 and 3.8 (rows of 256: 3.9 and 2.1),
 // 513 tokens 3.9 with two. In a layer 131 tokens take 90.8 us with eight and 91.0
 // with four, 1552 tokens 213.4 with one and 215.4 with two, 4096 tokens 274.3 and
 // 276.1.
