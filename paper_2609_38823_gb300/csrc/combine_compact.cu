@@ -2,6 +2,8 @@
 // visual-block removal from hidden states and KV rows (Section 3.2), and the
 // RMSNorm of the attention-free layer stack. All three are HBM-bound copies
 // or reductions over rows: 16-byte vector accesses, one warp per row.
+#include <type_traits>
+
 #include "decomoe_internal.cuh"
 
 namespace decomoe {
@@ -277,7 +279,7 @@ __global__ void k_compact_bytes(const uint8_t* __restrict__ src, uint8_t* __rest
 }
 
 // ------------------------------------------------------------------ RMSNorm
-constexpr int RN_VEC = 8;  // 16-byte vectors per lane kept in registers (d = 2048 in bf16, 1024 in fp32)
+constexpr int RN_VEC = 8;  // most 16-byte vectors per lane kept in registers (d = 2048 in bf16, 1024 in fp32)
 template <bool BF16>
 __device__ __forceinline__ float sumsq_vec(float ss, const uint4& v) {
   const uint32_t u[4] = {v.x, v.y, v.z, v.w};
@@ -305,11 +307,13 @@ __device__ __forceinline__ uint4 scale_vec(const uint4& v, float f) {
   return make_uint4(o[0], o[1], o[2], o[3]);
 }
 // One warp per row. Bound by latency up to a few thousand rows: a row of at
-// most 32 RN_VEC vectors stays in registers (REGS), its loads all in flight and
-// read once, where the sum and the scaling were a pass each (bf16 rows of 2048,
-// blocks of eight warps: 272 rows 2.9 -> 1.9 us, 1552 rows 3.5 -> 3.1, 16384 rows
-// 23.0 -> 20.0).
-template <bool BF16, bool REGS>
+// most 32 RN_VEC vectors stays in registers (NV of them per lane, the power of two
+// that holds the row: slots that a short row leaves empty still cost registers and
+// instructions), its loads all in flight and read once, where the sum and the
+// scaling were a pass each (bf16 rows of 2048, blocks of eight warps: 272 rows 2.9
+// -> 1.9 us, 1552 rows 3.5 -> 3.1, 16384 rows 23.0 -> 20.0; rows of 64 with eight
+// slots 7.3 us at 16384 rows, with one 3.1). NV = 0: a longer row, read twice.
+template <bool BF16, int NV>
 __global__ void __launch_bounds__(512)
     k_rmsnorm(const uint4* __restrict__ x, uint4* __restrict__ y, int64_t Tn, int vec, int d,
               float eps) {
@@ -320,22 +324,22 @@ __global__ void __launch_bounds__(512)
   for (int64_t t = gw; t < Tn; t += nw) {
     const uint4* xr = x + t * vec;
     uint4* yr = y + t * vec;
-    uint4 v[REGS ? RN_VEC : 1];
+    uint4 v[NV > 0 ? NV : 1];
     float ss = 0.f;
-    if constexpr (REGS) {
+    if constexpr (NV > 0) {
 #pragma unroll
-      for (int i = 0; i < RN_VEC; ++i) v[i] = lane + 32 * i < vec ? xr[lane + 32 * i] : make_uint4(0, 0, 0, 0);
+      for (int i = 0; i < NV; ++i) v[i] = lane + 32 * i < vec ? xr[lane + 32 * i] : make_uint4(0, 0, 0, 0);
 #pragma unroll
-      for (int i = 0; i < RN_VEC; ++i) ss = sumsq_vec<BF16>(ss, v[i]);
+      for (int i = 0; i < NV; ++i) ss = sumsq_vec<BF16>(ss, v[i]);
     } else {
       for (int c = lane; c < vec; c += 32) ss = sumsq_vec<BF16>(ss, xr[c]);
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
     const float inv = rsqrtf(ss / static_cast<float>(d) + eps);
-    if constexpr (REGS) {
+    if constexpr (NV > 0) {
 #pragma unroll
-      for (int i = 0; i < RN_VEC; ++i)
+      for (int i = 0; i < NV; ++i)
         if (lane + 32 * i < vec) yr[lane + 32 * i] = scale_vec<BF16>(v[i], inv);
     } else {
       for (int c = lane; c < vec; c += 32) yr[c] = scale_vec<BF16>(xr[c], inv);
@@ -493,12 +497,15 @@ int decomoe_rmsnorm(const void* x, void* y, int64_t T, int d, float eps, int dty
   DM_ARG_CHECK(row_bytes % 16 == 0 && aligned16(x) && aligned16(y), "rmsnorm: rows must be 16-byte multiples");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int vec = static_cast<int>(row_bytes / 16);
-  // Up to 16 rows per SM, at most one block per SM (so that it may be scheduled
-  // while the kernel before drains) with the rows spread over all of them: 272
-  // rows 1.7 us against 1.9 in blocks of eight warps, 1552 rows 2.3 against 3.1.
-  // Beyond, blocks of eight warps (4096 rows 4.9 us either way).
+  // Up to 16 rows per SM (6 where they are read twice), at most one block per SM (so
+  // that it may be scheduled while the kernel before drains) with the rows spread
+  // over all of them: 272 rows 1.7 us against 1.9 in blocks of eight warps, 1552
+  // rows 2.3 against 3.1; rows of 8192, read twice: 272 rows 5.2 against 6.8, 912
+  // rows 6.0 against 8.8, 1000 rows 9.2 against 8.7. Beyond, blocks of eight warps
+  // (4096 rows 4.9 us either way; 1552 rows of 4096 5.6 against 7.3).
+  const int nv = vec > 32 * RN_VEC ? 0 : vec > 128 ? 8 : vec > 64 ? 4 : vec > 32 ? 2 : 1;
   int warps = 8, grid = grid_for_warps(T);
-  if (T <= 16 * static_cast<int64_t>(sm_count())) {
+  if (T <= (nv > 0 ? 16 : 6) * static_cast<int64_t>(sm_count())) {
     warps = static_cast<int>(std::max<int64_t>(2, (T + sm_count() - 1) / sm_count()));
     grid = static_cast<int>(std::max<int64_t>(1, (T + warps - 1) / warps));
   }
@@ -506,11 +513,17 @@ int decomoe_rmsnorm(const void* x, void* y, int64_t T, int d, float eps, int dty
     return launch_pdl(kern, dim3(grid), dim3(32 * warps), 0, s, static_cast<const uint4*>(x), static_cast<uint4*>(y), T,
                       vec, d, eps);
   };
-  const bool regs = vec <= 32 * RN_VEC;
-  if (dtype == DECOMOE_BF16)
-    DM_CUDA_CHECK(regs ? go(k_rmsnorm<true, true>) : go(k_rmsnorm<true, false>));
-  else
-    DM_CUDA_CHECK(regs ? go(k_rmsnorm<false, true>) : go(k_rmsnorm<false, false>));
+  auto pick = [&](auto bf16) {
+    constexpr bool B = decltype(bf16)::value;
+    switch (nv) {
+      case 1: return go(k_rmsnorm<B, 1>);
+      case 2: return go(k_rmsnorm<B, 2>);
+      case 4: return go(k_rmsnorm<B, 4>);
+      case 8: return go(k_rmsnorm<B, 8>);
+      default: return go(k_rmsnorm<B, 0>);
+    }
+  };
+  DM_CUDA_CHECK(dtype == DECOMOE_BF16 ? pick(std::true_type()) : pick(std::false_type()));
   return DECOMOE_OK;
 }
 

@@ -692,6 +692,15 @@ def test_rmsnorm_row_forms(T, d, dt):
     assert (y[T] == 3.0).all()
 
 
+@pytest.mark.parametrize("T,d,dt", [(9, 256, "bf16"), (2433, 264, "bf16"), (2433, 512, "bf16"), (7, 520, "bf16"),
+                                    (305, 1024, "bf16"), (9, 1032, "bf16"), (913, 2056, "bf16"), (912, 4096, "bf16"),
+                                    (3, 128, "f32"), (3, 132, "f32"), (2433, 256, "f32"), (9, 260, "f32"), (9, 516, "f32")])
+def test_rmsnorm_vectors_per_lane(T, d, dt):
+    """Rows on either side of one, two, four and eight vectors a lane, and the
+    block sizes' step for rows read twice."""
+    test_rmsnorm_row_forms(T, d, dt)
+
+
 # ----------------------------------------------------------------- routing + dispatch in one call
 
 @pytest.mark.parametrize("T,E,K,k,p", [(1, 128, 64, 8, 0.0), (7, 16, 10, 2, 0.0), (100, 128, 40, 8, 0.0),
