@@ -217,6 +217,13 @@ def test_dispatch_cluster_sizes(T, k, K):
         assert np.array_equal(offsets.cpu().numpy(), np.concatenate([[0], np.cumsum(c)]))
 
 
+@pytest.mark.parametrize("tiles", [17, 19, 20, 24, 27, 31, 33, 48])
+def test_dispatch_last_few_tiles(tiles):
+    """Every batch of tile histograms that the second pass adds up at once,
+    and the tiles left over."""
+    test_dispatch_cluster_sizes(tiles * 512 - 3, 2, 130)
+
+
 def test_dispatch_flags_bad_expert_id():
     T, k, K = 50, 2, 8
     idx = np.random.default_rng(0).integers(0, K, size=(T, k))
