@@ -303,11 +303,11 @@ int dispatch_with_mass(const int32_t* topk_idx, int64_t T, int k, int K, const v
   const int ntiles = static_cast<int>((N + DSP_TILE - 1) / DSP_TILE);
   int32_t* tile_hist = static_cast<int32_t*>(ws);
   const bool gather_here = ntiles == 1 && x_perm != nullptr && static_cast<size_t>(N) * row_bytes <= 64 * 1024;
-  if (gather_here) {
+  if (gather_here || (x_perm == nullptr && N <= 32)) {
     // one tile with few rows to copy: count, scan, rank and copy in one block.
-    // Without the copy the cluster below is faster from 16 pairs on (8 pairs 2.3
-    // us here and 2.4 there, 128 pairs 3.5 and 2.3, 512 4.2 and 2.8, 1024 5.0 and
-    // 3.1)
+    // Without the copy only as many pairs as one warp has lanes: the cluster below
+    // takes 2.5 us for 8 and for 32 pairs of 128 experts, this 2.2 and 2.4, but 2.6
+    // and 4.2 for 128 pairs, 2.8 and 4.2 for 512
     DM_CUDA_CHECK(launch_pdl(k_dispatch_scatter<true>, dim3(1 + mblocks), dim3(DSP_THREADS), 0, s, topk_idx, N,
                              k, K, static_cast<const int32_t*>(nullptr), 1, counts, offsets, perm_token, inv_slot,
                              status_dev, static_cast<const uint4*>(x), static_cast<int>(row_bytes / 16),
