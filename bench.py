@@ -228,9 +228,9 @@ class Buffers:
 
 def layer_gathers(R):
     """Whether the timed expert call at R routed rows reads x by index, as the
-    layer does, and writes the grouped copy beside it (the range of
-    decomoe_expert_swiglu_fused_gather's one launch timed here), or takes
-    grouped rows from the dispatch."""
+    layer does above 8 K rows, and writes the grouped copy beside it
+    (decomoe_expert_swiglu_fused_gather, up to its limit of 32768 rows), or
+    takes grouped rows from the dispatch."""
     return 8192 <= R <= 32768
 
 

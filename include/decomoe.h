@@ -279,8 +279,8 @@ DECOMOE_API int decomoe_weight_layout(const void* w_gate, const void* w_up, void
  * [E, d, m]; h_ws: [rows, m] dtype (intermediate, caller-owned); y_perm:
  * [rows, d] dtype. rows = T*k = offsets[K] (upper bound used to size tensor
  * maps; offsets stay on the device). Experts with no rows cost nothing.
- * bf16: tcgen05 tensor-core kernels for rows > 64, a weight-streaming kernel
- * for rows <= 64 (decode); fp32 accumulate, h rounded to bf16. f32: CUDA-core
+ * bf16: tcgen05 kernels, weights-stationary up to 8*K rows (decode sizes), on
+ * pairs of SMs above; fp32 accumulate, h rounded to bf16. f32: CUDA-core
  * kernels with h kept in fp32. Needs m % 64 == 0; bf16 also m % 128 == 0,
  * d % 256 == 0 and 16-byte aligned pointers (DECOMOE_ERR_INVALID_ARG
  * otherwise, before any launch).
@@ -427,9 +427,11 @@ DECOMOE_API int decomoe_drop_visual_block_if(const int32_t* exit_flag, const voi
  * 16-byte aligned). p_exit, exit_flag: one fp32 / int32 on the device.
  * ws: decomoe_savb_gate_workspace_bytes(d, H) bytes, 16-byte aligned (down to
  * 8d + 4H bytes, each rounded up to 256, and 256 more, pooling runs in fewer row
- * classes; less is DECOMOE_ERR_WORKSPACE); it need not start at zero. Two launches; no host synchronisation (the caller
- * reads exit_flag to decide whether to remove the visual block before the
- * next layer, which changes the shapes of every later launch).
+ * classes, another order of the sums and so p_exit's last bits; less is
+ * DECOMOE_ERR_WORKSPACE); it need not start at zero. Two launches; no host
+ * synchronisation (the caller reads exit_flag to decide whether to remove the
+ * visual block before the next layer, which changes the shapes of every later
+ * launch).
  * ------------------------------------------------------------------------ */
 DECOMOE_API size_t decomoe_savb_gate_workspace_bytes(int d, int H);
 DECOMOE_API int decomoe_savb_gate(const void* h, int64_t T, int d, int dtype, int64_t v0, int64_t nv,
@@ -563,7 +565,10 @@ DECOMOE_API int decomoe_moe_layer_workspace_layout(int64_t T, int d, int E, int 
  *   (few query tiles over a long cache) each tile's keys are split over
  *   several CTAs, whose rows a second small launch merges in key order; a
  *   workspace of at least the bytes for (n', C) at some other n' but too small
- *   for the split gives whole tiles instead.
+ *   for the split gives whole tiles instead. The same call gives the same bits
+ *   every time, but split rows and whole ones round differently: the last bits
+ *   of a row depend on how a sequence is cut into calls (n, C, the heads), on
+ *   whether the workspace holds the split, and on the number of SMs.
  *   ws: decomoe_attention_workspace_bytes(n, C, Hq, Hkv, D) bytes, 16-byte
  *   aligned. A wait that runs past the time limit records
  *   DECOMOE_ERR_TIMEOUT in status_dev (may be null).

@@ -455,9 +455,10 @@ def decomoe_gather_rows(x, perm_token, offsets, K, x_perm, stream=None):
 
 def decomoe_expert_swiglu_fused_gather(x, perm_token, offsets, K, w_gate_up, w_down, x_perm, h, y_perm, ready,
                                        status=None, stream=None):
-    """The one-launch expert FFN as the layer runs it from 8192 routed rows:
-    it gathers x_perm[r] = x[perm_token[r]] itself (dispatch called without
-    x_perm); ready: int32 counters, zero at the call."""
+    """The one-launch expert FFN reading its rows by index, as the layer runs
+    it from more than 8 K up to 32768 routed rows; x_perm[r] = x[perm_token[r]] is
+    written too (dispatch called without x_perm); ready: int32 counters, zero
+    at the call."""
     _need_cuda(x, perm_token, offsets, w_gate_up, w_down, x_perm, h, y_perm, ready, status)
     T, d = x.shape
     rows = x_perm.shape[0]

@@ -22,7 +22,6 @@ enum {
   WS_YPERM,
   WS_ROUTE,
   WS_KDEV,
-  WS_SCHED,
   WS_RSPLIT,
   WS_SYNC,
   WS_DSYNC,
@@ -181,7 +180,6 @@ static LayerLayout layer_layout(int64_t T, int d, int E, int k, int m, int dtype
   sz[WS_YPERM] = R * d * eb;
   sz[WS_ROUTE] = decomoe_route_dispatch_workspace_bytes(T, k, E);
   sz[WS_KDEV] = 16;
-  sz[WS_SCHED] = 16;
   sz[WS_RSPLIT] = decomoe_router_logits_ws_bytes(T, d, E);
   sz[WS_SYNC] = expert_ffn_sync_ints(static_cast<int64_t>(T) * k, E) * 4;  // counters of the fused expert launch
   sz[WS_DSYNC] = decode_layer_sync_ints(T, d, E) * 4;  // counters of the one-launch decode layer

@@ -47,8 +47,8 @@ def test_ffn_bound_is_hbm_at_the_measured_peaks():
 
 
 def test_ffn_algorithmic_bytes_with_the_row_gather():
-    """The layer's own launch from 8192 routed rows reads x once instead of
-    the gathered rows: 704.6 MB per launch at T=2048, K=64 (105.9 us at the
+    """A launch that reads its rows by index, as the layer's does, reads x once
+    instead of the gathered rows: 704.6 MB per launch at T=2048, K=64 (105.9 us at the
     measured HBM peak against 80.2 us of tensor work: still HBM-bound)."""
     b = _bench()
     wl = b.W.PREFILL
@@ -60,8 +60,9 @@ def test_ffn_algorithmic_bytes_with_the_row_gather():
 
 
 def test_layer_gather_range_matches_the_layer():
-    """bench.py times the gathering launch exactly where the layer uses it:
-    from 8192 routed rows up to the one-launch limit of 32768."""
+    """bench.py times the one launch that reads by index from 8192 routed rows
+    up to the one-launch limit of 32768, inside the layer's own range (from 8 K
+    rows, 1024 of 128 experts)."""
     b = _bench()
     assert not b.layer_gathers(8191)
     assert b.layer_gathers(8192) and b.layer_gathers(16384) and b.layer_gathers(32768)

@@ -260,7 +260,7 @@ EXPERT_CASES = [
     (64, 2, 16, 256, 128, "route"),
     (300, 1, 3, 256, 256, "one_expert"),  # one expert, 3 M tiles (300 rows)
     (512, 8, 64, 2048, 768, "route"),     # full layer width, 4096 rows
-    (1100, 8, 64, 2048, 768, "route"),    # 8800 rows: the layer's launch gathers its own rows
+    (1100, 8, 64, 2048, 768, "route"),    # 8800 rows
     (129, 8, 16, 2048, 768, "uniform"),
     (1, 8, 64, 2048, 768, "route"),       # decode T=1 (8 rows)
     (8, 8, 64, 2048, 768, "route"),       # decode T=8 (64 rows)
@@ -293,14 +293,15 @@ def test_expert_swiglu_bf16_parity(T, k, K, d, m, pattern):
     dm.decomoe_expert_swiglu_ref(xp, off, K, w_gu, g["w_down"], h2, y2)
     torch.cuda.synchronize()
     assert_close_out(f64(y), f64(y2), 2e-3, 1e-2, "tensor-core vs CUDA-core reference")
-    # dynamic tile scheduling hands the same tiles out in another order: same bits
-    sched = torch.zeros(1, dtype=torch.int32, device=DEV)
+    # the scheduling word is accepted and not used: whatever it holds, it stays
+    # and the bits are the same
+    sched = torch.full((1,), 12345, dtype=torch.int32, device=DEV)
     h4 = torch.empty_like(h)
     y4 = torch.empty_like(y)
     dm.decomoe_expert_swiglu(xp, off, K, w_gu, g["w_down"], h4, y4, status, sched)
     torch.cuda.synchronize()
     assert dm.decomoe_read_status(status) == 0
-    assert torch.equal(y4, y) and torch.equal(h4, h)
+    assert torch.equal(y4, y) and torch.equal(h4, h) and int(sched) == 12345
     # gather form: rows read from the token-ordered x through perm_token give
     # the same shared-memory tiles, so the same bits
     h3 = torch.empty_like(h)
@@ -319,9 +320,9 @@ def test_expert_swiglu_bf16_parity(T, k, K, d, m, pattern):
     torch.cuda.synchronize()
     assert dm.decomoe_read_status(status) == 0
     assert torch.equal(y5, y) and torch.equal(h5, h)
-    # the one launch that also gathers the dispatched rows (as the layer runs
-    # it from 8192 routed rows): same tiles, same bits, and the gathered rows
-    # are x[perm_token]
+    # the one launch that reads its rows by index, as the layer's does, and also
+    # writes them grouped: same tiles, same bits, and the grouped rows are
+    # x[perm_token]
     if 8 * K < R <= 32768 and (2 * m) % 256 == 0:
         ready.zero_()
         xg = torch.zeros_like(xp)
