@@ -1086,17 +1086,15 @@ __global__ void __launch_bounds__(DL_THREADS, 1)
       }
       xpar ^= 1;
       if (!dn) {
-        // this item's h slice is stored (by every warp: one that gave up raised
-        // the flag ahead of the barrier): publish it to the down items of eg
+        // this item's h slice is stored (unless a warp gave up): publish it to the
+        // down items of eg
         fence_proxy_async_all();
-        named_bar_sync(1, 128);
-        if (et == 0 && !*s_abort) red_add_release_s32(ready + eg, 1);
+        if (named_bar_all(1, 128, ok) && et == 0) red_add_release_s32(ready + eg, 1);
       } else {
-        // y rows of block wb stored (by every warp): count them per token; the tile that
-        // completes a token's k slots of this block combines them
+        // y rows of block wb stored (unless a warp gave up): count them per token;
+        // the tile that completes a token's k slots of this block combines them
         if (et == 0) s_flag[2] = 0;
-        named_bar_sync(1, 128);
-        if (et < nr && !*s_abort) {
+        if (named_bar_all(1, 128, ok) && et < nr) {
           const int tok = s_perm[r0 + et];
           // release this tile's y rows; the k-th arrival acquires the others'
           const int old = atom_add_acq_rel_s32(comb + tok * nfb + wb, 1);

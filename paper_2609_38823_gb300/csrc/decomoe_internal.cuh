@@ -257,6 +257,19 @@ __device__ __forceinline__ void report_status(int32_t* status, int32_t code) {
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
+// The same barrier; whether p held in every thread that met at it.
+__device__ __forceinline__ bool named_bar_all(int id, int nthreads, bool p) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred a, b;\n\t"
+      "setp.ne.u32 a, %3, 0;\n\t"
+      "bar.red.and.pred b, %1, %2, a;\n\t"
+      "selp.u32 %0, 1, 0, b;\n\t}"
+      : "=r"(r)
+      : "r"(id), "r"(nthreads), "r"(static_cast<uint32_t>(p))
+      : "memory");
+  return r != 0;
+}
 // Order this thread's generic-proxy global writes before later async-proxy
 // (TMA) accesses of the same memory.
 __device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }

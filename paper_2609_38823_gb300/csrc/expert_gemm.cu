@@ -1148,11 +1148,10 @@ __global__ void __launch_bounds__(192, 1)
       tc_fence_before();
       mbar_arrive(TEMPTY_BAR(acc));
       if (!dn) {
-        // this item's h slice is stored (by every warp: a warp that gave up
-        // raised the flag ahead of the barrier): publish it to the down items of T.g
+        // this item's h slice is stored (unless a warp gave up): publish it to the
+        // down items of T.g
         fence_proxy_async_all();
-        named_bar_sync(1, 128);
-        if (et == 0 && !*s_abort) {
+        if (named_bar_all(1, 128, ok) && et == 0) {
           __threadfence();
           atomicAdd(g.ready + T.g, 1);
         }
