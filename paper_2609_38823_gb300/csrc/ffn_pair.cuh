@@ -35,9 +35,9 @@
 // branch with two barriers per k-block, the same kernel took 637 cycles per
 // k-block (gate/up 1576 TFLOP/s) instead of 512, and an arrival with cluster
 // release 1900. Layer against the one-SM kernels: T = 2048, K = 64 222 -> 187 us;
-// 4096 361 -> 282; 16384, K = 128 1237 -> 976; 1552, K = 128 237 -> 216; 272, K =
+// 4096 361 -> 282; 16384, K = 128 1272 -> 1029 (two launches); 1552, K = 128 237 -> 216; 272, K =
 // 57 114 -> 106; 131, K = 64 97.6 -> 91.3. With one ring for both operands it had
-// been 199, 301, 1037, 228, 109 and 93.7; with eight slots for weights and four
+// been 199, 301, 1037 (in one launch), 228, 109 and 93.7; with eight slots for weights and four
 // for rows gate/up from L2 ran at 1654 TFLOP/s instead of 1805.
 #pragma once
 
