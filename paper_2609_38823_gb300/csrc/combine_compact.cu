@@ -196,9 +196,9 @@ static cudaError_t launch_combine_w(cudaStream_t s, const uint4* y, const int32_
 // for each (from 32 tokens on; below, few tokens leave SMs idle either way). bf16
 // rows of 2048, top 8, calls after one another, on 152 SMs: 272 tokens 2.6 us with
 // four warps and 4.1 with two, 511 tokens 4.8 and 3.8 (rows of 256: 3.9 and 2.1),
-// 513 tokens 3.9 with two. In a layer 131 tokens take 90.8 us with eight and 91.0
-// with four, 1552 tokens 213.4 with one and 215.4 with two, 4096 tokens 274.3 and
-// 276.1.
+// 513 tokens 3.9 with two; without a residual 150 tokens 2.3 us with eight and 2.4
+// with four, of 4096 2.5 and 3.4. In a layer 1552 tokens take 213.4 us with one and
+// 215.4 with two, 4096 tokens 274.3 and 276.1.
 template <bool BF16, bool DROP>
 static cudaError_t launch_combine_k(cudaStream_t s, const uint4* y, const int32_t* inv, const float* w, int64_t T,
                                     int k, int vec, const uint4* res, uint4* out, DropRows drop, int dc) {
